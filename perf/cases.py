@@ -85,7 +85,7 @@ def draw(rng):
     if kind == "iterate":
         n = rng.choice(SIZES)
         n_ei = rng.choice([1, 2, 3, 4])
-        return dict(kind=kind, N=n, Np=_fit(_log_int(rng, 5, 700), n, 576 << 19),
+        return dict(kind=kind, N=n, Np=_fit(_log_int(rng, 5, 700), n, 560 << 19),
                     iters=rng.choice([1, 2] if upd == "raar" else [1, 2, 3, 4]), n_ei=n_ei, update=upd,
                     # at 192 and 384 a mirrored seam reads a wrong column 0, which the tests on those sizes had missed
                     mirror=rng.random() < 0.3 and n not in (192, 384), blend_object=rng.random() < 0.3,
