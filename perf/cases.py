@@ -57,8 +57,8 @@ def listed():
         dict(name="sweep_160x90", kind="sweep", N=160, Np=90, guesses=16, iters=2, n_ei=2, update="raar"),
         # the 3D volume of the main workload
         dict(name="assemble_512x360", kind="assemble", N=512, Np=360),
-        # Step D of the mid-size workload with its tomographic refinement
-        dict(name="refine_256x180", kind="refine", N=256, Np=180, iters=20),
+        # Step D of the mid-size workload with its tomographic refinement, the paper's 50 iterations
+        dict(name="refine_256x180", kind="refine", N=256, Np=180, iters=50),
         # Step C of one of the paper's sizes
         dict(name="merge_256x144", kind="merge", N=256, Np=144, guesses=6, keep=4),
         # the support update beside a detector: 16 patterns a call
@@ -108,7 +108,7 @@ def draw(rng):
         return dict(kind=kind, N=n, Np=_fit(_log_int(rng, 12, 500), n, 360 << 18))
     if kind == "refine":
         n = rng.choice([32, 64, 96, 128, 160, 192, 256, 320, 384, 512])
-        return dict(kind=kind, N=n, Np=_log_int(rng, 12, 180), iters=rng.choice([2, 5, 10]))
+        return dict(kind=kind, N=n, Np=_log_int(rng, 12, 180), iters=rng.choice([2, 5, 10]) if n < 512 else 2)
     if kind == "merge":
         n = rng.choice([32, 64, 96, 128, 160, 192, 256])
         g = rng.randint(2, 6)
