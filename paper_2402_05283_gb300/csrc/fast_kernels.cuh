@@ -340,7 +340,7 @@ __device__ __forceinline__ void blend_tap(float2 (&a)[FL::TA][FL::E1], const flo
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
       const int x = FL::a_x(t, m);
-      const int xs_ = MIR ? (m == 0 ? (N - x) & (N - 1) : N - x) : x;
+      const int xs_ = MIR ? (m == 0 && x == 0 ? 0 : N - x) : x;
       float v0 = __ldg(r0 + xs_);
       float v1 = __ldg(r0 + N + xs_);
       if constexpr (OBJ) {
