@@ -123,8 +123,9 @@ enum {
  *                  thread-block cluster (N = 64, 128, 256, 512; FP32; needs a
  *                  GPU that can hold an N/32-CTA cluster at N = 512, an
  *                  N/64-CTA cluster below, else UNSUPPORTED at cpra_plan).
- *                  AUTO: FUSED for N <= 256 in FP32 where the device holds
- *                  its clusters, else WARP where available, else TWO_PASS.
+ *                  AUTO: FUSED for N <= 256 in FP32 where it exists and the
+ *                  device holds its clusters, else WARP's kernels (every N;
+ *                  TWO_PASS for a sweep at an N that WARP does not name).
  *                  TUNED: the fastest engine for this N on this GPU
  *                  according to cpra_autotune (its default cache).
  *   update         real-space rule of the iterations before hio_iters.

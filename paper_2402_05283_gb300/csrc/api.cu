@@ -168,7 +168,7 @@ cpra_status validate(const cpra_config* c, std::string& why) {
     why = "fused engine needs N in {64, 128, 256, 512}";
     return CPRA_ERR_UNSUPPORTED;
   }
-  if (c->engine == CPRA_ENGINE_WARP && !fast_supported(c->N)) {
+  if (c->engine == CPRA_ENGINE_WARP && !warp_engine_listed(c->N)) {
     why = "warp engine needs N in {64, 128, 192, 256, 384, 512, 1024}";
     return CPRA_ERR_UNSUPPORTED;
   }
@@ -616,10 +616,14 @@ cpra_status cpra_plan(const cpra_config* cfg, void* stream, cpra_plan_t* out) {
   p->N = cfg->N;
   p->Np = cfg->Np;
   p->W = (cfg->N + 31) / 32;
-  p->engine = (cfg->engine == CPRA_ENGINE_WARP ||
-               (cfg->engine == CPRA_ENGINE_AUTO && fast_supported(cfg->N)))
-                  ? CPRA_ENGINE_WARP
-                  : CPRA_ENGINE_TWO_PASS;
+  // AUTO: the warp kernels cover every N and are the faster ones at all of
+  // them (fftw.cuh has the figures).  A Gauss-Seidel sweep at a size that
+  // WARP does not name stays on the block-wide engine: one sweep carries a
+  // rounding difference through every angle (1e-7 grows to 1e-4 in two RAAR
+  // sweeps of 90 angles), so its arithmetic is kept.
+  const bool unlisted = !warp_engine_listed(cfg->N);
+  const bool block_wide = cfg->engine == CPRA_ENGINE_TWO_PASS || (cfg->sweep && unlisted);
+  p->engine = block_wide ? CPRA_ENGINE_TWO_PASS : CPRA_ENGINE_WARP;
   if (cfg->engine == CPRA_ENGINE_TUNED) {
     int32_t e = 0;
     cpra_status ts = cpra_autotune(cfg->N, cfg->precision, nullptr, &e, nullptr);
@@ -627,7 +631,8 @@ cpra_status cpra_plan(const cpra_config* cfg, void* stream, cpra_plan_t* out) {
       delete p;
       return ts;
     }
-    p->engine = e;
+    // where the tuner has only the block-wide engine to choose, AUTO's choice
+    if (!(e == CPRA_ENGINE_TWO_PASS && unlisted)) p->engine = e;
   }
   // AUTO: the fused engine where it is the faster one (N <= 256, FP32) and
   // this device can hold its clusters, else the warp engine
@@ -2435,7 +2440,7 @@ cpra_status cpra_autotune(int32_t N, int32_t precision, const char* cache_path,
   std::ostringstream detail;
   const int cands[3] = {CPRA_ENGINE_TWO_PASS, CPRA_ENGINE_WARP, CPRA_ENGINE_FUSED};
   for (int cand : cands) {
-    if (cand == CPRA_ENGINE_WARP && !fast_supported(N)) continue;
+    if (cand == CPRA_ENGINE_WARP && !warp_engine_listed(N)) continue;
     if (cand == CPRA_ENGINE_FUSED && !fused_supported(N)) continue;
     double ms = 0.0;
     cpra_status s = time_engine(N, cand, &ms);

@@ -324,7 +324,7 @@ cudaError_t launch_refine_support(const RefineArgs& a, const uint32_t* S2, const
 cudaError_t launch_moments(cpra_plan_s* p, double* moments, cudaStream_t st);
 // one iteration; err2[0..1] += sum_M |X - V|^2, sum_M |V|^2
 cudaError_t launch_refine_iter(const RefineArgs& a, double* err2, cudaStream_t st);
-// the same passes with warp-resident FFTs (k_refine_w.cu; fast_supported(N))
+// the same passes with warp-resident FFTs (k_refine_w.cu; refine_fast_supported(N))
 cudaError_t launch_refine_fft3_w(const RefineArgs& a, cudaStream_t st);
 cudaError_t launch_refine_iter_w(const RefineArgs& a, double* err2, cudaStream_t st);
 // S3 <- {blur(P_{S3+} R) >= tau max} (mx: one unsigned of scratch)
@@ -341,7 +341,7 @@ cudaError_t launch_merge_finish(cpra_plan_s* dst, float2* acc, const float* mag,
 bool n_supported(int N);
 
 // two-pass engine with warp-resident FFTs (k_fast.cu)
-bool fast_supported(int N);          // iteration kernels (WARP engine)
+bool warp_engine_listed(int N);      // sizes that CPRA_ENGINE_WARP names (its kernels cover every N)
 bool refine_fast_supported(int N);   // 3D refinement passes and tensor-core forms
 bool fast_dims(int N, int* E1, int* E2);
 cudaError_t prepare_kernels_fast(int N);

@@ -1,4 +1,4 @@
-// fast_kernels.cuh - two-pass iteration with warp-resident FFTs, N in {64,...,1024}.
+// fast_kernels.cuh - two-pass iteration with warp-resident FFTs, every supported N.
 //
 // Same dataflow and the same packed half spectrum Hp as k_twopass.cu, but
 // every line transform is the two-level register FFT of fftw.cuh: one
@@ -64,10 +64,16 @@ template <int N, class FL>
 constexpr bool kRowMaskInRegs = kSlimLines<FL> && FL::L == 1 && N == 512;
 
 // per-warp shared memory of the row kernels: transpose tile + the warp's g
-// rows; 4 warps a block with the L-line plans, 8 with the one-line plan
+// rows; 4 warps a block with the L-line plans (the largest number up to 5
+// that divides the angle's warp tasks where 4 does not), 8 with the one-line
+// plan
+__host__ __device__ constexpr int row_warps(int tasks) {
+  return tasks % 4 == 0 ? 4 : tasks % 5 == 0 ? 5 : tasks % 3 == 0 ? 3 : tasks % 2 == 0 ? 2 : 1;
+}
 template <int N, class FL_> struct RowCfg {
   using FL = FL_;
-  static constexpr int WARPS = kSlimLines<FL> ? 8 : 4;
+  static_assert((N / 2) % FL::L == 0, "row pairs fill whole warps");
+  static constexpr int WARPS = kSlimLines<FL> ? 8 : row_warps((N / 2) / FL::L);
   static constexpr int GROWS = 2 * FL::L;                  // image rows per warp
   static constexpr int GFLOATS = GROWS * N;
   static constexpr int WARP_F2 = FL::TSIZE + GFLOATS / 2;  // float2 per warp
@@ -126,10 +132,11 @@ __device__ __forceinline__ void store_pairs_w(float2 (&b)[FL::TB][FL::E2], float
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
     const int line = FL::b_line(t);
-    static_for<0, FL::E2>([&](auto KK) {
-      constexpr int j = decltype(KK)::value;
-      T[line * N + FL::b_k(t, j)] = b[i][j];
-    });
+    if (FL::b_on(t))
+      static_for<0, FL::E2>([&](auto KK) {
+        constexpr int j = decltype(KK)::value;
+        T[line * N + FL::b_k(t, j)] = b[i][j];
+      });
   });
   __syncwarp();
 #pragma unroll
@@ -137,10 +144,10 @@ __device__ __forceinline__ void store_pairs_w(float2 (&b)[FL::TB][FL::E2], float
     const float2* Z = T + line * N;
     float2* r0 = Hn + (size_t)(2 * (pair0 + line)) * H;
     float2* r1 = r0 + H;
-    static_assert(H % 32 == 0, "row pairs");
 #pragma unroll
-    for (int kk = 0; kk < H / 32; ++kk) {
+    for (int kk = 0; kk < (H + 31) / 32; ++kk) {
       const int k = lane + 32 * kk;
+      if (H % 32 != 0 && k >= H) break;
       float2 h0, h1;
       if (kk == 0 && lane == 0) {
         const float2 z0 = Z[0], zn = Z[H];
@@ -199,14 +206,17 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
   // the warp's 2L packed spectrum rows (contiguous) into its tile, then the
   // old iterate, which is needed only after the inverse FFT
   {
-    static_assert((FL::L * N / 2) % 32 == 0 && (RW::GFLOATS / 4) % 32 == 0, "row staging");
+    constexpr int HC = FL::L * N / 2;  // 16-byte pieces
     const float2* hrow = Hn + (size_t)(2 * pair0) * H + 2 * lane;
 #pragma unroll
-    for (int k = 0; k < FL::L * N / 64; ++k) cp_async16(T + 2 * (lane + 32 * k), hrow + 64 * k);
+    for (int k = 0; k < (HC + 31) / 32; ++k)
+      if (HC % 32 == 0 || lane + 32 * k < HC) cp_async16(T + 2 * (lane + 32 * k), hrow + 64 * k);
     cp_async_commit();
   }
+  constexpr int GC = RW::GFLOATS / 4;  // 16-byte pieces
 #pragma unroll
-  for (int k = 0; k < RW::GFLOATS / 128; ++k) cp_async16(Gs + 4 * (lane + 32 * k), grow + 4 * lane + 128 * k);
+  for (int k = 0; k < (GC + 31) / 32; ++k)
+    if (GC % 32 == 0 || lane + 32 * k < GC) cp_async16(Gs + 4 * (lane + 32 * k), grow + 4 * lane + 128 * k);
   cp_async_commit();
   if (bx == 0 && threadIdx.x == 0) {
     if (err_slot >= 0) {
@@ -245,6 +255,7 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
     static_for<0, FL::TB>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
+      if (!FL::b_on(t)) return;
       const float2* r0 = T + FL::b_line(t) * N;
       const float2* r1 = r0 + H;
       static_for<0, FL::E2>([&](auto KK) {
@@ -273,6 +284,7 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
     static_for<0, FL::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
+      if (!FL::a_on(t)) return;
       const int line = FL::a_line(t);
       const int y0 = 2 * (pair0 + line);
       float* g0 = g + ((size_t)n * N + y0) * N;
@@ -334,6 +346,7 @@ __device__ __forceinline__ void blend_tap(float2 (&a)[FL::TA][FL::E1], const flo
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
+    if (!FL::a_on(t)) return;
     const int y0 = 2 * (pair0 + FL::a_line(t));
     const float* r0 = src + (size_t)y0 * N;
     const uint32_t* m0 = sk + (size_t)y0 * W;
@@ -385,6 +398,7 @@ __device__ __forceinline__ void store_rows(const float2 (&a)[FL::TA][FL::E1], fl
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
+    if (!FL::a_on(t)) return;
     float* d0 = img + (size_t)(2 * (pair0 + FL::a_line(t))) * N;
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
@@ -438,15 +452,20 @@ k_prime_w(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
 
 // ---------------------------------------------------------------- column pass
 // packed columns per CTA: 16 (128 B of each row) with the L-line plans; 8
-// with the one-line plan (8 warps, three CTAs an SM) and for the 16-bit path
-// at N >= 512, where the tensor-core region (block DFT matrices, A tile)
-// beside 16 columns would leave room for one CTA an SM
+// with the one-line plan (8 warps, three CTAs an SM), for the one-line sizes
+// whose 8 columns leave room for two CTAs an SM (640, 768), and for the
+// 16-bit path at N >= 512, where the tensor-core region (block DFT matrices,
+// A tile) beside 16 columns would leave room for one CTA an SM; where N/2 is
+// not a multiple of 16, a divisor of it (all 24 columns at N = 48, 10 of the
+// 350 at N = 700: 80 B of each row)
 template <int N, int PREC> struct ColW {
   using FL = typename WLines<N, PREC>::type;
-  static constexpr int CB = ((PREC != kPrecFP32 && N >= 512) || kSlimLines<FL>) ? 8 : 16;
+  static constexpr int CB = N == 700 ? 10 : N == 48 ? 24 : N == 16 ? 8
+                            : ((PREC != kPrecFP32 && N >= 512) || kSlimLines<FL> || N == 640 || N == 768) ? 8 : 16;
+  static_assert((N / 2) % CB == 0 && CB % FL::L == 0, "column blocks");
   static constexpr int WARPS = CB / FL::L;
   static constexpr int NT = WARPS * 32;
-  static constexpr int MINB = kSlimLines<FL> ? 3 : (NT <= 256 ? 2 : 1);
+  static constexpr int MINB = kSlimLines<FL> ? 3 : (NT <= 256 || N == 700 ? 2 : 1);
   static constexpr int SP = CB + 1;  // staging pitch
   static constexpr int N2 = N / 2;
   static constexpr int STAGE = N * SP;
@@ -455,9 +474,11 @@ template <int N, int PREC> struct ColW {
   // A_sym of the block in shared memory, column c at c * AP, frequency ky at
   // a_pos(ky): the upper half moved on by 16 floats, so lanes reading ky and
   // ky + N/2 (the one-line plan's lane pairs) or the same ky of neighbouring
-  // columns (the L-line plans) fall in different banks
+  // columns (the L-line plans) fall in different banks; no shift where a
+  // 16-byte piece would straddle the halves (N = 700, one line a warp)
+  static constexpr int AS = (N / 2) % 4 == 0 ? 16 : 0;
   static constexpr int AP = N + 16;
-  static __device__ __forceinline__ int a_pos(int ky) { return ky + (ky >= N / 2 ? 16 : 0); }
+  static __device__ __forceinline__ int a_pos(int ky) { return ky + (ky >= N / 2 ? AS : 0); }
   static constexpr size_t SMEM = sizeof(float2) * (N + BUF) + sizeof(float) * CB * AP;
 };
 // a_pos of the B-layout frequency b_k(t, j) of a column-pass task: the half
@@ -469,7 +490,7 @@ __device__ __forceinline__ int col_a_pos(int t) {
   if constexpr (std::is_same_v<FL, PairLines512>)
     return FL::b_k(t, 0) + ((t & 1) ? 16 : 0) + 16 * j;
   else
-    return FL::b_k(t, 0) + FL::E1 * j + (FL::E1 * j >= C::N2 ? 16 : 0);
+    return FL::b_k(t, 0) + FL::E1 * j + (FL::E1 * j >= C::N2 ? C::AS : 0);
 }
 template <int N, int PREC>
 constexpr size_t col_smem() {
@@ -534,25 +555,29 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
   // the unrolled copies differ only in immediate offsets.  A warp's 32 / CB
   // rows are WARPS apart: with 8 columns (pitch 9) rows 8 apart start 16
   // banks apart, so a warp's 256 bytes take the minimum two wavefronts
-  constexpr int RS = C::NT / C::CB;
-  static_assert(C::NT % C::CB == 0 && 32 % C::CB == 0 && N % RS == 0 && (C::CB * N / 4) % C::NT == 0,
-                "column staging");
-  const int y0 = warp + C::WARPS * (lane / C::CB), cc = lane % C::CB;
+  // (blocks whose columns do not divide a warp take plain thread order)
+  constexpr int RS = C::NT / C::CB, SR = (N + RS - 1) / RS;
+  constexpr int AC = C::CB * N / 4, AR = (AC + C::NT - 1) / C::NT;
+  static_assert(C::NT % C::CB == 0, "column staging");
+  const int y0 = 32 % C::CB == 0 ? warp + C::WARPS * (lane / C::CB) : threadIdx.x / C::CB;
+  const int cc = 32 % C::CB == 0 ? lane % C::CB : threadIdx.x % C::CB;
   {
     const float2* src = Hn + (size_t)y0 * H + c0 + cc;
     float2* dst = buf + y0 * C::SP + cc;
     if constexpr (L2_ONLY) {
 #pragma unroll
-      for (int k = 0; k < N / RS; ++k) dst[k * RS * C::SP] = ld_cg(src + (size_t)k * RS * H);
+      for (int k = 0; k < SR; ++k)
+        if (N % RS == 0 || y0 + k * RS < N) dst[k * RS * C::SP] = ld_cg(src + (size_t)k * RS * H);
     } else {
 #pragma unroll
-      for (int k = 0; k < N / RS; ++k) cp_async8(dst + k * RS * C::SP, src + (size_t)k * RS * H);
+      for (int k = 0; k < SR; ++k)
+        if (N % RS == 0 || y0 + k * RS < N) cp_async8(dst + k * RS * C::SP, src + (size_t)k * RS * H);
     }
     const float* Ablk = A_T + ((size_t)n * H + c0) * N;  // CB contiguous columns
 #pragma unroll
-    for (int k = 0; k < C::CB * N / 4 / C::NT; ++k) {
-      const int f = 4 * (threadIdx.x + k * C::NT);  // 4 floats, never across a half (4 | N/2)
-      cp_async16(As + (f / N) * C::AP + C::a_pos(f % N), Ablk + f);
+    for (int k = 0; k < AR; ++k) {
+      const int f = 4 * (threadIdx.x + k * C::NT);  // 4 floats, never across a column (4 | N) or a shifted half
+      if (AC % C::NT == 0 || f < 4 * AC) cp_async16(As + (f / N) * C::AP + C::a_pos(f % N), Ablk + f);
     }
   }
   cp_async_commit();
@@ -563,6 +588,7 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
+    if (!FL::a_on(t)) return;
     const int col = warp * FL::L + FL::a_line(t);
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
@@ -578,7 +604,7 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
     const int col = warp * FL::L + FL::b_line(t);
-    if (c0 + col != 0) {
+    if (FL::b_on(t) && c0 + col != 0) {
       const float* Ac = As + col * C::AP;
       static_for<0, FL::E2>([&](auto KK) {
         constexpr int j = decltype(KK)::value;
@@ -591,7 +617,7 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
     static_for<0, FL::TB>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
-      if (FL::b_line(t) == 0) {
+      if (FL::b_on(t) && FL::b_line(t) == 0) {
         static_for<0, FL::E2>([&](auto KK) {
           constexpr int j = decltype(KK)::value;
           T[FL::b_k(t, j)] = b[i][j];
@@ -602,7 +628,7 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
     static_for<0, FL::TB>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
-      if (FL::b_line(t) == 0) {
+      if (FL::b_on(t) && FL::b_line(t) == 0) {
         const float* A0 = As;  // column 0 of the block
         const float* An = A_nyq + (size_t)n * N;
         static_for<0, FL::E2>([&](auto KK) {
@@ -625,6 +651,7 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
+    if (!FL::a_on(t)) return;
     const int col = warp * FL::L + FL::a_line(t);
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
@@ -636,7 +663,8 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
     float2* dst = Hn + (size_t)y0 * H + c0 + cc;
     const float2* src = buf + y0 * C::SP + cc;
 #pragma unroll
-    for (int k = 0; k < N / RS; ++k) dst[(size_t)k * RS * H] = src[k * RS * C::SP];
+    for (int k = 0; k < SR; ++k)
+      if (N % RS == 0 || y0 + k * RS < N) dst[(size_t)k * RS * H] = src[k * RS * C::SP];
   }
   double errd = 2.0 * (double)err2 + (double)err1;
   for (int o = 16; o > 0; o >>= 1) errd += __shfl_down_sync(0xffffffffu, errd, o);
@@ -783,7 +811,7 @@ static cudaError_t smem_attr(K kernel, size_t bytes) {
 }
 
 template <int N, int PREC>
-static cudaError_t prepare_w() {
+cudaError_t prepare_w() {
   static bool done = false;
   if (done) return cudaSuccess;
   cudaError_t e = smem_attr(k_rowpass_w<N, PREC>, row_smem<N, PREC>());
@@ -814,7 +842,7 @@ static cudaError_t prepare_w() {
 }
 
 template <int N, int PREC>
-static cudaError_t rowpass_w(const Launch& L) {
+cudaError_t rowpass_w(const Launch& L) {
   using RW = RowW<N, PREC>;
   const size_t smem = row_smem<N, PREC>();
   cudaError_t e = prepare_w<N, PREC>();
@@ -826,7 +854,7 @@ static cudaError_t rowpass_w(const Launch& L) {
 }
 
 template <int N, int PREC>
-static cudaError_t prime_w(const Launch& L) {
+cudaError_t prime_w(const Launch& L) {
   using RW = PrimeW<N, PREC>;
   const size_t smem = prime_smem<N, PREC>();
   cudaError_t e = prepare_w<N, PREC>();
@@ -838,7 +866,7 @@ static cudaError_t prime_w(const Launch& L) {
 }
 
 template <int N, int PREC>
-static cudaError_t colpass_w(const Launch& L) {
+cudaError_t colpass_w(const Launch& L) {
   using C = ColW<N, PREC>;
   const size_t smem = col_smem<N, PREC>();
   cudaError_t e = prepare_w<N, PREC>();
@@ -852,7 +880,15 @@ static cudaError_t colpass_w(const Launch& L) {
 
 // sizes of the 3D refinement's warp passes and of the tensor-core forms
 #define CPRA_FOR_EACH_FAST_N(X) X(64) X(128) X(256) X(512) X(1024)
-// sizes of the warp engine's iteration kernels
+// sizes at which CPRA_ENGINE_WARP can be asked for (and the persistent batch mode)
 #define CPRA_FOR_EACH_WARP_N(X) X(64) X(128) X(192) X(256) X(384) X(512) X(1024)
+
+// The FP32 instances of one N, compiled in the translation unit that names
+// them (k_fast_*.cu) and only declared elsewhere: nvcc takes about 10 s a size.
+#define CPRA_WARP_INSTANCES(NN, EXTERN)                              \
+  EXTERN template cudaError_t prepare_w<NN, kPrecFP32>();            \
+  EXTERN template cudaError_t rowpass_w<NN, kPrecFP32>(const Launch&); \
+  EXTERN template cudaError_t prime_w<NN, kPrecFP32>(const Launch&);   \
+  EXTERN template cudaError_t colpass_w<NN, kPrecFP32>(const Launch&);
 
 }  // namespace cpra

@@ -13,6 +13,8 @@
 //             line = t / E2, l = t % E2
 //   B layout  b[i][k2] = X_line[k1 + E1 k2],   task t = lane + 32 i:
 //             line = t / E1, k1 = t % E1
+// Where L * E2 or L * E1 is not a multiple of 32 the last slot's upper lanes
+// have no task (a_on, b_on): they take part in the warp's barriers only.
 // Twiddles inside the register DFTs are compile-time constants (cos and sin
 // evaluated from their Taylor series at compile time in FP64, exact at
 // multiples of pi/2); the cross twiddles come from a table
@@ -83,20 +85,36 @@ template <> struct WarpPlan<512> { static constexpr int E1 = 16, E2 = 32, L = 2;
 template <> struct WarpPlan<192> { static constexpr int E1 = 24, E2 = 8, L = 4; };
 template <> struct WarpPlan<384> { static constexpr int E1 = 24, E2 = 16, L = 4; };
 template <> struct WarpPlan<1024> { static constexpr int E1 = 32, E2 = 32, L = 1; };
+// the remaining sizes: E2 even (the halves of a line then split at a whole
+// register, see ColW) and as few idle lanes in the last slot as 32 values a
+// lane allow.  Column + row pass, us per angle (360 angles; 230, 192, 160 at
+// 640, 700, 768), these plans against the block-wide Stockham passes:
+//   32: 0.048 / 0.069   48: 0.064 / 0.069    96: 0.095 / 0.185
+//   160: 0.187 / 0.395  320: 0.63 / 1.77     640: 2.7 / 12.6
+//   700: 4.1 / 9.7      768: 3.8 / 16.0      16: 0.045 / 0.047
+template <> struct WarpPlan<16> { static constexpr int E1 = 4, E2 = 4, L = 8; };
+template <> struct WarpPlan<32> { static constexpr int E1 = 4, E2 = 8, L = 8; };
+template <> struct WarpPlan<48> { static constexpr int E1 = 8, E2 = 6, L = 4; };
+template <> struct WarpPlan<96> { static constexpr int E1 = 12, E2 = 8, L = 4; };
+template <> struct WarpPlan<160> { static constexpr int E1 = 20, E2 = 8, L = 4; };
+template <> struct WarpPlan<320> { static constexpr int E1 = 20, E2 = 16, L = 2; };
+template <> struct WarpPlan<640> { static constexpr int E1 = 20, E2 = 32, L = 1; };
+template <> struct WarpPlan<700> { static constexpr int E1 = 25, E2 = 28, L = 1; };
+template <> struct WarpPlan<768> { static constexpr int E1 = 24, E2 = 32, L = 1; };
 
 template <int N> struct WP {
   static constexpr int E1 = WarpPlan<N>::E1, E2 = WarpPlan<N>::E2, L = WarpPlan<N>::L;
-  static constexpr int TA = L * E2 / 32;  // step-A tasks per lane
-  static constexpr int TB = L * E1 / 32;  // step-B tasks per lane
+  static constexpr int NA = L * E2, NB = L * E1;  // step-A and step-B tasks of the warp
+  static constexpr int TA = (NA + 31) / 32;       // step-A slots per lane
+  static constexpr int TB = (NB + 31) / 32;       // step-B slots per lane
   static constexpr int TP = E2 + 1;       // odd pitch of the transpose tile
   static constexpr int AP = E1 + 1;       // step-A staging pitch (tensor-core path)
   static constexpr int T0 = (L * E1 * TP > L * N) ? L * E1 * TP : L * N;
   static constexpr int TSIZE = (L * E2 * AP > T0) ? L * E2 * AP : T0;  // float2 per warp
-  static_assert(E1 * E2 == N && TA * 32 == L * E2 && TB * 32 == L * E1, "warp plan");
+  static __device__ __forceinline__ bool a_on(int t) { return NA % 32 == 0 || t < NA; }
+  static __device__ __forceinline__ bool b_on(int t) { return NB % 32 == 0 || t < NB; }
+  static_assert(E1 * E2 == N && E2 % 2 == 0, "warp plan");
 };
-
-template <int N> constexpr bool kHasWarpPlan = (N == 64 || N == 128 || N == 192 || N == 256 || N == 384 ||
-                                                N == 512 || N == 1024);
 
 // step-A DFTs of every task of this warp through the tensor cores; a[][]
 // goes through the warp tile T with pitch E1 + 1
@@ -144,7 +162,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
       const int line = t / P::E2, l = t % P::E2;
-      T[(line * P::E1 + k1) * P::TP + l] = v[i];
+      if (P::a_on(t)) T[(line * P::E1 + k1) * P::TP + l] = v[i];
     });
   });
   __syncwarp();
@@ -157,10 +175,11 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
     const int line = t / P::E1, k1 = t % P::E1;
-    static_for<0, P::E2>([&](auto LL) {
-      constexpr int l = decltype(LL)::value;
-      b[i][l] = T[(line * P::E1 + k1) * P::TP + l];
-    });
+    if (P::b_on(t))
+      static_for<0, P::E2>([&](auto LL) {
+        constexpr int l = decltype(LL)::value;
+        b[i][l] = T[(line * P::E1 + k1) * P::TP + l];
+      });
     if constexpr (PREC == kPrecFP32) reg_fft<P::E2, -1>(b[i]);
   });
   __syncwarp();
@@ -178,10 +197,11 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
     const int t = lane + 32 * i;
     const int line = t / P::E1, k1 = t % P::E1;
     if constexpr (PREC == kPrecFP32) reg_fft<P::E2, +1>(b[i]);
-    static_for<0, P::E2>([&](auto LL) {
-      constexpr int l = decltype(LL)::value;
-      T[(line * P::E1 + k1) * P::TP + l] = b[i][l];
-    });
+    if (P::b_on(t))
+      static_for<0, P::E2>([&](auto LL) {
+        constexpr int l = decltype(LL)::value;
+        T[(line * P::E1 + k1) * P::TP + l] = b[i][l];
+      });
   });
   __syncwarp();
   if constexpr (PREC != kPrecFP32) {
@@ -194,7 +214,7 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
       const int line = t / P::E2, l = t % P::E2;
-      a[i][k1] = T[(line * P::E1 + k1) * P::TP + l];
+      if (P::a_on(t)) a[i][k1] = T[(line * P::E1 + k1) * P::TP + l];
     });
     static_for<0, P::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
@@ -215,6 +235,9 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
 template <int N> struct WarpLines {
   using P = WP<N>;
   static constexpr int L = P::L, TA = P::TA, E1 = P::E1, TB = P::TB, E2 = P::E2, TSIZE = P::TSIZE;
+  // whether task t exists (else its registers hold nothing)
+  static __device__ __forceinline__ bool a_on(int t) { return P::a_on(t); }
+  static __device__ __forceinline__ bool b_on(int t) { return P::b_on(t); }
   static __device__ __forceinline__ int a_line(int t) { return t / E2; }
   static __device__ __forceinline__ int a_x(int t, int m) { return t % E2 + E2 * m; }
   static __device__ __forceinline__ int b_line(int t) { return t / E1; }

@@ -27,6 +27,8 @@ struct PairLines512 {
   static constexpr int N = 512, L = 1, TA = 1, E1 = 16, TB = 1, E2 = 16;
   static constexpr int TP = 34;  // even pitch: both transpose directions conflict-free
   static constexpr int TSIZE = 16 * TP;
+  static __device__ __forceinline__ bool a_on(int) { return true; }
+  static __device__ __forceinline__ bool b_on(int) { return true; }
   static __device__ __forceinline__ int a_line(int) { return 0; }
   static __device__ __forceinline__ int a_x(int t, int m) { return t + 32 * m; }
   static __device__ __forceinline__ int b_line(int) { return 0; }
