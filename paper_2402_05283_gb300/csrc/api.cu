@@ -479,6 +479,26 @@ cpra_status build_gridding(cpra_plan_s* p) {
   return CPRA_OK;
 }
 
+// The step-table row of a whole sweep episode of p in one launch, from
+// iteration t and the buffers g -> g_alt (launch_sweep; the engine's kernels
+// take the same row for one angle).
+JobStep sweep_step(const cpra_plan_s* p, int64_t t, float* g, float* g_alt) {
+  const cpra_config& c = p->cfg;
+  JobStep s{};
+  s.prime = 1;
+  s.ca = coupling_args(c);
+  s.g_src = g;
+  s.g_dst = g_alt;
+  s.g = g_alt;
+  s.err_slot = t;
+  s.algo = t < c.hio_iters ? update_rule(c) : kER;
+  s.forward = 1 < c.n_ei;
+  s.active = 1;
+  s.n_iters = c.n_ei;
+  s.hio_left = (int)std::max<int64_t>(0, std::min<int64_t>(c.n_ei, (int64_t)c.hio_iters - t));
+  return s;
+}
+
 // every angle that iterates has intensities
 bool present_loaded(const cpra_plan_s* p) {
   for (int n = 0; n < p->Np; ++n)
@@ -910,8 +930,9 @@ static cpra_status iterate_core(cpra_plan_s* p, int32_t n_iters, double* err_out
 // Gauss-Seidel episodes (cfg.sweep): angle n starts from Eq. 4 over this
 // episode's images of the angles before it (g_alt, written as the sweep
 // goes) and the previous episode's of the others (g), then runs the
-// episode's n_ei iterations alone; one launch per angle with the fused
-// engine, prime + n_ei (column + row) launches per angle with the others.
+// episode's n_ei iterations alone; one launch an episode where the sweep
+// kernel covers the plan, else one launch per angle with the fused engine,
+// prime + n_ei (column + row) launches per angle with the others.
 static cpra_status iterate_sweep(cpra_plan_s* p, int32_t n_iters, double* err_out) {
   const cpra_config& c = p->cfg;
   const int E = c.n_ei, Np = p->Np;
@@ -925,25 +946,39 @@ static cpra_status iterate_sweep(cpra_plan_s* p, int32_t n_iters, double* err_ou
   cpra_status st = ensure_err_cap(p, p->t + n_iters);
   if (st != CPRA_OK) return st;
   const bool fused = p->engine == CPRA_ENGINE_FUSED;
+  const bool whole = sweep_supported(p->N, p->engine);
   const int64_t t0 = p->t;
+  if (whole) {
+    std::vector<JobStep> rows;
+    float *src = p->g, *dst = p->g_alt;
+    for (int ep = 0; ep < n_iters / E; ++ep, std::swap(src, dst))
+      rows.push_back(sweep_step(p, t0 + (int64_t)ep * E, src, dst));
+    st = upload_steps(p, rows);
+    if (st != CPRA_OK) return st;
+  }
   for (int ep = 0; ep < n_iters / E; ++ep) {
     const int64_t t = p->t;
+    if (whole) {
+      CK(timed(p, CPRA_KERNEL_FUSED, [&] { return launch_sweep(plan_launch(p, ep, 1)); }), "sweep");
+      std::swap(p->g, p->g_alt);
+      p->t += E;
+      p->hp_valid = false;
+      if (c.shrinkwrap_every > 0 && p->t % c.shrinkwrap_every == 0)
+        CK(timed(p, CPRA_KERNEL_SHRINKWRAP, [&] { return launch_shrinkwrap(p); }), "shrinkwrap");
+      continue;
+    }
     std::vector<JobStep> steps;
     steps.reserve((size_t)Np * (fused ? 1 : E));
     for (int n = 0; n < Np; ++n) {
       for (int it = 0; it < (fused ? 1 : E); ++it) {
-        JobStep s{};
-        s.prime = it == 0;
-        s.ca = it == 0 ? coupling_args(c) : plain_args();
-        s.g_src = p->g;
-        s.g_dst = p->g_alt;
-        s.g = p->g_alt;
+        JobStep s = sweep_step(p, t, p->g, p->g_alt);
+        if (it > 0) {
+          s.prime = 0;
+          s.ca = plain_args();
+        }
         s.err_slot = t + it;
         s.algo = t + it < c.hio_iters ? update_rule(c) : kER;
         s.forward = it + 1 < E;
-        s.active = 1;
-        s.n_iters = E;
-        s.hio_left = (int)std::max<int64_t>(0, std::min<int64_t>(E, (int64_t)c.hio_iters - t));
         steps.push_back(s);
       }
     }
@@ -1795,6 +1830,15 @@ cpra_status cpra_batch_create(const cpra_plan_t* plans, int32_t n, int32_t use_g
 
 namespace {
 
+// Launches of a Gauss-Seidel group's n_iters iterations: one an episode
+// (sweep kernel), or per episode and angle one fused launch, or prime + n_ei
+// (column, row).
+int64_t sweep_launches(const cpra_batch_s::Group& g, int32_t n_iters) {
+  const int64_t episodes = n_iters / g.n_ei;
+  if (sweep_supported(g.N, g.engine)) return episodes;
+  return episodes * g.np_max * (g.engine == CPRA_ENGINE_FUSED ? 1 : 1 + 2 * (int64_t)g.n_ei);
+}
+
 // upload steps to a group's table (grown as needed; the group's graph, if
 // any, is never used for Gauss-Seidel groups)
 cudaError_t group_steps(cpra_batch_s* b, cpra_batch_s::Group& g, const std::vector<JobStep>& steps) {
@@ -1898,6 +1942,41 @@ cpra_status batch_sweep_group(cpra_batch_s* b, cpra_batch_s::Group& g, int32_t n
     p->state_ready = true;
     p->hp_valid = false;
   }
+  if (sweep_supported(g.N, g.engine)) {
+    // one launch an episode: every member's chain of angles on its own cluster
+    const int eps = n_iters / E;
+    std::vector<JobStep> rows((size_t)eps * m);
+    for (size_t j = 0; j < m; ++j) {
+      cpra_plan_s* p = b->plans[g.members[j]];
+      float *src = p->g, *dst = p->g_alt;
+      for (int ep = 0; ep < eps; ++ep, std::swap(src, dst))
+        rows[(size_t)ep * m + j] = sweep_step(p, p->t + (int64_t)ep * E, src, dst);
+    }
+    e = group_steps(b, g, rows);
+    for (int ep = 0; e == cudaSuccess && ep < eps; ++ep) {
+      Launch L;
+      L.N = g.N;
+      L.engine = g.engine;
+      L.prec = g.prec;
+      L.masked = masked;
+      L.stream = st;
+      L.js = g.d_js;
+      L.st = g.d_steps + (size_t)ep * m;
+      L.tiles = g.d_sweep_tiles;  // (j, 0) of every member
+      L.ntiles = (int)m;
+      e = launch_sweep(L);
+      for (int mi : g.members) {
+        cpra_plan_s* p = b->plans[mi];
+        std::swap(p->g, p->g_alt);
+        p->t += E;
+        p->hp_valid = false;
+        if (e == cudaSuccess && p->cfg.shrinkwrap_every > 0 && p->t % p->cfg.shrinkwrap_every == 0)
+          e = launch_shrinkwrap(p);  // the members share the batch's stream
+      }
+    }
+    if (e != cudaSuccess) return bfail(b, CPRA_ERR_CUDA, std::string("batch sweep: ") + cudaGetErrorString(e));
+    return CPRA_OK;
+  }
   const int per_n = fused ? 1 : E;
   for (int ep = 0; ep < n_iters / E; ++ep) {
     std::vector<JobStep> steps((size_t)g.np_max * per_n * m);
@@ -1909,17 +1988,14 @@ cpra_status batch_sweep_group(cpra_batch_s* b, cpra_batch_s::Group& g, int32_t n
           const cpra_config& c = p->cfg;
           const int64_t t = p->t;
           JobStep& s = steps[((size_t)n * per_n + it) * m + j];
-          s.prime = it == 0;
-          s.ca = it == 0 ? coupling_args(c) : plain_args();
-          s.g_src = p->g;
-          s.g_dst = p->g_alt;
-          s.g = p->g_alt;
+          s = sweep_step(p, t, p->g, p->g_alt);
+          if (it > 0) {
+            s.prime = 0;
+            s.ca = plain_args();
+          }
           s.err_slot = t + it;
           s.algo = t + it < c.hio_iters ? update_rule(c) : kER;
           s.forward = it + 1 < E;
-          s.active = 1;
-          s.n_iters = E;
-          s.hio_left = (int)std::max<int64_t>(0, std::min<int64_t>(E, (int64_t)c.hio_iters - t));
         }
     e = group_steps(b, g, steps);
     for (int n = 0; e == cudaSuccess && n < g.np_max; ++n)
@@ -2219,8 +2295,7 @@ int64_t cpra_batch_launches(cpra_batch_t b, int32_t n_iters) {
     int jacobi = 0;
     for (auto& g : b->groups) {
       if (g.sweep) {
-        k += (int64_t)(n_iters / g.n_ei) * g.np_max *
-             (g.engine == CPRA_ENGINE_FUSED ? 1 : 1 + 2 * (int64_t)g.n_ei);
+        k += sweep_launches(g, n_iters);
         continue;
       }
       ++jacobi;
@@ -2241,9 +2316,8 @@ int64_t cpra_batch_launches(cpra_batch_t b, int32_t n_iters) {
     return k;
   }
   for (auto& g : b->groups) {
-    if (g.sweep) {  // per episode and angle: one fused launch, or prime + n_ei (column, row)
-      k += (int64_t)(n_iters / g.n_ei) * g.np_max *
-           (g.engine == CPRA_ENGINE_FUSED ? 1 : 1 + 2 * (int64_t)g.n_ei);
+    if (g.sweep) {
+      k += sweep_launches(g, n_iters);
       continue;
     }
     if (g.engine == CPRA_ENGINE_FUSED) {  // one launch per round of windows

@@ -211,18 +211,22 @@ __device__ __forceinline__ float2 twiddle(const float2* tw, int k) {
 }
 
 // One Stockham pass and the rest, recursively, for lines of length N.
-// NS = product of the radices already applied.  Caller's threads: NT.
-template <int N, int NS, int DIR, int B, int PI, int NT>
-__device__ __forceinline__ void stockham(float2* buf, const float2* tw) {
+// NS = product of the radices already applied.  Caller's threads: NT, this
+// one tid.  OPQ: the index arithmetic of each pass starts from an opaque copy
+// of tid, so that a kernel that loops over many transforms does not hold the
+// addresses of all of them in registers.
+template <int N, int NS, int DIR, int B, int PI, int NT, bool OPQ = false>
+__device__ __forceinline__ void stockham(float2* buf, const float2* tw, int tid) {
   if constexpr (NS < N) {
     constexpr int R = pick_radix(N / NS);
     constexpr int NB = N / R;
     constexpr int TASKS = B * NB;
     constexpr int PER = (TASKS + NT - 1) / NT;
     float2 v[PER][R];
+    if constexpr (OPQ) asm volatile("" : "+r"(tid));
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
-      const int t = threadIdx.x + p * NT;
+      const int t = tid + p * NT;
       if (TASKS % NT == 0 || t < TASKS) {
         const int b = t % B, j = t / B;
         const int k = j % NS;
@@ -236,9 +240,10 @@ __device__ __forceinline__ void stockham(float2* buf, const float2* tw) {
       }
     }
     __syncthreads();
+    if constexpr (OPQ) asm volatile("" : "+r"(tid));
 #pragma unroll
     for (int p = 0; p < PER; ++p) {
-      const int t = threadIdx.x + p * NT;
+      const int t = tid + p * NT;
       if (TASKS % NT == 0 || t < TASKS) {
         const int b = t % B, j = t / B;
         const int base = (j / NS) * NS * R + (j % NS);
@@ -247,15 +252,15 @@ __device__ __forceinline__ void stockham(float2* buf, const float2* tw) {
       }
     }
     __syncthreads();
-    stockham<N, NS * R, DIR, B, PI, NT>(buf, tw);
+    stockham<N, NS * R, DIR, B, PI, NT, OPQ>(buf, tw, tid);
   }
 }
 
 // B lines of length N in buf[i * PI + b]; all NT threads of the block call it.
 // Entry and exit are block-synchronised.
-template <int N, int DIR, int B, int PI, int NT>
+template <int N, int DIR, int B, int PI, int NT, bool OPQ = false>
 __device__ __forceinline__ void fft_lines(float2* buf, const float2* tw) {
-  stockham<N, 1, DIR, B, PI, NT>(buf, tw);
+  stockham<N, 1, DIR, B, PI, NT, OPQ>(buf, tw, threadIdx.x);
 }
 
 // Asynchronous global -> shared copies (LDGSTS); completion by wait_all.

@@ -13,6 +13,7 @@
 #include "fft.cuh"
 #include "taps.cuh"
 #include "tiling.cuh"
+#include "twopass.cuh"
 
 namespace cpra {
 
@@ -37,11 +38,6 @@ __device__ __forceinline__ void store_row_pair_spectra(const float2* buf, float2
     Hp_rows[(size_t)(2 * p) * H + k] = h0;
     Hp_rows[(size_t)(2 * p + 1) * H + k] = h1;
   }
-}
-
-template <int N>
-__device__ __forceinline__ void load_twiddles(float2* tw_s, const float2* tw) {
-  for (int i = threadIdx.x; i < N; i += blockDim.x) tw_s[i] = tw[i];
 }
 
 // ---------------------------------------------------------------- prime
@@ -102,32 +98,6 @@ k_prime(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
 }
 
 // ---------------------------------------------------------------- column pass
-// G' = a G / |G|; err += w (|G| - a)^2 in FP32 (a thread's few dozen
-// terms; FP64 across threads and blocks)
-__device__ __forceinline__ float2 project(float2 G, float a, float& err, float w) {
-  if (a < 0.0f) return G;  // an unmeasured pair (mask): free, no error term
-  const float m = sqrtf(G.x * G.x + G.y * G.y);
-  const float d = m - a;
-  err = fmaf(w * d, d, err);
-  if (m > 0.0f) {
-    const float s = a / m;
-    return make_float2(G.x * s, G.y * s);
-  }
-  return make_float2(a, 0.0f);
-}
-
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < NT / 32; ++i) s += red[i];
-  return s;
-}
-
 template <int N>
 __global__ void __launch_bounds__(ColTile<N>::NT)
 k_colpass(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
@@ -164,20 +134,9 @@ k_colpass(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
     if (c == 0) continue;
     buf[idx] = project(buf[idx], An[(size_t)c * N + ky], err, 2.0f);
   }
-  if (c0 == 0) {
-    // packed column: Z = G(.,0) + i G(.,N/2), both Hermitian along ky
-    for (int ky = threadIdx.x; ky <= H; ky += NT) {
-      const int km = (N - ky) % N;
-      const float2 z = buf[ky * B], zm = buf[km * B];
-      const float2 g0 = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
-      const float2 gn = make_float2(0.5f * (z.y + zm.y), 0.5f * (zm.x - z.x));
-      const float w = (ky == 0 || ky == H) ? 1.0f : 2.0f;
-      const float2 p0 = project(g0, An[ky], err, w);
-      const float2 pn = project(gn, A_nyq[(size_t)n * N + ky], err, w);
-      buf[ky * B] = make_float2(p0.x - pn.y, p0.y + pn.x);
-      if (km != ky) buf[km * B] = make_float2(p0.x + pn.y, pn.x - p0.y);
-    }
-  }
+  if (c0 == 0) 
+    project_column0<N, B, NT>(buf, [&](int ky) { return An[ky]; },
+                              [&](int ky) { return A_nyq[(size_t)n * N + ky]; }, err);
   __syncthreads();
   fft_lines<N, +1, B, B, NT>(buf, tw_s);
   const float inv = 1.0f / N;
