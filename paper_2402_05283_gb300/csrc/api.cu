@@ -413,13 +413,17 @@ Launch plan_launch(const cpra_plan_s* p, int64_t step, int ntiles, int first_til
 cpra_status build_gridding(cpra_plan_s* p) {
   const int N = p->N, Np = p->Np, NN = N * N;
   std::vector<double> wsum(NN, 0.0);
-  struct Ent { int32_t cell, idx; double w; };
+  const int HC = N / 2 + 1;
+  struct Ent { int32_t cell; uint32_t at; double w; };
   std::vector<Ent> ents;
   ents.reserve((size_t)4 * Np * N);
   for (int n = 0; n < Np; ++n) {
     const double c = std::cos(p->theta[n]), s = std::sin(p->theta[n]);
     for (int k = 0; k < N; ++k) {
       const double ku = k < N / 2 ? k : k - N;
+      // the line of F: columns ku = 0 .. N/2 - 1 and -N/2 are stored, the others
+      // are their partners' conjugates
+      const uint32_t at = (uint32_t)(n * HC + (k <= N / 2 ? k : N - k)) | (k > N / 2 ? 0x80000000u : 0u);
       const double px = ku * c, py = ku * s;
       const double i0 = std::floor(px), j0 = std::floor(py);
       const double fx = px - i0, fy = py - j0;
@@ -432,7 +436,7 @@ cpra_status build_gridding(cpra_plan_s* p) {
           ii = ii < 0 ? ii + N : (ii >= N ? ii - N : ii);
           jj = jj < 0 ? jj + N : (jj >= N ? jj - N : jj);
           const int cell = jj * N + ii;
-          ents.push_back({cell, n * N + k, w});
+          ents.push_back({cell, at, w});
           wsum[cell] += w;
         }
     }
@@ -442,37 +446,27 @@ cpra_status build_gridding(cpra_plan_s* p) {
     if (wsum[e.cell] >= 1e-12) ptr[e.cell + 1]++;
   for (int i = 0; i < NN; ++i) ptr[i + 1] += ptr[i];
   const int64_t n_ent = ptr[NN];
-  std::vector<int32_t> idx(n_ent > 0 ? n_ent : 1);
-  std::vector<double> wv(n_ent > 0 ? n_ent : 1);
+  std::vector<GridEnt> list(n_ent > 0 ? n_ent : 1);
   std::vector<int32_t> fillp(ptr.begin(), ptr.end() - 1);
   for (const Ent& e : ents) {
     if (wsum[e.cell] < 1e-12) continue;
-    const int32_t o = fillp[e.cell]++;
-    idx[o] = e.idx;
-    wv[o] = e.w / wsum[e.cell];
+    list[fillp[e.cell]++] = {e.at, (float)(e.w / wsum[e.cell])};
   }
   Assembly& a = p->asmb;
-  if (a.ent_idx && a.n_ent < n_ent) {
-    dev_free(p, a.ent_idx);
-    dev_free(p, a.ent_w);
-    a.ent_idx = nullptr;
-    a.ent_w = nullptr;
+  if (a.ents && a.n_ent < n_ent) {
+    dev_free(p, a.ents);
+    a.ents = nullptr;
   }
-  if (!a.ent_idx) {
-    const int64_t cap = n_ent > 0 ? n_ent : 1;
-    a.ent_idx = (int32_t*)dev_alloc(p, sizeof(int32_t) * cap);
-    a.ent_w = (double*)dev_alloc(p, sizeof(double) * cap);
-    if (!a.ent_idx || !a.ent_w) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "gridding allocation failed");
+  if (!a.ents) {
+    a.ents = (GridEnt*)dev_alloc(p, sizeof(GridEnt) * (n_ent > 0 ? n_ent : 1));
+    if (!a.ents) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "gridding allocation failed");
   }
   a.n_ent = n_ent;
   CK(cudaMemcpyAsync(a.cell_ptr, ptr.data(), sizeof(int32_t) * (NN + 1), cudaMemcpyHostToDevice,
                      p->stream), "grid ptr upload");
-  if (n_ent > 0) {
-    CK(cudaMemcpyAsync(a.ent_idx, idx.data(), sizeof(int32_t) * n_ent, cudaMemcpyHostToDevice,
-                       p->stream), "grid idx upload");
-    CK(cudaMemcpyAsync(a.ent_w, wv.data(), sizeof(double) * n_ent, cudaMemcpyHostToDevice,
-                       p->stream), "grid w upload");
-  }
+  if (n_ent > 0)
+    CK(cudaMemcpyAsync(a.ents, list.data(), sizeof(GridEnt) * n_ent, cudaMemcpyHostToDevice, p->stream),
+       "grid upload");
   CK(cudaStreamSynchronize(p->stream), "grid upload sync");
   a.ready = true;
   a.grid_ok = true;
@@ -1118,11 +1112,13 @@ static cpra_status ensure_assembly(cpra_plan_s* p) {
   const size_t N = p->N, Np = p->Np, NN = N * N;
   Assembly& a = p->asmb;
   if (!a.F) {
-    a.F = (float2*)dev_alloc(p, Np * NN * 8);
+    a.F = (float2*)dev_alloc(p, spectra_bytes(p->N, p->Np));
+    a.corr = (float2*)dev_alloc(p, corr_bytes(p->N, p->Np));
+    a.ramps = (float2*)dev_alloc(p, ramps_bytes(p->N, p->Np));
     a.vol = (float2*)dev_alloc(p, N * NN * 8);
     a.cell_ptr = (int32_t*)dev_alloc(p, (NN + 1) * 4);
     a.moments = (double*)dev_alloc(p, 3 * Np * 8);
-    if (!a.F || !a.vol || !a.cell_ptr || !a.moments)
+    if (!a.F || !a.corr || !a.ramps || !a.vol || !a.cell_ptr || !a.moments)
       return fail(p, CPRA_ERR_OUT_OF_MEMORY, "assembly allocation failed");
   }
   if (!a.grid_ok) return build_gridding(p);
@@ -1198,50 +1194,63 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
   if (!p->mg_acc) {
     p->mg_acc = (float2*)dev_alloc(p, Np * NN * 8);
     p->mg_ref = (float2*)dev_alloc(p, NN * 8);
-    p->mg_dist = (double*)dev_alloc(p, 2 * 8);
-    if (!p->mg_acc || !p->mg_ref || !p->mg_dist) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
+    if (!p->mg_acc || !p->mg_ref) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
   }
-  if (prtf && !p->mg_mag) {
-    p->mg_mag = (float*)dev_alloc(p, Np * NN * 4);
-    if (!p->mg_mag) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
+  if (prtf && !p->mg_rings) {
+    p->mg_rings = (double*)dev_alloc(p, sizeof(double) * Np * (N / 2) + sizeof(unsigned) * (N / 2));
+    if (!p->mg_rings) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
+  }
+  if (p->mg_cap < n_l) {  // (the stream is idle)
+    dev_free(p, p->mg_guess);
+    dev_free(p, p->mg_dist);
+    dev_free(p, p->mg_ramps);
+    p->mg_cap = 0;
+    p->mg_guess = (MergeGuess*)dev_alloc(p, sizeof(MergeGuess) * n_l);
+    p->mg_dist = (double*)dev_alloc(p, sizeof(double) * 2 * n_l);
+    p->mg_ramps = (float2*)dev_alloc(p, ramps_bytes(N, Np) * n_l);
+    if (!p->mg_guess || !p->mg_dist || !p->mg_ramps) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
+    p->mg_cap = n_l;
   }
   p->merged = false;
-  CK(cudaMemsetAsync(p->mg_acc, 0, Np * NN * 8, p->stream), "merge clear");
-  if (prtf) CK(cudaMemsetAsync(p->mg_mag, 0, Np * NN * 4, p->stream), "merge clear");
-  CK(cudaStreamSynchronize(p->stream), "merge sync");
-  std::vector<int32_t> flips(n_l, 0);
+  // R2C rows of rho and the mass-centre ramps of every kept guess, each on
+  // its own stream
+  std::vector<MergeGuess> table(n_l);
+  const size_t ramp_step = ramps_bytes(N, Np) / sizeof(float2);
   for (int k = 0; k < n_l; ++k) {
     cpra_plan_s* g = guesses[order[k]];
-    cudaStream_t gs = g->stream;
     st = upload_rho_rows(g);
     if (st != CPRA_OK) return fail(p, st, std::string("guess: ") + g->err);
-    MergeArgs ma{};
-    ma.ref = p->mg_ref;
-    ma.n0 = twin_ref;
-    cudaError_t e = timed(g, CPRA_KERNEL_ASSEMBLE, [&] {
-      cudaError_t r = launch_prime(plan_launch(g, 0, Np));
-      if (r != cudaSuccess) return r;
-      if (k == 0) return launch_merge_guess(g, p->asmb.moments, kSpecRef, ma, 1, gs);
-      ma.dist = p->mg_dist;
-      r = cudaMemsetAsync(p->mg_dist, 0, 2 * sizeof(double), gs);
-      return r == cudaSuccess ? launch_merge_guess(g, p->asmb.moments, kSpecDist, ma, 1, gs) : r;
-    });
-    CK(e, "merge spectra");
-    g->hp_valid = false;
-    if (k > 0) {  // R16: the version nearer to the best episode's reference PO
-      double d[2];
-      CK(cudaMemcpyAsync(d, p->mg_dist, sizeof(d), cudaMemcpyDeviceToHost, gs), "merge distances");
-      CK(cudaStreamSynchronize(gs), "merge sync");
-      flips[k] = d[1] < d[0] ? 1 : 0;
-    }
-    ma = MergeArgs{};
-    ma.acc = p->mg_acc;
-    ma.mag = prtf ? p->mg_mag : nullptr;
-    ma.inv = flips[k];
+    float2* ramps = p->mg_ramps + ramp_step * k;
     CK(timed(g, CPRA_KERNEL_ASSEMBLE, [&] {
-         return launch_merge_guess(g, p->asmb.moments, kSpecAcc, ma, Np, gs);
-       }), "merge accumulate");
-    CK(cudaStreamSynchronize(gs), "merge sync");
+         cudaError_t r = launch_prime(plan_launch(g, 0, Np));
+         return r == cudaSuccess ? launch_ramps(g, p->asmb.moments, ramps, g->stream) : r;
+       }), "merge spectra");
+    g->hp_valid = false;
+    table[k] = MergeGuess{g->Hp, ramps, 0, 0};
+    // the moments buffer is shared: the next guess waits for this one unless
+    // they share a stream
+    if (g->stream != p->stream || (k + 1 < n_l && guesses[order[k + 1]]->stream != g->stream))
+      CK(cudaStreamSynchronize(g->stream), "merge sync");
+  }
+  MergeArgs ma{};
+  ma.n0 = twin_ref;
+  ma.guess = p->mg_guess;
+  ma.ref = p->mg_ref;
+  ma.dist = p->mg_dist;
+  std::vector<int32_t> flips(n_l, 0);
+  auto upload_table = [&] {
+    return cudaMemcpyAsync(p->mg_guess, table.data(), sizeof(MergeGuess) * n_l, cudaMemcpyHostToDevice,
+                           p->stream);
+  };
+  CK(upload_table(), "merge table");
+  if (n_l > 1) {  // R16: the version nearer to the best episode's reference PO
+    CK(timed(p, CPRA_KERNEL_ASSEMBLE, [&] { return launch_merge_twins(p, ma, n_l); }), "merge twins");
+    std::vector<double> d(2 * (size_t)n_l);
+    CK(cudaMemcpyAsync(d.data(), p->mg_dist, sizeof(double) * 2 * n_l, cudaMemcpyDeviceToHost, p->stream),
+       "merge distances");
+    CK(cudaStreamSynchronize(p->stream), "merge sync");
+    for (int k = 1; k < n_l; ++k) table[k].inv = flips[k] = d[2 * k + 1] < d[2 * k] ? 1 : 0;
+    CK(upload_table(), "merge table");
   }
   float* prtf_dev = nullptr;
   const bool prtf_host = prtf && !is_device_ptr(prtf);
@@ -1253,8 +1262,8 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
     prtf_dev = prtf_host ? p->mg_prtf : prtf;
   }
   CK(timed(p, CPRA_KERNEL_ASSEMBLE, [&] {
-       return launch_merge_finish(p, p->mg_acc, p->mg_mag, prtf_dev, n_l);
-     }), "merge finish");
+       return launch_merge(p, ma, n_l, p->mg_acc, prtf ? p->mg_rings : nullptr, prtf_dev);
+     }), "merge");
   p->asmb.ready = true;
   p->merged = true;
   p->vol_state = 1;

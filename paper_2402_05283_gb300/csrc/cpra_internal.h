@@ -26,6 +26,7 @@ namespace cpra {
 
 struct JobStatic;
 struct JobStep;
+struct MergeGuess;
 
 // Device-side status of a plan.  It lives in mapped, pinned host memory, so
 // kernels set it with plain stores and the host reads it without waiting
@@ -37,12 +38,20 @@ struct DevStatus {
 constexpr unsigned kStatusNonFinite = 1u;
 constexpr unsigned kStatusTimeout = 2u;  // a bounded device wait gave up
 
+// A sample of a grid cell: its line of F, n * (N/2 + 1) + |ku| (bit 31: ku < 0,
+// the conjugate is read), and its bilinear weight (normalised in FP64).
+struct GridEnt {
+  uint32_t at;
+  float w;
+};
+
 struct Assembly {
-  float2* F = nullptr;        // [Np][N][N] z-transformed spectra, [n][ku][z]
+  float2* F = nullptr;        // z-transformed spectra, [z / 8][n][ku = 0 .. N/2][z % 8]
+  float2* corr = nullptr;     // [Np][N/2 + 1] what F(-ku) is beside conj F(ku) (k_assemble.cu)
+  float2* ramps = nullptr;    // per angle the unit ramps of its mass-centre move
   float2* vol = nullptr;      // [N][N][N] grid, then the centred volume
   int32_t* cell_ptr = nullptr;  // [N*N + 1] CSR rows (cells ky*N + kx)
-  int32_t* ent_idx = nullptr;   // sample index n*N + ku
-  double* ent_w = nullptr;      // normalised bilinear weight
+  cpra::GridEnt* ents = nullptr;  // samples of the cells
   double* moments = nullptr;    // [Np][3] sum rho, sum rho*z, sum rho*u
   int64_t n_ent = 0;
   bool ready = false;    // a volume of the current angles may be read
@@ -102,10 +111,13 @@ struct cpra_plan_s {
   bool masked = false;         // intensities were loaded under a mask (kernels check A_sym < 0)
   cpra::Assembly asmb;
   // Step C merge scratch (cpra_merge with this plan as destination)
-  float2* mg_acc = nullptr;    // [Np][N][N] merged spectra (sums, then the mean)
-  float* mg_mag = nullptr;     // [Np][N][N] sums of |E| for the PRTF
+  float2* mg_acc = nullptr;    // [Np][N][N] merged spectra (the mean)
   float2* mg_ref = nullptr;    // [N][N] E of the reference PO of the best guess
-  double* mg_dist = nullptr;   // [2] twin distances
+  double* mg_rings = nullptr;  // [Np][N/2] ring sums of the PRTF, then N/2 ring populations
+  int32_t mg_cap = 0;          // kept guesses that mg_guess, mg_dist and mg_ramps hold
+  cpra::MergeGuess* mg_guess = nullptr;
+  double* mg_dist = nullptr;   // [mg_cap][2] twin distances
+  float2* mg_ramps = nullptr;  // [mg_cap] ramps of the kept guesses
   float* mg_prtf = nullptr;    // [Np][N/2] PRTF staging for host outputs
   bool merged = false;         // mg_acc holds the mean of the last merge
   // Step D refinement (cpra_refine_3d)
@@ -287,21 +299,37 @@ cudaError_t launch_shrinkwrap(cpra_plan_s* p);
 
 // assembly (k_assemble.cu)
 cudaError_t launch_assemble(cpra_plan_s* p);
+size_t spectra_bytes(int N, int Np);  // Assembly::F, ::corr and ::ramps
+size_t corr_bytes(int N, int Np);
+size_t ramps_bytes(int N, int Np);
 
 // Step C merge (k_assemble.cu): modes of the spectra kernel
-enum SpecMode { kSpecF = 0, kSpecRef = 1, kSpecDist = 2, kSpecAcc = 3 };
-struct MergeArgs {
-  int n0;         // first angle of the launch
-  int inv;        // ACC: add conj(E), the spectrum of the centrally inverted PO
-  float2* ref;    // REF: E of one PO, [kz][ku] (written); DIST: read
-  float2* acc;    // ACC: [Np][kz][ku] += E or conj(E)
-  float* mag;     // ACC: [Np][kz][ku] += |E| (NULL = skip)
-  double* dist;   // DIST: [0] += sum |ref - E|^2, [1] += sum |ref - conj E|^2
+enum SpecMode { kSpecF = 0, kSpecRef = 1, kSpecDist = 2 };
+// a kept guess: its R2C rows of rho, its ramps, whether it is inverted
+struct MergeGuess {
+  const float2* Hp;
+  const float2* ramps;
+  int inv, pad;
 };
-// moments of guess g into `moments`, then the spectra kernel in `mode` over
-// angles ma.n0 .. ma.n0 + count - 1 (the R2C rows of rho are in g's Hp)
-cudaError_t launch_merge_guess(cpra_plan_s* g, double* moments, int mode, const MergeArgs& ma,
-                               int count, cudaStream_t st);
+struct MergeArgs {
+  int n0;                   // REF, DIST: the PO
+  const MergeGuess* guess;  // device table of the kept guesses, best first
+  float2* ref;              // E of PO n0 of the best guess, [kz][ku]
+  double* dist;             // [kept][2] sum |ref - E|^2, sum |ref - conj E|^2
+};
+// FP64 moments (sum rho, sum rho z, sum rho u) of rho = P_{S+} g of every angle
+cudaError_t launch_moments(cpra_plan_s* p, double* moments, cudaStream_t st);
+// the same, then the unit ramps of the mass-centre moves
+cudaError_t launch_ramps(cpra_plan_s* p, double* moments, float2* ramps, cudaStream_t st);
+// twin distances of the kept guesses, on dst's stream
+cudaError_t launch_merge_twins(cpra_plan_s* dst, const MergeArgs& ma, int n_l);
+// acc = mean of the corrected spectra, PRTF (rings and prtf not NULL), its
+// IDFT_z, gridding and the plane IFFTs into dst's volume, on dst's stream
+cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, double* rings,
+                         float* prtf);
+// inverse FFT along y of every plane of a volume, in place (k_refine_w.cu)
+cudaError_t launch_volume_ylines(int N, float2* vol, const float2* xtw, cudaStream_t st);
+
 // Step D refinement (k_refine.cu): buffers of one plan's refinement
 struct RefineArgs {
   int N, W;            // W = ceil(N/32) words per x row of S3
@@ -320,8 +348,6 @@ cudaError_t launch_refine_setup(const RefineArgs& a, const float2* vol, cudaStre
 // (cos, sin) of every angle; M from the gridding lists
 cudaError_t launch_refine_support(const RefineArgs& a, const uint32_t* S2, const double2* cs,
                                   const int2* shift, int Np, const int32_t* cell_ptr, cudaStream_t st);
-// FP64 moments (sum rho, sum rho z, sum rho u) of rho = P_{S+} g of every angle
-cudaError_t launch_moments(cpra_plan_s* p, double* moments, cudaStream_t st);
 // one iteration; err2[0..1] += sum_M |X - V|^2, sum_M |V|^2
 cudaError_t launch_refine_iter(const RefineArgs& a, double* err2, cudaStream_t st);
 // the same passes with warp-resident FFTs (k_refine_w.cu; refine_fast_supported(N))
@@ -332,11 +358,6 @@ cudaError_t launch_refine_shrink(const RefineArgs& a, const float* taps, int nta
                                  unsigned* mx, cudaStream_t st);
 // vol = P_{S3+} R
 cudaError_t launch_refine_output(const RefineArgs& a, float2* vol, cudaStream_t st);
-
-// PRTF (prtf != NULL, needs mag), acc <- acc / n_l, its IDFT_z into dst's F,
-// gridding and the plane IFFTs into dst's volume, on dst's stream
-cudaError_t launch_merge_finish(cpra_plan_s* dst, float2* acc, const float* mag, float* prtf,
-                                int n_l);
 
 bool n_supported(int N);
 

@@ -14,6 +14,7 @@
 // dozen terms) and across threads and blocks in FP64.
 #include "cpra_internal.h"
 #include "fast_kernels.cuh"
+#include "tiling.cuh"
 
 namespace cpra {
 
@@ -122,12 +123,15 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
   float2* vbuf = buf + C::BUF;  // kVConstrain: the data of the block's columns
   // thread (row y0 + k RS, column cc): a warp's rows WARPS apart, so its
   // 8-byte pieces fall on distinct banks of the odd-pitch staging rows
-  constexpr int RS = C::NT / C::CB;
-  static_assert(32 % C::CB == 0 && N % RS == 0, "line staging");
-  const int y0 = warp + C::WARPS * (lane / C::CB), cc = lane % C::CB;
+  // (blocks whose columns do not divide a warp take plain thread order)
+  constexpr int RS = C::NT / C::CB, SR = (N + RS - 1) / RS;
+  static_assert(N % C::CB == 0, "line staging");
+  const int y0 = 32 % C::CB == 0 ? warp + C::WARPS * (lane / C::CB) : threadIdx.x / C::CB;
+  const int cc = 32 % C::CB == 0 ? lane % C::CB : threadIdx.x % C::CB;
 #pragma unroll 4
-  for (int k = 0; k < N / RS; ++k) {
+  for (int k = 0; k < SR; ++k) {
     const int y = y0 + k * RS;
+    if (N % RS != 0 && y >= N) break;
     cp_async8(buf + y * C::SP + cc, base + y * estride + cc);
     if constexpr (MODE == kVConstrain)
       cp_async8(vbuf + y * C::SP + cc, V + blockIdx.y * outer + c0 + y * estride + cc);
@@ -142,6 +146,7 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
     static_for<0, FL::TB>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
+      if (!FL::b_on(t)) return;
       const int col = warp * FL::L + FL::b_line(t);
       static_for<0, FL::E2>([&](auto JJ) {
         constexpr int j = decltype(JJ)::value;
@@ -152,6 +157,7 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
     static_for<0, FL::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
+      if (!FL::a_on(t)) return;
       const int col = warp * FL::L + FL::a_line(t);
       static_for<0, FL::E1>([&](auto MM) {
         constexpr int m = decltype(MM)::value;
@@ -169,7 +175,7 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
       const int col = warp * FL::L + FL::b_line(t);
-      if (M[(size_t)ky * N + c0 + col]) {
+      if (FL::b_on(t) && M[(size_t)ky * N + c0 + col]) {
         static_for<0, FL::E2>([&](auto JJ) {
           constexpr int j = decltype(JJ)::value;
           const float2 v = vbuf[FL::b_k(t, j) * C::SP + col];
@@ -186,6 +192,7 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
     static_for<0, FL::TB>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
+      if (!FL::b_on(t)) return;
       const int col = warp * FL::L + FL::b_line(t);
       static_for<0, FL::E2>([&](auto JJ) {
         constexpr int j = decltype(JJ)::value;
@@ -199,6 +206,7 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
     static_for<0, FL::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int t = lane + 32 * i;
+      if (!FL::a_on(t)) return;
       const int col = warp * FL::L + FL::a_line(t);
       static_for<0, FL::E1>([&](auto MM) {
         constexpr int m = decltype(MM)::value;
@@ -208,8 +216,9 @@ k_vw(float2* X, const float2* __restrict__ V, const uint8_t* __restrict__ M,
   }
   __syncthreads();
 #pragma unroll 4
-  for (int k = 0; k < N / RS; ++k) {
+  for (int k = 0; k < SR; ++k) {
     const int y = y0 + k * RS;
+    if (N % RS != 0 && y >= N) break;
     base[y * estride + cc] = buf[y * C::SP + cc];
   }
   if constexpr (MODE == kVConstrain) {
@@ -296,6 +305,31 @@ cudaError_t launch_refine_fft3_w(const RefineArgs& a, cudaStream_t st) {
 #define CPRA_CASE(NN) \
   case NN: return setup_w<NN>(a, st);
     CPRA_FOR_EACH_FAST_N(CPRA_CASE)
+#undef CPRA_CASE
+    default:
+      return cudaErrorInvalidValue;
+  }
+}
+
+template <int N>
+static cudaError_t volume_ylines_n(float2* vol, const float2* xtw, cudaStream_t st) {
+  static bool done = false;
+  if (!done) {
+    cudaError_t e = attr_w(k_vw<N, kVInv>, vw_smem<N>());
+    if (e != cudaSuccess) return e;
+    done = true;
+  }
+  g_launches += 1;
+  k_vw<N, kVInv><<<dim3(N / VW<N>::CB, N), VW<N>::NT, vw_smem<N>(), st>>>(
+      vol, nullptr, nullptr, xtw, nullptr, (size_t)N * N, (size_t)N);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_volume_ylines(int N, float2* vol, const float2* xtw, cudaStream_t st) {
+  switch (N) {
+#define CPRA_CASE(NN) \
+  case NN: return volume_ylines_n<NN>(vol, xtw, st);
+    CPRA_FOR_EACH_N(CPRA_CASE)
 #undef CPRA_CASE
     default:
       return cudaErrorInvalidValue;
