@@ -154,7 +154,7 @@ cpra_status validate(const cpra_config* c, std::string& why) {
     return CPRA_ERR_INVALID_ARG;
   }
   if (c->precision != CPRA_FP32 &&
-      !(refine_fast_supported(c->N) && (c->engine == CPRA_ENGINE_AUTO || c->engine == CPRA_ENGINE_WARP))) {
+      !(tc_supported(c->N) && (c->engine == CPRA_ENGINE_AUTO || c->engine == CPRA_ENGINE_WARP))) {
     why = "tensor-core precision runs on the warp engine (N in {64, 128, 256, 512, 1024})";
     return CPRA_ERR_UNSUPPORTED;
   }
@@ -1292,7 +1292,8 @@ cpra_status cpra_refine_3d(cpra_plan_t p, int32_t n_iters, int32_t shrink_every,
   const size_t NN = (size_t)N * N, N3 = NN * N;
   if (!p->rf_X) {
     p->rf_X = (float2*)dev_alloc(p, N3 * 8);
-    p->rf_V = (float2*)dev_alloc(p, N3 * 8);
+    p->rf_W = (float2*)dev_alloc(p, N3 * 8);
+    p->rf_konst = (double*)dev_alloc(p, 2 * sizeof(double));
     p->rf_R = (float*)dev_alloc(p, N3 * 4);
     p->rf_B = (float*)dev_alloc(p, N3 * 4);
     p->rf_S3 = (uint32_t*)dev_alloc(p, NN * W3 * 4);
@@ -1301,7 +1302,7 @@ cpra_status cpra_refine_3d(cpra_plan_t p, int32_t n_iters, int32_t shrink_every,
     p->rf_taps = (float*)dev_alloc(p, sizeof(float) * N);
     p->rf_max = (unsigned*)dev_alloc(p, sizeof(unsigned));
     p->rf_shift = (int2*)dev_alloc(p, sizeof(int2) * Np);
-    if (!p->rf_X || !p->rf_V || !p->rf_R || !p->rf_B || !p->rf_S3 || !p->rf_M || !p->rf_cs ||
+    if (!p->rf_X || !p->rf_W || !p->rf_konst || !p->rf_R || !p->rf_B || !p->rf_S3 || !p->rf_M || !p->rf_cs ||
         !p->rf_taps || !p->rf_max || !p->rf_shift)
       return fail(p, CPRA_ERR_OUT_OF_MEMORY, "refinement allocation failed");
   }
@@ -1311,7 +1312,7 @@ cpra_status cpra_refine_3d(cpra_plan_t p, int32_t n_iters, int32_t shrink_every,
     if (!p->rf_err) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "refinement allocation failed");
     p->rf_err_cap = n_iters;
   }
-  RefineArgs a{N, W3, p->rf_X, p->rf_V, p->rf_R, p->rf_B, p->rf_S3, p->rf_M, p->tw, p->xtw};
+  RefineArgs a{N, W3, p->rf_X, p->rf_W, p->rf_R, p->rf_B, p->rf_S3, p->rf_M, p->xtw, p->rf_konst};
   cudaStream_t st = p->stream;
   if (p->vol_state == 1) {  // start from the Step D volume of the last assemble / merge
     // each 2D support moves with its PO: the whole-pixel part of its
@@ -1336,9 +1337,9 @@ cpra_status cpra_refine_3d(cpra_plan_t p, int32_t n_iters, int32_t shrink_every,
        "refine upload");
     CK(timed(p, CPRA_KERNEL_REFINE, [&] {
          cudaError_t e = launch_refine_setup(a, p->asmb.vol, st);
-         return e == cudaSuccess
-                    ? launch_refine_support(a, p->S, p->rf_cs, p->rf_shift, Np, p->asmb.cell_ptr, st)
-                    : e;
+         if (e == cudaSuccess)
+           e = launch_refine_support(a, p->S, p->rf_cs, p->rf_shift, Np, p->asmb.cell_ptr, st);
+         return e == cudaSuccess ? launch_refine_data(a, st) : e;
        }), "refine setup");
     CK(cudaStreamSynchronize(st), "refine sync");  // cs and shift live on this stack
     p->rf_t = 0;
@@ -1351,10 +1352,14 @@ cpra_status cpra_refine_3d(cpra_plan_t p, int32_t n_iters, int32_t shrink_every,
     CK(cudaStreamSynchronize(st), "refine sync");
   }
   if (n_iters > 0) CK(cudaMemsetAsync(p->rf_err, 0, sizeof(double) * 2 * n_iters, st), "refine clear");
+  bool in_r = true;  // the iterate is in R (else its rows are already transformed)
   for (int i = 0; i < n_iters; ++i) {
-    CK(timed(p, CPRA_KERNEL_REFINE, [&] { return launch_refine_iter(a, p->rf_err + 2 * i, st); }),
+    const bool shrink = shrink_every > 0 && (p->rf_t + 1) % shrink_every == 0;
+    const bool last = shrink || i + 1 == n_iters;
+    CK(timed(p, CPRA_KERNEL_REFINE, [&] { return launch_refine_iter(a, p->rf_err + 2 * i, in_r, last, st); }),
        "refine iteration");
-    if (shrink_every > 0 && (p->rf_t + 1) % shrink_every == 0)
+    in_r = last;
+    if (shrink)
       CK(timed(p, CPRA_KERNEL_REFINE, [&] {
            return launch_refine_shrink(a, p->rf_taps, ntaps, tau, p->rf_max, st);
          }), "refine shrink-wrap");

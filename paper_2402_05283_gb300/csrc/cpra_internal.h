@@ -123,7 +123,8 @@ struct cpra_plan_s {
   // Step D refinement (cpra_refine_3d)
   int vol_state = 0;           // 0 none, 1 Step D volume (assemble or merge), 2 refined
   float2* rf_X = nullptr;
-  float2* rf_V = nullptr;
+  float2* rf_W = nullptr;
+  double* rf_konst = nullptr;  // [2]
   float* rf_R = nullptr;
   float* rf_B = nullptr;
   uint32_t* rf_S3 = nullptr;
@@ -333,26 +334,26 @@ cudaError_t launch_volume_ylines(int N, float2* vol, const float2* xtw, cudaStre
 // Step D refinement (k_refine.cu): buffers of one plan's refinement
 struct RefineArgs {
   int N, W;            // W = ceil(N/32) words per x row of S3
-  float2* X;           // [N^3] working spectrum / volume
-  float2* V;           // [N^3] gridded spectrum, FFT order
+  float2* X;           // N^3: the data volume, then the half spectrum [z][y][HP]
+  float2* Wd;          // N^3: the data of the half spectrum (k_refine_w.cu), same layout
   float* R;            // [N^3] real iterate rho
   float* Bv;           // [N^3] shrink-wrap blur scratch
   uint32_t* S3;        // [N][N][W] 3D support bits
   uint8_t* M;          // [N][N] measured (ky, kx) cells
-  const float2* tw;    // twiddles exp(-2 pi i k/N)
-  const float2* xtw;   // warp-FFT cross twiddles (N = 64 ... 1024, powers of two)
+  const float2* xtw;   // warp-FFT cross twiddles
+  double* konst;       // [2] constant parts of the error sums
 };
-// X = vol (centred), R = Re vol, V = FFT3(X)
+// X = vol (centred), R = Re vol
 cudaError_t launch_refine_setup(const RefineArgs& a, const float2* vol, cudaStream_t st);
 // S3 from the 2D supports S2 [Np][N][W] moved by shift[n] = (dz, du), with
 // (cos, sin) of every angle; M from the gridding lists
 cudaError_t launch_refine_support(const RefineArgs& a, const uint32_t* S2, const double2* cs,
                                   const int2* shift, int Np, const int32_t* cell_ptr, cudaStream_t st);
-// one iteration; err2[0..1] += sum_M |X - V|^2, sum_M |V|^2
-cudaError_t launch_refine_iter(const RefineArgs& a, double* err2, cudaStream_t st);
-// the same passes with warp-resident FFTs (k_refine_w.cu; refine_fast_supported(N))
-cudaError_t launch_refine_fft3_w(const RefineArgs& a, cudaStream_t st);
-cudaError_t launch_refine_iter_w(const RefineArgs& a, double* err2, cudaStream_t st);
+// Wd and konst from X and M; X is free afterwards
+cudaError_t launch_refine_data(const RefineArgs& a, cudaStream_t st);
+// one iteration (first: it starts from R; last: it ends in R); err2[0] +=
+// sum_M |X - V|^2, err2[1] = sum_M |V|^2
+cudaError_t launch_refine_iter(const RefineArgs& a, double* err2, bool first, bool last, cudaStream_t st);
 // S3 <- {blur(P_{S3+} R) >= tau max} (mx: one unsigned of scratch)
 cudaError_t launch_refine_shrink(const RefineArgs& a, const float* taps, int ntaps, float tau,
                                  unsigned* mx, cudaStream_t st);
@@ -363,7 +364,7 @@ bool n_supported(int N);
 
 // two-pass engine with warp-resident FFTs (k_fast.cu)
 bool warp_engine_listed(int N);      // sizes that CPRA_ENGINE_WARP names (its kernels cover every N)
-bool refine_fast_supported(int N);   // 3D refinement passes and tensor-core forms
+bool tc_supported(int N);            // tensor-core forms
 bool fast_dims(int N, int* E1, int* E2);
 cudaError_t prepare_kernels_fast(int N);
 cudaError_t prepare_kernels_fast_tc(int N, int prec);

@@ -878,7 +878,7 @@ cudaError_t colpass_w(const Launch& L) {
   return cudaGetLastError();
 }
 
-// sizes of the 3D refinement's warp passes and of the tensor-core forms
+// sizes of the tensor-core forms
 #define CPRA_FOR_EACH_FAST_N(X) X(64) X(128) X(256) X(512) X(1024)
 // sizes at which CPRA_ENGINE_WARP can be asked for (and the persistent batch mode)
 #define CPRA_FOR_EACH_WARP_N(X) X(64) X(128) X(192) X(256) X(384) X(512) X(1024)

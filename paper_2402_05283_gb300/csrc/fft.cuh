@@ -286,6 +286,26 @@ __device__ __forceinline__ void cp_async_wait_group() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(pending) : "memory");
 }
 
+// Sums kept as a pair of FP32, s + e (48 bits): the FP64 pipe runs at about
+// one warp instruction in 16 cycles, so FP64 adds and shuffles of doubles are
+// left out of inner loops and warp reductions.
+// (s + e) <- s + e + v with the rounding error kept in e (TwoSum, Knuth)
+__device__ __forceinline__ void two_add(float& s, float& e, float v) {
+  const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+  s = t;
+}
+// the sum over the warp's lanes of s + e, in every lane
+__device__ __forceinline__ double warp_sum(float s, float e) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+    two_add(s, e, s2);
+    e = __fadd_rn(e, e2);
+  }
+  return (double)s + (double)e;
+}
+
 // support bit x of the row whose first word is at S[row_off]
 __device__ __forceinline__ bool sbit(const uint32_t* S, size_t row_off, int x) {
   return (S[row_off + (x >> 5)] >> (x & 31)) & 1u;

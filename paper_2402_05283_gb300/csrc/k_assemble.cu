@@ -34,13 +34,6 @@ CPRA_FOR_EACH_N(CPRA_CASE)
 #undef CPRA_CASE
 
 // ---------------------------------------------------------------- moments
-// (s + e) <- s + v with the rounding error kept in e (TwoSum)
-__device__ __forceinline__ void two_add(float& s, float& e, float v) {
-  const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
-  e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
-  s = t;
-}
-
 // One warp per kMomRows rows: each lane sums its pixels of a row in FP32 (at
 // most N/32 terms) and its rows as pairs of FP32 (48 bits, with the exact
 // products by y); FP64 across lanes, warps and CTAs.  Bound by HBM: the FP64
@@ -73,12 +66,7 @@ __global__ void k_moments(const float* __restrict__ g, const uint32_t* __restric
     two_add(sz, ez, pz);
     ez = __fadd_rn(ez, fmaf(p0, (float)y, -pz));
   }
-  double m0 = (double)s0 + (double)e0, mz = (double)sz + (double)ez, mu = (double)su + (double)eu;
-  for (int o = 16; o > 0; o >>= 1) {
-    m0 += __shfl_down_sync(0xffffffffu, m0, o);
-    mz += __shfl_down_sync(0xffffffffu, mz, o);
-    mu += __shfl_down_sync(0xffffffffu, mu, o);
-  }
+  const double m0 = warp_sum(s0, e0), mz = warp_sum(sz, ez), mu = warp_sum(su, eu);
   if (lane == 0) {
     red[0][warp] = m0;
     red[1][warp] = mz;

@@ -10,7 +10,7 @@ namespace cpra {
 CPRA_FOR_EACH_N(CPRA_CASE)
 #undef CPRA_CASE
 
-bool refine_fast_supported(int N) {
+bool tc_supported(int N) {
   switch (N) {
 #define CPRA_CASE(NN) case NN:
     CPRA_FOR_EACH_FAST_N(CPRA_CASE)

@@ -61,20 +61,10 @@ __device__ __forceinline__ int opaque_tid() {
   return t;
 }
 
-// Adds the warp's error terms to hist[at] (at < 0: nowhere) in FP64.  The
-// sum across lanes runs on pairs of FP32 (TwoSum, 48 bits): FP64 shuffles and
-// adds on the critical path of every iteration took 2500 cycles, these 400.
+// adds the warp's error terms to hist[at] (at < 0: nowhere) in FP64
 __device__ __forceinline__ void add_error(float e, double* hist, long long at) {
-  float lo = 0.0f;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, e, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    const float s = __fadd_rn(e, h2), b = __fsub_rn(s, e);
-    const float r = __fadd_rn(__fsub_rn(e, __fsub_rn(s, b)), __fsub_rn(h2, b));
-    lo = __fadd_rn(__fadd_rn(lo, l2), r);
-    e = s;
-  }
-  if ((threadIdx.x & 31) == 0 && at >= 0) atomicAdd(hist + at, (double)e + (double)lo);
+  const double s = warp_sum(e, 0.0f);
+  if ((threadIdx.x & 31) == 0 && at >= 0) atomicAdd(hist + at, s);
 }
 
 template <int N>
