@@ -187,6 +187,159 @@ __global__ void k_sw_thresh(const float* __restrict__ b, const unsigned* __restr
   }
 }
 
+// ---------------------------------------------------------------- one tile a block
+// Both blurs of a 64 x 32 tile in one kernel: rho = P_{S+} g of the tile and
+// its halo is staged once, the rows are blurred into shared memory for the
+// tile and its vertical halo, then the columns from there; every output adds
+// its terms in the order t = 0, 1, ... of the separate blurs, so it is the
+// same float.  The tile's maximum goes to tmax[plane][tile] and the threshold
+// kernel takes the maximum over tiles, so nothing has to be cleared first.
+// The halo costs 1.9 times the row work of the separate kernels and saves
+// their intermediate array and, above all, launches: a support update beside a
+// detector is a few patterns, and each launch is 2 to 10 us of latency.  Taken
+// for up to kTileTaps taps (sigma 2 has 29) and N >= 64, where one wrap of an
+// index is enough; the separate blurs stay for the rest.
+// 16 patterns of N = 256: seven launches 40 us a call, two launches 23.
+constexpr int kTileX = 64, kTileY = 32, kTileTaps = 33;
+constexpr int kTileRows = kTileY + kTileTaps - 1;      // staged rows at most
+constexpr int kTilePA = kTileX + kTileTaps;            // pitches: odd
+constexpr int kTilePB = kTileX + 1;
+struct TileTaps {
+  float v[kTileTaps];
+};
+__host__ __device__ constexpr int sw_tiles_x(int N) { return (N + kTileX - 1) / kTileX; }
+__host__ __device__ constexpr int sw_tiles(int N) { return sw_tiles_x(N) * ((N + kTileY - 1) / kTileY); }
+
+// U8: the support is bytes (nonzero = in), else bits, W words a row
+template <bool U8>
+__global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, const void* __restrict__ S, float* b,
+                                                 float* tmax, const TileTaps taps, int ntaps, int lo, int N, int W) {
+  static_assert(kTilePA % 2 == 1 && kTilePB % 2 == 1, "pitches");
+  __shared__ float A[kTileRows * kTilePA];
+  __shared__ float B[kTileRows * kTilePB];
+  __shared__ float tp[kTileTaps];
+  __shared__ float red[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = blockIdx.y, tx = blockIdx.x % sw_tiles_x(N), ty = blockIdx.x / sw_tiles_x(N);
+  const int x0 = tx * kTileX, y0 = ty * kTileY;
+  const int rows = kTileY + ntaps - 1, cols = kTileX + ntaps - 1;
+  const int off = -lo - (ntaps - 1);  // staged element k is pixel x0 + k + off (mod N)
+  if (threadIdx.x < ntaps) tp[threadIdx.x] = taps.v[threadIdx.x];
+  for (int r = warp; r < rows; r += 8) {
+    int y = y0 + r + off;
+    y = y < 0 ? y + N : (y >= N ? y - N : y);
+    const size_t row = (size_t)n * N + y;
+#pragma unroll 3
+    for (int c = lane; c < cols; c += 32) {
+      int x = x0 + c + off;
+      x = x < 0 ? x + N : (x >= N ? x - N : x);
+      const float v = __ldg(g + row * N + x);
+      bool in;
+      if constexpr (U8) in = __ldg(static_cast<const uint8_t*>(S) + row * N + x) != 0;
+      else in = (__ldg(static_cast<const uint32_t*>(S) + row * W + (x >> 5)) >> (x & 31)) & 1u;
+      A[r * kTilePA + c] = (in && v >= 0.0f) ? v : 0.0f;
+    }
+  }
+  __syncthreads();
+  // rows: a lane a row (odd pitch: no bank conflicts), eight outputs a thread
+  // from a register window, one shared load a tap
+  for (int q = warp; q < (kTileX / 8) * ((rows + 31) / 32); q += 8) {
+    const int r = (q / (kTileX / 8)) * 32 + lane, xb = (q % (kTileX / 8)) * 8;
+    if (r >= rows) continue;
+    const float* h = A + r * kTilePA + xb + ntaps - 1;  // output xb + i at tap t reads h[i - t]
+    float w[8], acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      w[i] = h[i];
+      acc[i] = 0.0f;
+    }
+    for (int t = 0; t < ntaps; ++t) {
+      const float c = tp[t];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] = fmaf(c, w[i], acc[i]);
+#pragma unroll
+      for (int i = 7; i > 0; --i) w[i] = w[i - 1];
+      if (t + 1 < ntaps) w[0] = h[-t - 1];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) B[r * kTilePB + xb + i] = acc[i];
+  }
+  __syncthreads();
+  // columns: a thread eight rows of one column
+  const int x = threadIdx.x % kTileX, yb = (threadIdx.x / kTileX) * 8;
+  float m = 0.0f;
+  {
+    const float* h = B + (yb + ntaps - 1) * kTilePB + x;
+    float w[8], acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      w[i] = h[i * kTilePB];
+      acc[i] = 0.0f;
+    }
+    for (int t = 0; t < ntaps; ++t) {
+      const float c = tp[t];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] = fmaf(c, w[i], acc[i]);
+#pragma unroll
+      for (int i = 7; i > 0; --i) w[i] = w[i - 1];
+      if (t + 1 < ntaps) w[0] = h[-(t + 1) * kTilePB];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (x0 + x < N && y0 + yb + i < N) {
+        b[((size_t)n * N + y0 + yb + i) * N + x0 + x] = acc[i];
+        m = fmaxf(m, acc[i]);
+      }
+  }
+  m = warp_max(m);
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float t = 0.0f;
+    for (int i = 0; i < 8; ++i) t = fmaxf(t, red[i]);
+    tmax[(size_t)n * sw_tiles(N) + blockIdx.x] = t;
+  }
+}
+
+// the maximum of a plane from its tiles, in every thread of the block
+__device__ __forceinline__ float sw_plane_max(const float* __restrict__ tmax, int tiles, float* red) {
+  float m = 0.0f;
+  for (int i = threadIdx.x; i < tiles; i += blockDim.x) m = fmaxf(m, __ldg(tmax + i));
+  m = warp_max(m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = 0.0f;
+  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) m = fmaxf(m, red[i]);
+  return m;
+}
+
+// out <- {b >= tau max b} as bytes (in, as 0 / 1, where max b is 0), four
+// consecutive pixels a thread where WIDE (4-byte aligned supports), else one
+template <bool WIDE>
+__global__ void __launch_bounds__(256) k_sw_thresh_u8(const float* __restrict__ b, const float* __restrict__ tmax,
+                                                      const uint8_t* in, uint8_t* out, float tau, int N) {
+  __shared__ float red[8];
+  const int n = blockIdx.y;
+  const float m = sw_plane_max(tmax + (size_t)n * sw_tiles(N), sw_tiles(N), red);
+  const float thr = tau * m;
+  const size_t base = (size_t)n * N * N;
+  const int i = (blockIdx.x * 256 + threadIdx.x) * (WIDE ? 4 : 1);
+  if (i >= N * N) return;
+  if constexpr (WIDE) {
+    uchar4 o;
+    if (m > 0.0f) {
+      const float4 v = *reinterpret_cast<const float4*>(b + base + i);
+      o = make_uchar4(v.x >= thr, v.y >= thr, v.z >= thr, v.w >= thr);
+    } else {
+      const uchar4 s = *reinterpret_cast<const uchar4*>(in + base + i);
+      o = make_uchar4(s.x != 0, s.y != 0, s.z != 0, s.w != 0);
+    }
+    *reinterpret_cast<uchar4*>(out + base + i) = o;
+  } else {
+    out[base + i] = m > 0.0f ? b[base + i] >= thr : in[base + i] != 0;
+  }
+}
+
 template <int CW>
 static cudaError_t blur_cols_go(dim3 grid, size_t smem, const float* in, float* out, const float* taps,
                                 int ntaps, int lo, int N, size_t outer, size_t estride, unsigned* mx,
@@ -349,6 +502,7 @@ extern "C" cpra_status cpra_shrinkwrap_static(const float* g, const uint8_t* S_i
   for (int d = 0; d < N; ++d)
     for (int m = -M; m <= M; ++m) {
       const double t = d + (double)m * N;
+      if (t * t > 1500.0 * sg * sg) continue;  // exp(-750) is 0 in FP64
       w[d] += std::exp(-t * t / (2.0 * sg * sg));
     }
   double sum = 0.0;
@@ -369,6 +523,22 @@ extern "C" cpra_status cpra_shrinkwrap_static(const float* g, const uint8_t* S_i
   cudaStream_t st = (cudaStream_t)stream;
   const int W = (N + 31) / 32;
   const int lo = -(ntaps / 2) + ((ntaps % 2) ? 0 : 1);
+  if (N >= kTileX && ntaps <= kTileTaps) {
+    TileTaps tt{};
+    for (int t = 0; t < ntaps; ++t) tt.v[t] = taps.v[t];
+    float* tmax = reinterpret_cast<float*>(sc.mx);  // 64 x 32 pixels a tile: fewer than its 4096 entries
+    const bool wide = (((uintptr_t)S_in | (uintptr_t)S_out) & 3) == 0;
+    g_launches += 2;
+    k_sw_tile<true><<<dim3(sw_tiles(N), count), 256, 0, st>>>(g, S_in, sc.b, tmax, tt, ntaps, lo, N, W);
+    if (wide)
+      k_sw_thresh_u8<true><<<dim3((N * N / 4 + 255) / 256, count), 256, 0, st>>>(sc.b, tmax, S_in, S_out, tau, N);
+    else
+      k_sw_thresh_u8<false><<<dim3((N * N + 255) / 256, count), 256, 0, st>>>(sc.b, tmax, S_in, S_out, tau, N);
+    e = cudaGetLastError();
+    if (e != cudaSuccess)
+      return record_error(CPRA_ERR_CUDA, std::string("shrink-wrap launch: ") + cudaGetErrorString(e));
+    return CPRA_OK;
+  }
   g_launches += 1;
   k_sw_static_taps<<<1, 256, 0, st>>>(taps, sc.taps, ntaps);
   e = cudaGetLastError();
