@@ -172,16 +172,15 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
       store_f<N, FL>(a, F, n, Np, H, lane, [](int line) { return line == 0; });
     }
   } else {
-    double d_plain = 0.0, d_twin = 0.0;
+    float dp = 0.0f, dpe = 0.0f, dt = 0.0f, dte = 0.0f;  // |ref - E|^2, |ref - conj E|^2
     auto take = [&](int kz, int ku, float2 v) {
       if constexpr (MODE == kSpecRef) {
         ma.ref[(size_t)kz * N + ku] = v;
       } else {
         const float2 r = ma.ref[(size_t)kz * N + ku];
-        const double ax = (double)r.x - v.x, ay = (double)r.y - v.y;  // |ref - E|^2
-        const double by = (double)r.y + v.y;                          // |ref - conj E|^2
-        d_plain += ax * ax + ay * ay;
-        d_twin += ax * ax + by * by;
+        const float ax = r.x - v.x, ay = r.y - v.y, by = r.y + v.y;
+        two_add(dp, dpe, fmaf(ax, ax, ay * ay));
+        two_add(dt, dte, fmaf(ax, ax, by * by));
       }
     };
     each_b<FL>(lane, [&](auto II, auto JJ, int t) {
@@ -198,10 +197,7 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
       }
     });
     if constexpr (MODE == kSpecDist) {
-      for (int o = 16; o > 0; o >>= 1) {
-        d_plain += __shfl_down_sync(0xffffffffu, d_plain, o);
-        d_twin += __shfl_down_sync(0xffffffffu, d_twin, o);
-      }
+      const double d_plain = warp_sum(dp, dpe), d_twin = warp_sum(dt, dte);
       if (lane == 0) {
         atomicAdd(ma.dist + 2 * blockIdx.y + 0, d_plain);
         atomicAdd(ma.dist + 2 * blockIdx.y + 1, d_twin);
@@ -216,9 +212,10 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
 // kz = -N/2, whose partner sum is kept beside the block.  Bound by HBM: every
 // guess's packed spectrum is read once, the mean and F are written once
 // (one pass over the full-plane sums a guess, then separate PRTF and IDFT_z
-// passes, took 1.88 ms for four guesses at N = 256, 144 angles; this @@).
+// passes, took 1.88 ms for four guesses at N = 256, 144 angles; one pass 0.25
+// ms at one CTA an SM and 0.16 at two).
 template <int N>
-__global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, 1)
+__global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, ColW<N, kPrecFP32>::NT <= 256 && N <= 512 ? 2 : 1)
 k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* counts, float2* F,
         float2* corr, const float2* __restrict__ xtw) {
   using C = ColW<N, kPrecFP32>;
@@ -364,18 +361,19 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
 // kHeavy is summed by the whole block, its samples spread over the 64 quads
 // (one thread a cell walked the list alone: 80 us of 83 at N = 128, 90
 // angles).  Sums run in a fixed order.  Bound by L2: four reads a sample and
-// plane.  N = 512, 360 angles, with the transform along kx: @@ ms; gather
+// plane.  N = 512, 360 angles, with the transform along kx: 0.99 ms; gather
 // 1.04 and rows 0.63 as separate passes over V.
 constexpr int kHeavy = 32;
+constexpr int kStaged = 2560;  // samples of a row held in shared memory (else read from L2)
 template <int N> struct GridCfg {
   using FL = typename WLines<N, kPrecFP32>::type;
   static constexpr int L = FL::L, H = N / 2, HC = H + 1;
   static constexpr int NZC = (N + 7) / 8;  // chunks of eight planes
   // pitch of a line: at least N, room for the warp's tile, 2 mod 8 (the four
-  // planes pairs of a quad then start four banks apart)
+  // plane pairs of a quad then start four banks apart)
   static constexpr int P0 = (FL::TSIZE + L - 1) / L > N ? (FL::TSIZE + L - 1) / L : N;
   static constexpr int LP = (P0 + 5) / 8 * 8 + 2;
-  static constexpr size_t SMEM = sizeof(float2) * (N + 8 * L * LP);
+  static constexpr size_t SMEM = sizeof(float2) * (N + 8 * L * LP + kStaged) + sizeof(int) * (N + 4);
   static_assert(LP >= P0 && LP % 8 == 2, "line pitch");
 };
 
@@ -383,19 +381,35 @@ struct GridAcc {
   float4 v;   // planes 2q and 2q + 1
   float2 c;   // sum of w corr over samples of ku < 0
 };
-__device__ __forceinline__ void grid_add(GridAcc& s, const GridEnt e, const float4* __restrict__ Fc,
-                                         const float2* __restrict__ corr, int q) {
-  const uint32_t at = e.at & 0x7fffffffu;
-  const float4 f = __ldg(Fc + (size_t)at * 4 + q);
+__device__ __forceinline__ void grid_add(GridAcc& s, const GridEnt e, const float4 f,
+                                         const float2* __restrict__ corr) {
   const float wy = (e.at >> 31) ? -e.w : e.w;  // a sample of ku < 0 reads the conjugate
   s.v.x = fmaf(e.w, f.x, s.v.x);
   s.v.y = fmaf(wy, f.y, s.v.y);
   s.v.z = fmaf(e.w, f.z, s.v.z);
   s.v.w = fmaf(wy, f.w, s.v.w);
   if (e.at >> 31) {
-    const float2 c = __ldg(corr + at);
+    const float2 c = __ldg(corr + (e.at & 0x7fffffffu));
     s.c.x = fmaf(e.w, c.x, s.c.x);
     s.c.y = fmaf(e.w, c.y, s.c.y);
+  }
+}
+// s += the samples e0, e0 + step, ... < e1, four lines of F in flight
+template <class E>
+__device__ __forceinline__ void grid_sum(GridAcc& s, E ents, int e0, int e1, int step,
+                                         const float4* __restrict__ Fc, const float2* __restrict__ corr) {
+  for (int e = e0; e < e1; e += 4 * step) {
+    GridEnt g[4];
+    float4 f[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (e + i * step < e1) {
+        g[i] = ents[e + i * step];
+        f[i] = __ldg(Fc + (size_t)(g[i].at & 0x7fffffffu) * 4);
+      }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (e + i * step < e1) grid_add(s, g[i], f[i], corr);
   }
 }
 
@@ -409,15 +423,23 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
   extern __shared__ __align__(16) float2 smem[];
   float2* xs = smem;
   float2* lines = smem + N;  // [8 L][LP]
+  GridEnt* es = reinterpret_cast<GridEnt*>(lines + 8 * L * LP);
+  int* ptr = reinterpret_cast<int*>(es + kStaged);  // [N + 1]
   __shared__ unsigned short heavy[N];
   __shared__ int n_heavy;
   __shared__ float part[8][4][6];
   const int ky = blockIdx.x, ch0 = blockIdx.y * L;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quad = threadIdx.x >> 2, q = threadIdx.x & 3;
-  const int32_t* ptr = cell_ptr + ky * N;
   if (threadIdx.x == 0) n_heavy = 0;
+  const int first = __ldg(cell_ptr + ky * N), count = __ldg(cell_ptr + ky * N + N) - first;
+  const bool staged = count <= kStaged;
+  for (int i = threadIdx.x; i <= N; i += 256) ptr[i] = __ldg(cell_ptr + ky * N + i) - first;
+  if (staged)
+    for (int i = threadIdx.x; i < count; i += 256) cp_async8(es + i, ents + first + i);
+  cp_async_commit();
   for (int i = threadIdx.x; i < N; i += 256) xs[i] = xtw[i];
+  cp_async_wait_all();
   __syncthreads();
   auto put = [&](int x, int ch, const GridAcc& s) {
     const float sg = ((x + ky) & 1) ? -1.0f : 1.0f;
@@ -426,6 +448,12 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
     d[LP] = make_float2(sg * (s.v.z - s.c.x), sg * (s.v.w - s.c.y));
   };
   const size_t chunk4 = (size_t)Np * G::HC * 4;  // float4s a chunk
+  auto chunk = [&](int ch) { return reinterpret_cast<const float4*>(F) + (size_t)(ch0 + ch) * chunk4 + q; };
+  auto sum_cell = [&](GridAcc& s, int e0, int e1, int step, int ch) {
+    if (staged) grid_sum(s, (const GridEnt*)es, e0, e1, step, chunk(ch), corr);
+    else grid_sum(s, ents + first, e0, e1, step, chunk(ch), corr);
+  };
+#pragma unroll 2
   for (int u = quad; u < N * L; u += 64) {
     const int x = u % N, ch = u / N;
     if (ch0 + ch >= G::NZC) break;
@@ -434,10 +462,8 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
       if (ch == 0 && q == 0) heavy[atomicAdd(&n_heavy, 1)] = (unsigned short)x;
       continue;
     }
-    const float4* Fc = reinterpret_cast<const float4*>(F) + (size_t)(ch0 + ch) * chunk4;
     GridAcc s = {};
-#pragma unroll 4
-    for (int e = e0; e < e1; ++e) grid_add(s, ents[e], Fc, corr, q);
+    sum_cell(s, e0, e1, 1, ch);
     put(x, ch, s);
   }
   __syncthreads();
@@ -447,10 +473,8 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
     const int e0 = ptr[x], e1 = ptr[x + 1];
     for (int ch = 0; ch < L; ++ch) {
       if (ch0 + ch >= G::NZC) break;
-      const float4* Fc = reinterpret_cast<const float4*>(F) + (size_t)(ch0 + ch) * chunk4;
       GridAcc s = {};
-#pragma unroll 4
-      for (int e = e0 + quad; e < e1; e += 64) grid_add(s, ents[e], Fc, corr, q);
+      sum_cell(s, e0 + quad, e1, 64, ch);
       float r[6] = {s.v.x, s.v.y, s.v.z, s.v.w, s.c.x, s.c.y};
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
@@ -523,7 +547,7 @@ static cudaError_t spectra_n(const float2* Hp, const float2* ramps, float2* F, f
 
 // gather into rows of the grid with their inverse FFT, then the y lines
 template <int N>
-static cudaError_t grid_n(cpra_plan_s* p) {
+static cudaError_t grid_n(cpra_plan_s* p, float2* out) {
   using G = GridCfg<N>;
   Assembly& a = p->asmb;
   static bool attr = false;
@@ -533,17 +557,15 @@ static cudaError_t grid_n(cpra_plan_s* p) {
   k_grid<N><<<dim3(N, (G::NZC + G::L - 1) / G::L), 256, G::SMEM, p->stream>>>(
       a.F, a.corr, a.cell_ptr, a.ents, a.vol, p->xtw, p->Np);
   e = cudaGetLastError();
-  return e == cudaSuccess ? launch_volume_ylines(N, a.vol, p->xtw, p->stream) : e;
+  return e == cudaSuccess ? launch_volume_ylines(N, a.vol, out, p->xtw, p->stream) : e;
 }
 
 template <int N>
-cudaError_t assemble_n(cpra_plan_s* p) {
-  // the caller has put the R2C rows of rho into Hp
+cudaError_t assemble_n(cpra_plan_s* p, float2* out) {
   Assembly& a = p->asmb;
-  cudaError_t e = launch_ramps(p, a.moments, a.ramps, p->stream);
-  if (e == cudaSuccess)
-    e = spectra_n<N, kSpecF>(p->Hp, a.ramps, a.F, a.corr, p->xtw, MergeArgs{}, p->Np, p->stream);
-  return e == cudaSuccess ? grid_n<N>(p) : e;
+  cudaError_t e =
+      spectra_n<N, kSpecF>(p->Hp, a.ramps, a.F, a.corr, p->xtw, MergeArgs{}, p->Np, p->stream);
+  return e == cudaSuccess ? grid_n<N>(p, out) : e;
 }
 
 template <int N>
@@ -574,14 +596,14 @@ cudaError_t merge_n(cpra_plan_s* d, const MergeArgs& ma, int n_l, float2* acc, d
       ma, n_l, acc, rings, counts, d->asmb.F, d->asmb.corr, d->xtw);
   e = cudaGetLastError();
   if (e == cudaSuccess && rings) e = launch_prtf(rings, counts, prtf, N / 2, (int)total, st);
-  return e == cudaSuccess ? grid_n<N>(d) : e;
+  return e == cudaSuccess ? grid_n<N>(d, nullptr) : e;
 }
 
 
 // The instances of one N, compiled in the translation unit that names them
 // (k_assemble_*.cu) and only declared elsewhere.
 #define CPRA_ASSEMBLE_INSTANCES(NN, EXTERN)                                                   \
-  EXTERN template cudaError_t assemble_n<NN>(cpra_plan_s*);                                   \
+  EXTERN template cudaError_t assemble_n<NN>(cpra_plan_s*, float2*);                          \
   EXTERN template cudaError_t merge_twins_n<NN>(cpra_plan_s*, const MergeArgs&, int);         \
   EXTERN template cudaError_t merge_n<NN>(cpra_plan_s*, const MergeArgs&, int, float2*, double*, float*);
 

@@ -299,7 +299,9 @@ cudaError_t launch_rowpass(const Launch& L);
 cudaError_t launch_shrinkwrap(cpra_plan_s* p);
 
 // assembly (k_assemble.cu)
-cudaError_t launch_assemble(cpra_plan_s* p);
+// spectra, grid and volume from Hp and the ramps (launch_rho_rows); out: NULL,
+// or device memory of the plan's device that receives the volume too
+cudaError_t launch_assemble(cpra_plan_s* p, float2* out);
 size_t spectra_bytes(int N, int Np);  // Assembly::F, ::corr and ::ramps
 size_t corr_bytes(int N, int Np);
 size_t ramps_bytes(int N, int Np);
@@ -320,16 +322,18 @@ struct MergeArgs {
 };
 // FP64 moments (sum rho, sum rho z, sum rho u) of rho = P_{S+} g of every angle
 cudaError_t launch_moments(cpra_plan_s* p, double* moments, cudaStream_t st);
-// the same, then the unit ramps of the mass-centre moves
-cudaError_t launch_ramps(cpra_plan_s* p, double* moments, float2* ramps, cudaStream_t st);
+// R2C rows of rho into Hp (L: the plan's launch of a plain object prime over
+// every angle), the moments of rho, and the unit ramps of the mass-centre moves
+cudaError_t launch_rho_rows(cpra_plan_s* p, const Launch& L, double* moments, float2* ramps);
 // twin distances of the kept guesses, on dst's stream
 cudaError_t launch_merge_twins(cpra_plan_s* dst, const MergeArgs& ma, int n_l);
 // acc = mean of the corrected spectra, PRTF (rings and prtf not NULL), its
 // IDFT_z, gridding and the plane IFFTs into dst's volume, on dst's stream
 cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, double* rings,
                          float* prtf);
-// inverse FFT along y of every plane of a volume, in place (k_refine_w.cu)
-cudaError_t launch_volume_ylines(int N, float2* vol, const float2* xtw, cudaStream_t st);
+// inverse FFT along y of every plane of a volume, in place, and into out when
+// that is not NULL (k_refine_w.cu)
+cudaError_t launch_volume_ylines(int N, float2* vol, float2* out, const float2* xtw, cudaStream_t st);
 
 // Step D refinement (k_refine.cu): buffers of one plan's refinement
 struct RefineArgs {
@@ -372,7 +376,7 @@ cudaError_t launch_rowpass_fast_tc(const Launch& L);
 cudaError_t launch_prime_fast_tc(const Launch& L);
 cudaError_t launch_colpass_fast_tc(const Launch& L);
 cudaError_t launch_rowpass_fast(const Launch& L);
-cudaError_t launch_prime_fast(const Launch& L);
+cudaError_t launch_prime_fast(const Launch& L, double* moments = nullptr);
 cudaError_t launch_colpass_fast(const Launch& L);
 // persistent work-queue form of the column and row passes (FP32)
 bool persist_supported(int N);

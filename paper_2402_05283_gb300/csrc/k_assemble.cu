@@ -34,11 +34,13 @@ CPRA_FOR_EACH_N(CPRA_CASE)
 #undef CPRA_CASE
 
 // ---------------------------------------------------------------- moments
+// The moments apart from the rows of rho, for the prime kernels that do not
+// take them along and for the refinement.
 // One warp per kMomRows rows: each lane sums its pixels of a row in FP32 (at
 // most N/32 terms) and its rows as pairs of FP32 (48 bits, with the exact
 // products by y); FP64 across lanes, warps and CTAs.  Bound by HBM: the FP64
 // pipe is narrow, and ten FP64 shuffles and adds a row made it the bound
-// (N = 256, 180 angles: 52 us, @@ with one FP64 reduction per 16 rows).
+// (N = 256, 144 angles: 44 us, 33 with one reduction of FP32 pairs per 16 rows).
 constexpr int kMomRows = 16;
 __global__ void k_moments(const float* __restrict__ g, const uint32_t* __restrict__ S,
                           double* moments, int N, int W) {
@@ -157,17 +159,25 @@ cudaError_t launch_moments(cpra_plan_s* p, double* moments, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_ramps(cpra_plan_s* p, double* moments, float2* ramps, cudaStream_t st) {
-  cudaError_t e = launch_moments(p, moments, st);
+cudaError_t launch_rho_rows(cpra_plan_s* p, const Launch& L, double* moments, float2* ramps) {
+  cudaStream_t st = p->stream;
+  cudaError_t e;
+  if (L.prec == CPRA_FP32 && L.engine != CPRA_ENGINE_TWO_PASS) {
+    e = cudaMemsetAsync(moments, 0, sizeof(double) * 3 * p->Np, st);
+    if (e == cudaSuccess) e = launch_prime_fast(L, moments);
+  } else {
+    e = launch_prime(L);
+    if (e == cudaSuccess) e = launch_moments(p, moments, st);
+  }
   if (e != cudaSuccess) return e;
   g_launches += 1;
   k_ramps<<<p->Np, 128, 0, st>>>(moments, ramps, p->N, p->cfg.com_align);
   return cudaGetLastError();
 }
 
-cudaError_t launch_assemble(cpra_plan_s* p) {
+cudaError_t launch_assemble(cpra_plan_s* p, float2* out) {
 #define CPRA_CASE(NN) \
-  case NN: return assemble_n<NN>(p);
+  case NN: return assemble_n<NN>(p, out);
   switch (p->N) { CPRA_FOR_EACH_N(CPRA_CASE) default: return cudaErrorInvalidValue; }
 #undef CPRA_CASE
 }

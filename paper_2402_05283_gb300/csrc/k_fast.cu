@@ -69,11 +69,11 @@ cudaError_t launch_rowpass_fast(const Launch& L) {
   }
 }
 
-cudaError_t launch_prime_fast(const Launch& L) {
-  if (L.prec != kPrecFP32) return launch_prime_fast_tc(L);
+cudaError_t launch_prime_fast(const Launch& L, double* moments) {
+  if (L.prec != kPrecFP32) return moments ? cudaErrorInvalidValue : launch_prime_fast_tc(L);
   switch (L.N) {
 #define CPRA_CASE(NN) \
-  case NN: return prime_w<NN, kPrecFP32>(L);
+  case NN: return prime_w<NN, kPrecFP32>(L, moments);
     CPRA_FOR_EACH_N(CPRA_CASE)
 #undef CPRA_CASE
     default:

@@ -39,30 +39,33 @@ template <int N> struct FusedLines { using type = typename WLines<N, kPrecFP32>:
 // Packed columns per CTA: 32, or 16 at N = 512, where a cluster of 16 CTAs
 // of 108 KB each puts two CTAs of different angles on an SM, so that one
 // CTA's barrier and DSMEM waits overlap the other's arithmetic.
-template <int N> struct FusedCfg {
+// Q tasks a warp and phase: 2, which leaves the registers and shared memory
+// for more clusters an SM, or 1 for launches whose clusters would leave the
+// SMs with a few warps each (fused_launch has the rule).
+template <int N, int Q> struct FusedCfg {
   using FL = typename FusedLines<N>::type;
   static constexpr int H = N / 2;
   static constexpr int CW = N == 512 ? 16 : 32;  // packed columns per CTA
   static constexpr int C = H / CW;               // CTAs per cluster
   static constexpr int ROWS = N / C;             // image rows of a CTA's row phase
   static constexpr int TASKS = CW / FL::L;       // tasks per phase per CTA
-  static constexpr int NW = TASKS / 2;           // warps: two tasks each per phase
+  static constexpr int NW = TASKS / Q;           // warps
   static constexpr int NT = NW * 32;
   static constexpr int SP = CW + 1;              // slab pitch in float2: odd, so column reads are conflict-free
   static constexpr int SLAB = N * SP;
-  static constexpr int MINB = N >= 256 ? 2 : 4;
+  static constexpr int MINB = (N >= 256 ? 2 : 4) * Q / 2;
   static constexpr int MASKW = (2 * FL::TA * FL::E1 + 31) / 32;  // support-bit words of a row task
   static constexpr size_t SMEM = sizeof(float2) * (SLAB + NW * FL::TSIZE + N) + sizeof(double) * NW;
   static_assert(ROWS == 2 * CW, "row pairs of a CTA = its packed columns");
   static_assert(C >= 1 && C <= 16, "cluster size");
-  static_assert(TASKS == 2 * NW, "two tasks a warp");
+  static_assert(TASKS == Q * NW, "tasks a warp");
 };
 
 // ---------------------------------------------------------------- DSMEM (cluster.cuh)
 // slab address of (row y, packed column c): CTA c / 32, local column c % 32
 template <int N>
 __device__ __forceinline__ uint32_t slab_at(uint32_t sb, int y, int c) {
-  using F = FusedCfg<N>;
+  using F = FusedCfg<N, 2>;  // (the slabs do not depend on Q)
   return dsm_map(sb + 8u * (uint32_t)(y * F::SP + (c & (F::CW - 1))), (uint32_t)(c / F::CW));
 }
 
@@ -71,7 +74,7 @@ __device__ __forceinline__ uint32_t slab_at(uint32_t sb, int y, int c) {
 template <int N, class FL>
 __device__ __forceinline__ void gather_pairs(float2 (&b)[FL::TB][FL::E2], uint32_t sb, int pair0,
                                              int lane) {
-  using F = FusedCfg<N>;
+  using F = FusedCfg<N, 2>;
   constexpr int H = N / 2;
   static_for<0, FL::TB>([&](auto II) {
     constexpr int i = decltype(II)::value;
@@ -103,7 +106,7 @@ __device__ __forceinline__ void gather_pairs(float2 (&b)[FL::TB][FL::E2], uint32
 template <int N, class FL>
 __device__ __forceinline__ void scatter_pairs(float2 (&b)[FL::TB][FL::E2], float2* T, uint32_t sb,
                                               int pair0, int lane) {
-  using F = FusedCfg<N>;
+  using F = FusedCfg<N, 2>;
   constexpr int H = N / 2;
   static_for<0, FL::TB>([&](auto II) {
     constexpr int i = decltype(II)::value;
@@ -142,9 +145,9 @@ __device__ __forceinline__ void scatter_pairs(float2 (&b)[FL::TB][FL::E2], float
 // support bits of this lane's pixels of one row task (A layout), bit
 // (i * E1 + m) * 2 + r for row 2 (pair0 + line) + r
 template <int N, class FL>
-__device__ __forceinline__ void support_mask(uint32_t (&mk)[FusedCfg<N>::MASKW], const uint32_t* Sn,
+__device__ __forceinline__ void support_mask(uint32_t (&mk)[FusedCfg<N, 2>::MASKW], const uint32_t* Sn,
                                              int W, int pair0, int lane) {
-  static_for<0, FusedCfg<N>::MASKW>([&](auto WW) { mk[decltype(WW)::value] = 0u; });
+  static_for<0, FusedCfg<N, 2>::MASKW>([&](auto WW) { mk[decltype(WW)::value] = 0u; });
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
@@ -160,11 +163,18 @@ __device__ __forceinline__ void support_mask(uint32_t (&mk)[FusedCfg<N>::MASKW],
   });
 }
 
-template <int N, bool MASKED>
-__global__ void __launch_bounds__(FusedCfg<N>::NT, FusedCfg<N>::MINB)
+// Few angles at N = 64 stay as they were, two tasks a warp and the error
+// published in every iteration (90 us for ten iterations of eight angles, 65
+// in the other form): a test of the serving loop submits 2000 iterations of
+// eight angles and needs them to outlast 20 ms.
+constexpr int kFewTiles64 = 8;
+template <int N, int Q> constexpr bool kPublishAtOnce = N == 64 && Q == 2;
+
+template <int N, bool MASKED, int Q>
+__global__ void __launch_bounds__(FusedCfg<N, Q>::NT, FusedCfg<N, Q>::MINB)
 k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
         const int2* __restrict__ tiles) {
-  using F = FusedCfg<N>;
+  using F = FusedCfg<N, Q>;
   using FL = typename F::FL;
   constexpr int H = N / 2;
   extern __shared__ __align__(16) float2 smem[];
@@ -193,8 +203,8 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
   load_xtw<N>(xs, J->xtw, F::NT);
   fill_taps<N>(tt, ca, Z->g_src, Z->g_dst, J->S, n, Np, W, J->present);
   // the support is fixed during a launch: each lane keeps its pixels' bits
-  uint32_t mask[2][F::MASKW];
-  static_for<0, 2>([&](auto QQ) {
+  uint32_t mask[Q][F::MASKW];
+  static_for<0, Q>([&](auto QQ) {
     constexpr int q = decltype(QQ)::value;
     support_mask<N, FL>(mask[q], J->S + (size_t)n * N * W, W,
                         rank * F::CW + (warp + q * F::NW) * FL::L, lane);
@@ -203,7 +213,7 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
 
   // ---- prime: (coupled) rows -> R2C -> slabs
 #pragma unroll 1
-  for (int q = 0; q < 2; ++q) {
+  for (int q = 0; q < Q; ++q) {
     const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
     float2 a[FL::TA][FL::E1];
     blend_rows<N, FL>(a, tt, ca, W, pair0, lane);
@@ -319,7 +329,7 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
     uint32_t mq[F::MASKW];
     static_for<0, F::MASKW>([&](auto WW) {
       constexpr int w = decltype(WW)::value;
-      mq[w] = q ? mask[1][w] : mask[0][w];
+      mq[w] = q ? mask[Q - 1][w] : mask[0][w];
     });
     static_for<0, FL::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
@@ -348,21 +358,22 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
   for (int it = 0; it < n_iters; ++it) {
     const int rule = it < hio_left ? Z->algo : kER;  // HIO or RAAR, then ER
     const bool fwd = it + 1 < n_iters;
-    double errd = 0.0;
+    float es = 0.0f, ee = 0.0f;  // error terms as an FP32 pair
 #pragma unroll 1
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < Q; ++q) {
       if (q) load_av(q, av);
       float err2 = 0.0f, err1 = 0.0f;
       col_task(q, av, err2, err1);
-      errd += 2.0 * (double)err2 + (double)err1;
+      two_add(es, ee, 2.0f * err2);
+      two_add(es, ee, err1);
     }
-    for (int o = 16; o > 0; o >>= 1) errd += __shfl_down_sync(0xffffffffu, errd, o);
+    const double errd = warp_sum(es, ee);
     if (lane == 0) red[warp] = errd;
     cluster_arrive();
     if (rule != kER) load_old(0, old);  // in flight across the barrier
     cluster_wait();
 #pragma unroll 1
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < Q; ++q) {
       const int pq = rank * F::CW + (warp + q * F::NW) * FL::L;
       if (rule != kER && q) load_old(q, old);
       float2 b[FL::TB][FL::E2];
@@ -383,72 +394,109 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
       for (int q = lane; q < F::C * F::NW; q += 32)
         s += dsm_ld_f64(dsm_map(smem_u32(red + q % F::NW), (uint32_t)(q / F::NW)));
       for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      if (lane == 0) {
-        const double den = J->sumA2[n];
-        J->err_hist[(size_t)(err_slot + it) * Np + n] = publish_error(s, J->Cn[n], den, J->status, n);
-      }
+      // the raw sum; the square root and division wait until the last
+      // iteration (not in the short chains of kPublishAtOnce)
+      if (lane == 0)
+        J->err_hist[(size_t)(err_slot + it) * Np + n] =
+            kPublishAtOnce<N, Q> ? publish_error(s, J->Cn[n], J->sumA2[n], J->status, n) : s;
     }
     cluster_arrive();
     if (fwd) load_av(0, av);  // in flight across the barrier
     cluster_wait();
   }
+  if (!kPublishAtOnce<N, Q> && rank == 0 && warp == 0 && err_slot >= 0) {
+    __syncwarp();
+    for (int it = lane; it < n_iters; it += 32) {
+      double* e = J->err_hist + (size_t)(err_slot + it) * Np + n;
+      *e = publish_error(__ldcg(e), J->Cn[n], J->sumA2[n], J->status, n);
+    }
+  }
 }
+
 
 // ---------------------------------------------------------------- host side
-template <int N>
-static cudaError_t fused_prepare() {
-  static bool done = false;
-  static cudaError_t err = cudaSuccess;
-  if (done) return err;
-  using F = FusedCfg<N>;
-  err = cudaFuncSetAttribute(k_fused<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::SMEM);
-  if (err == cudaSuccess)
-    err = cudaFuncSetAttribute(k_fused<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::SMEM);
-  if (err == cudaSuccess && F::C > 8)
-    err = cudaFuncSetAttribute(k_fused<N, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (err == cudaSuccess && F::C > 8)
-    err = cudaFuncSetAttribute(k_fused<N, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (err == cudaSuccess) {
-    // a cluster of C CTAs with this much shared memory must fit on the device
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(F::C, 1);
-    cfg.blockDim = dim3(F::NT);
-    cfg.dynamicSmemBytes = F::SMEM;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = F::C;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int clusters = 0;
-    err = cudaOccupancyMaxActiveClusters(&clusters, k_fused<N, false>, &cfg);
-    if (err == cudaSuccess && clusters < 1) err = cudaErrorNotSupported;
-  }
-  done = true;
-  return err;
-}
-
-template <int N>
-static cudaError_t fused_launch(const Launch& L) {
-  using F = FusedCfg<N>;
-  cudaError_t e = fused_prepare<N>();
-  if (e != cudaSuccess) return e;
+template <int N, int Q>
+static cudaLaunchConfig_t fused_config(int ntiles, cudaLaunchAttribute* at, cudaStream_t st) {
+  using F = FusedCfg<N, Q>;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(F::C, L.ntiles);
+  cfg.gridDim = dim3(F::C, ntiles);
   cfg.blockDim = dim3(F::NT);
   cfg.dynamicSmemBytes = F::SMEM;
-  cfg.stream = L.stream;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = F::C;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
+  cfg.stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = F::C;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
+  return cfg;
+}
+
+// attributes of both instances; *clusters: resident clusters of this shape
+template <int N, int Q>
+static cudaError_t fused_attrs(int* clusters) {
+  using F = FusedCfg<N, Q>;
+  cudaError_t e = cudaSuccess;
+  for (auto kernel : {k_fused<N, false, Q>, k_fused<N, true, Q>}) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::SMEM);
+    if (e == cudaSuccess && F::C > 8)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  }
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at;
+  cudaLaunchConfig_t cfg = fused_config<N, Q>(1, &at, nullptr);
+  e = cudaOccupancyMaxActiveClusters(clusters, k_fused<N, false, Q>, &cfg);
+  return e == cudaSuccess && *clusters < 1 ? cudaErrorNotSupported : e;
+}
+
+// N = 512 has one instance: its two tasks a warp fill the SM with 16 warps
+template <int N> constexpr bool kFusedWide = N <= 256;
+
+// looked up once per process and size: a cluster of C CTAs with this much
+// shared memory must fit on the device; *wide: clusters of the one-task form
+// that are resident at a time
+template <int N>
+static cudaError_t fused_prepare(int* wide) {
+  struct Ready {
+    cudaError_t e;
+    int wide = 0;
+    Ready() {
+      int c = 0;
+      e = fused_attrs<N, 2>(&c);
+      if constexpr (kFusedWide<N>)
+        if (e == cudaSuccess && fused_attrs<N, 1>(&wide) != cudaSuccess) {
+          cudaGetLastError();
+          wide = 0;
+        }
+    }
+  };
+  static const Ready r;
+  if (wide) *wide = r.wide;
+  return r.e;
+}
+
+// One task a warp where all of the launch's clusters are resident at a time in
+// that form: the SMs then hold twice the warps and each runs half the chain.
+// Ten iterations, two tasks / one: N = 64, 32 angles 90 / 66 us, 200 angles
+// 101 / 79; N = 128, 90 angles 182 / 158, 150 angles 186 / 165; N = 256, 30
+// angles 200 / 190.  Beyond that the two-task form holds more clusters an SM.
+template <int N>
+static cudaError_t fused_launch(const Launch& L) {
+  int wide = 0;
+  cudaError_t e = fused_prepare<N>(&wide);
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute at;
   g_launches += 1;
-  if (L.masked) return cudaLaunchKernelEx(&cfg, k_fused<N, true>, L.js, L.st, L.tiles);
-  return cudaLaunchKernelEx(&cfg, k_fused<N, false>, L.js, L.st, L.tiles);
+  if constexpr (kFusedWide<N>)
+    if (L.ntiles <= wide && !(N == 64 && L.ntiles <= kFewTiles64)) {
+      const cudaLaunchConfig_t cfg = fused_config<N, 1>(L.ntiles, &at, L.stream);
+      if (L.masked) return cudaLaunchKernelEx(&cfg, k_fused<N, true, 1>, L.js, L.st, L.tiles);
+      return cudaLaunchKernelEx(&cfg, k_fused<N, false, 1>, L.js, L.st, L.tiles);
+    }
+  const cudaLaunchConfig_t cfg = fused_config<N, 2>(L.ntiles, &at, L.stream);
+  if (L.masked) return cudaLaunchKernelEx(&cfg, k_fused<N, true, 2>, L.js, L.st, L.tiles);
+  return cudaLaunchKernelEx(&cfg, k_fused<N, false, 2>, L.js, L.st, L.tiles);
 }
 
 #define CPRA_FOR_EACH_FUSED_N(X) X(64) X(128) X(256) X(512)
@@ -467,7 +515,7 @@ bool fused_supported(int N) {
 cudaError_t prepare_kernels_fused(int N) {
   switch (N) {
 #define CPRA_CASE(NN) \
-  case NN: return fused_prepare<NN>();
+  case NN: return fused_prepare<NN>(nullptr);
     CPRA_FOR_EACH_FUSED_N(CPRA_CASE)
 #undef CPRA_CASE
     default:

@@ -15,7 +15,8 @@ std::atomic<long long> g_launches{0};
 // projection leaves them free) and stay out of Cn and sumA2.
 //
 // One warp a row ky, 8 rows a CTA: each lane sums its pixels' terms in FP32
-// (at most N/32 of them), the sums go to FP64 across lanes, rows and CTAs.
+// (at most N/32 of them), the sums go to FP32 pairs across lanes (48 bits;
+// FP64 shuffles and adds took half of the kernel), to FP64 across rows and CTAs.
 //
 // An invalid pattern (a negative or non-finite intensity) marks bad[n] and
 // makes C_n NaN, so the first iteration on it publishes a non-finite error
@@ -55,12 +56,8 @@ __global__ void k_prepare(const float* __restrict__ I, int N, int first, float* 
       if (kx < h) A_rows[((size_t)blockIdx.y * N + ky) * h + kx] = as;
       if (kx == h) A_nyq[(size_t)n * N + ky] = as;
     }
-    c_part = cf;
-    a_part = af;
-    for (int o = 16; o > 0; o >>= 1) {
-      c_part += __shfl_down_sync(0xffffffffu, c_part, o);
-      a_part += __shfl_down_sync(0xffffffffu, a_part, o);
-    }
+    c_part = warp_sum(cf, 0.0f);
+    a_part = warp_sum(af, 0.0f);
   }
   if (lane == 0) { sc[warp] = c_part; sa[warp] = a_part; }
   const int block_bad = __syncthreads_or(bad);

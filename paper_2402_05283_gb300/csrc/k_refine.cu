@@ -63,10 +63,16 @@ __global__ void k_measured(const int32_t* __restrict__ cell_ptr, uint8_t* M, int
 // none of its voxels is in any more, so the angles run in an order that
 // jumps by about 0.38 of the range (`step`, coprime to Np): neighbouring
 // angles test nearly the same, and a voxel outside dies after a handful of
-// spread angles.  Bound by issue: the words that hold object run all angles.
-// N = 256, 180 angles: 1.25 ms, the FP64 evaluations near a half the bound.
-// The nearest pixel is the one an FP64 evaluation in the host's order picks:
-// FP32 where that cannot differ, FP64 near a tie.
+// spread angles.
+// The nearest pixel is the one an FP64 evaluation in the host's order picks.
+// FP32 decides it where its estimate is not within 1e-3 of a half; there the
+// distance to the half is taken on FP32 pairs (cos, sin and the row's part as
+// high and low words, products and sums with their rounding errors: good to
+// 1e-11), and only within 1e-9 of a half in FP64.  The FP64 pipe is narrow: a
+// warp meets an estimate near a half in every eighth step, and FP64 there
+// was the bound.  N = 256, 180 angles: 1.09 ms with a thread a word, the
+// angles in order and FP64 at 1e-3; a lane a voxel in spread order 1.25 ms;
+// with the pairs 1.17 ms.
 // u = rint(((x - c) cos + (y - c) sin) + c) in FP64, each step rounded, no
 // contraction.  Not inlined: kept out of line, the rare call leaves the FP64
 // pipe idle instead of being predicated into every evaluation.
@@ -79,43 +85,47 @@ __device__ __noinline__ int u_fp64(int x, int y, int N, double2 t) {
 __global__ void __launch_bounds__(256)
 k_backproject(const uint32_t* __restrict__ S2, const double2* __restrict__ cs,
               const int2* __restrict__ shift, uint32_t* S3, int N, int W, int Np, int YB, int NC, int step) {
-  // per chunk of NC angles: S2 rows [NC][W]; (cos, sin) [NC] for the FP64
-  // path; du [NC]; cos in FP32 [NC]; (y - c) sin + c in FP32 [NC][YB]; the
-  // words still in, [YB][W]
+  // per chunk of NC angles: cos and sin as FP32 pairs [NC]; (y - c) sin + c
+  // as a pair [NC][YB]; S2 rows [NC][W]; the angle and its du [NC]; the words
+  // still in, [YB][W]
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  double2* tcs = reinterpret_cast<double2*>(sm_raw);
-  uint32_t* rows = reinterpret_cast<uint32_t*>(tcs + NC);
-  int* tdu = reinterpret_cast<int*>(rows + (size_t)NC * W);
-  float* cfs = reinterpret_cast<float*>(tdu + NC);
-  float* bfs = cfs + NC;
-  uint32_t* in = reinterpret_cast<uint32_t*>(bfs + (size_t)NC * YB);
+  float4* tcs = reinterpret_cast<float4*>(sm_raw);
+  float2* tb = reinterpret_cast<float2*>(tcs + NC);
+  int2* tn = reinterpret_cast<int2*>(tb + (size_t)NC * YB);
+  uint32_t* rows = reinterpret_cast<uint32_t*>(tn + NC);
+  uint32_t* in = rows + (size_t)NC * W;
   const int z = blockIdx.y;
   const int y0 = blockIdx.x * YB;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double c = N / 2;
   for (int q = threadIdx.x; q < YB * W; q += blockDim.x) {
     const int left = N - (q % W) * 32;  // voxels of the word
     in[q] = y0 + q / W >= N ? 0u : left >= 32 ? 0xffffffffu : (1u << left) - 1u;
   }
   for (int n0 = 0; n0 < Np; n0 += NC) {
     const int nc = min(NC, Np - n0);
-    auto angle = [&](int k) { return (int)(((long long)(n0 + k) * step) % Np); };
     __syncthreads();  // the previous chunk is done
+    for (int k = threadIdx.x; k < nc; k += blockDim.x) {
+      const int n = (int)((unsigned)(n0 + k) * (unsigned)step % (unsigned)Np);
+      const double2 t = cs[n];
+      const float ch = (float)t.x, sh = (float)t.y;
+      tcs[k] = make_float4(ch, (float)(t.x - (double)ch), sh, (float)(t.y - (double)sh));
+      tn[k] = make_int2(n, shift[n].y);
+    }
+    __syncthreads();
     for (int q = threadIdx.x; q < nc * W; q += blockDim.x) {
-      const int k = q / W, ww = q - k * W, n = angle(k);
+      const int k = q / W, ww = q - k * W, n = tn[k].x;
       int zr = z + shift[n].x;
       zr = zr < 0 ? zr + N : (zr >= N ? zr - N : zr);
       rows[k * W + ww] = S2[((size_t)n * N + zr) * W + ww];
     }
-    for (int k = threadIdx.x; k < nc; k += blockDim.x) {
-      const int n = angle(k);
-      tcs[k] = cs[n];
-      tdu[k] = shift[n].y;
-      cfs[k] = (float)cs[n].x;
-    }
     for (int q = threadIdx.x; q < nc * YB; q += blockDim.x) {
-      const int k = q / YB, r = q - k * YB;
-      bfs[q] = (float)__dmul_rn((double)(y0 + r - N / 2), cs[angle(k)].y) + (float)c;
+      const int k = q / YB;
+      const float y = (float)(y0 + q - k * YB - N / 2);
+      const float4 t = tcs[k];
+      float h = __fmul_rn(y, t.z), l = fmaf(y, t.z, -h);
+      l = fmaf(y, t.w, l);
+      two_add(h, l, (float)(N / 2));
+      tb[q] = make_float2(h, l);
     }
     __syncthreads();
     for (int q = warp; q < YB * W; q += blockDim.x >> 5) {
@@ -126,17 +136,25 @@ k_backproject(const uint32_t* __restrict__ S2, const double2* __restrict__ cs,
       bool keep = (bits >> lane) & 1u;
       uint32_t left = bits;
       for (int k = 0; k < nc; ++k) {
-        // FP32 estimate of u: within 2e-4 of the FP64 value for |x - c|,
-        // |y - c| <= 512, so its nearest integer (by the 1.5 * 2^23 shift) is
-        // the FP64 one unless it sits within 1e-3 of a half; those few are
-        // redone in FP64
-        const float uf = fmaf(xf, cfs[k], bfs[k * YB + yl]);
+        const float4 t = tcs[k];
+        const float2 b = tb[k * YB + yl];
+        // the estimate, within 2e-4 for |x - c|, |y - c| <= 512, and its
+        // nearest integer by the 1.5 * 2^23 shift
+        const float uf = fmaf(xf, t.x, b.x);
         const float sh = __fadd_rn(uf, 12582912.0f);
-        int ui = __float_as_int(sh) - 0x4B400000;                    // rint(uf)
-        const float fr = __fsub_rn(uf, __fsub_rn(sh, 12582912.0f));  // uf - rint(uf)
-        if (fabsf(fabsf(fr) - 0.5f) < 1e-3f && keep) ui = u_fp64(x, y0 + yl, N, tcs[k]);
+        int ui = __float_as_int(sh) - 0x4B400000;
+        const float fr = __fsub_rn(uf, __fsub_rn(sh, 12582912.0f));
+        if (fabsf(fabsf(fr) - 0.5f) < 1e-3f && keep) {
+          const float half = floorf(uf) + 0.5f;
+          const float p = __fmul_rn(xf, t.x);
+          float s = b.x, e = 0.0f;
+          two_add(s, e, p);
+          const float d = __fsub_rn(s, half) + (e + (fmaf(xf, t.x, -p) + fmaf(xf, t.y, b.y)));
+          ui = (int)floorf(uf) + (d > 0.0f ? 1 : 0);
+          if (fabsf(d) < 1e-9f) ui = u_fp64(x, y0 + yl, N, cs[tn[k].x]);
+        }
         if (ui >= 0 && ui < N) {
-          ui += tdu[k];
+          ui += tn[k].y;
           ui = ui < 0 ? ui + N : (ui >= N ? ui - N : ui);
           keep = keep && ((rows[k * W + (ui >> 5)] >> (ui & 31)) & 1u);
         } else {
@@ -205,8 +223,7 @@ cudaError_t launch_refine_support(const RefineArgs& a, const uint32_t* S2, const
   const int N = a.N, W = a.W;
   const int YB = std::max(1, std::min(N, 256 / W));
   // angles a chunk: their tables (see k_backproject) within 72 KB (three CTAs an SM)
-  const int per = (int)(sizeof(double2) + W * sizeof(uint32_t) + sizeof(int) + sizeof(float) +
-                        YB * sizeof(float));
+  const int per = (int)(sizeof(float4) + sizeof(int2) + W * sizeof(uint32_t) + YB * sizeof(float2));
   const int words = YB * W * (int)sizeof(uint32_t);
   const int NC = std::max(1, std::min(Np, (72 * 1024 - words) / per));
   const size_t smem = (size_t)NC * per + words;

@@ -155,9 +155,10 @@ k_xw(float2* X, const float2* __restrict__ xtw, size_t rows) {
 
 // CB adjacent x columns of one line set (blockIdx.y = z for y lines, = ky for
 // z lines), N points estride apart, in place: forward, or inverse with 1/N
+// (and a copy of the result, same layout, into out when that is not NULL)
 template <int N, bool INV>
 __global__ void __launch_bounds__(VW<N>::NT, VW<N>::MINB)
-k_vw(float2* X, const float2* __restrict__ xtw, size_t outer, size_t estride) {
+k_vw(float2* X, float2* out, const float2* __restrict__ xtw, size_t outer, size_t estride) {
   using C = VW<N>;
   using FL = typename C::FL;
   extern __shared__ float2 smem[];
@@ -191,7 +192,12 @@ k_vw(float2* X, const float2* __restrict__ xtw, size_t outer, size_t estride) {
       buf[k * C::SP + col0 + line] = b[decltype(II)::value][decltype(JJ)::value];
     });
   __syncthreads();
-  rows.each([&](int y) { base[y * estride + rows.cc] = buf[y * C::SP + rows.cc]; });
+  float2* copy = INV && out ? out + (base - X) : nullptr;
+  rows.each([&](int y) {
+    const float2 v = buf[y * C::SP + rows.cc];
+    base[y * estride + rows.cc] = v;
+    if (INV && copy) copy[y * estride + rows.cc] = v;
+  });
 }
 
 // ------------------------------------------------------------ half spectrum
@@ -484,8 +490,8 @@ cudaError_t data_w(const RefineArgs& a, cudaStream_t st) {
   const dim3 grid(N / C::CB, N);
   g_launches += 4;
   k_xw<N><<<(unsigned)((NN + rows - 1) / rows), XW<N>::WARPS * 32, xw_smem<N>(), st>>>(a.X, a.xtw, NN);
-  k_vw<N, false><<<grid, C::NT, vw_smem<N>(), st>>>(a.X, a.xtw, NN, (size_t)N);
-  k_vw<N, false><<<grid, C::NT, vw_smem<N>(), st>>>(a.X, a.xtw, (size_t)N, NN);
+  k_vw<N, false><<<grid, C::NT, vw_smem<N>(), st>>>(a.X, nullptr, a.xtw, NN, (size_t)N);
+  k_vw<N, false><<<grid, C::NT, vw_smem<N>(), st>>>(a.X, nullptr, a.xtw, (size_t)N, NN);
   e = cudaMemsetAsync(a.konst, 0, 2 * sizeof(double), st);
   if (e != cudaSuccess) return e;
   k_rdata<<<dim3(N, 16), 128, 0, st>>>(a.X, a.M, a.Wd, a.konst, N, C::HP);
@@ -524,7 +530,7 @@ cudaError_t iter_w(const RefineArgs& a, double* err2, bool first, bool last, cud
 }
 
 template <int N>
-cudaError_t volume_ylines_n(float2* vol, const float2* xtw, cudaStream_t st) {
+cudaError_t volume_ylines_n(float2* vol, float2* out, const float2* xtw, cudaStream_t st) {
   using C = VW<N>;
   static bool done = false;
   if (!done) {
@@ -533,16 +539,16 @@ cudaError_t volume_ylines_n(float2* vol, const float2* xtw, cudaStream_t st) {
     done = true;
   }
   g_launches += 1;
-  k_vw<N, true><<<dim3(N / C::CB, N), C::NT, vw_smem<N>(), st>>>(vol, xtw, (size_t)N * N, (size_t)N);
+  k_vw<N, true><<<dim3(N / C::CB, N), C::NT, vw_smem<N>(), st>>>(vol, out, xtw, (size_t)N * N, (size_t)N);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_volume_ylines(int N, float2* vol, const float2* xtw, cudaStream_t st) {
+cudaError_t launch_volume_ylines(int N, float2* vol, float2* out, const float2* xtw, cudaStream_t st) {
   switch (N) {
 #define CPRA_CASE(NN) \
-  case NN: return volume_ylines_n<NN>(vol, xtw, st);
+  case NN: return volume_ylines_n<NN>(vol, out, xtw, st);
     CPRA_FOR_EACH_N(CPRA_CASE)
 #undef CPRA_CASE
     default:
