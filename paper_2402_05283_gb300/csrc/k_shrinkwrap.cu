@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, co
   const int rows = kTileY + ntaps - 1, cols = kTileX + ntaps - 1;
   const int off = -lo - (ntaps - 1);  // staged element k is pixel x0 + k + off (mod N)
   if (threadIdx.x < ntaps) tp[threadIdx.x] = taps.v[threadIdx.x];
+#pragma unroll 4
   for (int r = warp; r < rows; r += 8) {
     int y = y0 + r + off;
     y = y < 0 ? y + N : (y >= N ? y - N : y);
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, co
       w[i] = h[i];
       acc[i] = 0.0f;
     }
+#pragma unroll 8
     for (int t = 0; t < ntaps; ++t) {
       const float c = tp[t];
 #pragma unroll
@@ -276,6 +278,7 @@ __global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, co
       w[i] = h[i * kTilePB];
       acc[i] = 0.0f;
     }
+#pragma unroll 8
     for (int t = 0; t < ntaps; ++t) {
       const float c = tp[t];
 #pragma unroll
