@@ -1125,11 +1125,12 @@ static cpra_status ensure_assembly(cpra_plan_s* p) {
   if (!a.F) {
     a.F = (float2*)dev_alloc(p, spectra_bytes(p->N, p->Np));
     a.corr = (float2*)dev_alloc(p, corr_bytes(p->N, p->Np));
+    a.Q = (float2*)dev_alloc(p, NN * 8);
     a.ramps = (float2*)dev_alloc(p, ramps_bytes(p->N, p->Np));
     a.vol = (float2*)dev_alloc(p, N * NN * 8);
     a.cell_ptr = (int32_t*)dev_alloc(p, (NN + 1) * 4);
     a.moments = (double*)dev_alloc(p, 3 * Np * 8);
-    if (!a.F || !a.corr || !a.ramps || !a.vol || !a.cell_ptr || !a.moments)
+    if (!a.F || !a.corr || !a.Q || !a.ramps || !a.vol || !a.cell_ptr || !a.moments)
       return fail(p, CPRA_ERR_OUT_OF_MEMORY, "assembly allocation failed");
   }
   if (!a.grid_ok) return build_gridding(p);

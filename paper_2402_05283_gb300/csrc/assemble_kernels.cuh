@@ -11,6 +11,8 @@ namespace cpra {
 // along u, the last one for ku = -N/2
 __host__ __device__ constexpr int ramp_len(int N) { return N + N / 2 + 1; }
 
+// Q = sum over a cell's samples of ku < 0 of weight * corr
+cudaError_t launch_grid_corr(cpra_plan_s* p);
 cudaError_t launch_prtf(const double* rings, const unsigned* counts, float* prtf, int H, int total,
                         cudaStream_t st);
 
@@ -361,7 +363,7 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
 // kHeavy is summed by the whole block, its samples spread over the 64 quads
 // (one thread a cell walked the list alone: 80 us of 83 at N = 128, 90
 // angles).  Sums run in a fixed order.  Bound by L2: four reads a sample and
-// plane.  N = 512, 360 angles, with the transform along kx: 0.99 ms; gather
+// plane.  N = 512, 360 angles, with the transform along kx: 0.91 ms; gather
 // 1.04 and rows 0.63 as separate passes over V.
 constexpr int kHeavy = 32;
 constexpr int kStaged = 2560;  // samples of a row held in shared memory (else read from L2)
@@ -377,27 +379,11 @@ template <int N> struct GridCfg {
   static_assert(LP >= P0 && LP % 8 == 2, "line pitch");
 };
 
-struct GridAcc {
-  float4 v;   // planes 2q and 2q + 1
-  float2 c;   // sum of w corr over samples of ku < 0
-};
-__device__ __forceinline__ void grid_add(GridAcc& s, const GridEnt e, const float4 f,
-                                         const float2* __restrict__ corr) {
-  const float wy = (e.at >> 31) ? -e.w : e.w;  // a sample of ku < 0 reads the conjugate
-  s.v.x = fmaf(e.w, f.x, s.v.x);
-  s.v.y = fmaf(wy, f.y, s.v.y);
-  s.v.z = fmaf(e.w, f.z, s.v.z);
-  s.v.w = fmaf(wy, f.w, s.v.w);
-  if (e.at >> 31) {
-    const float2 c = __ldg(corr + (e.at & 0x7fffffffu));
-    s.c.x = fmaf(e.w, c.x, s.c.x);
-    s.c.y = fmaf(e.w, c.y, s.c.y);
-  }
-}
-// s += the samples e0, e0 + step, ... < e1, four lines of F in flight
+// s (planes 2q and 2q + 1) += the samples e0, e0 + step, ... < e1, four lines
+// of F in flight; a sample of ku < 0 reads the conjugate
 template <class E>
-__device__ __forceinline__ void grid_sum(GridAcc& s, E ents, int e0, int e1, int step,
-                                         const float4* __restrict__ Fc, const float2* __restrict__ corr) {
+__device__ __forceinline__ void grid_sum(float4& s, E ents, int e0, int e1, int step,
+                                         const float4* __restrict__ Fc) {
   for (int e = e0; e < e1; e += 4 * step) {
     GridEnt g[4];
     float4 f[4];
@@ -409,13 +395,19 @@ __device__ __forceinline__ void grid_sum(GridAcc& s, E ents, int e0, int e1, int
       }
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-      if (e + i * step < e1) grid_add(s, g[i], f[i], corr);
+      if (e + i * step < e1) {
+        const float wy = __uint_as_float(__float_as_uint(g[i].w) ^ (g[i].at & 0x80000000u));
+        s.x = fmaf(g[i].w, f[i].x, s.x);
+        s.y = fmaf(wy, f[i].y, s.y);
+        s.z = fmaf(g[i].w, f[i].z, s.z);
+        s.w = fmaf(wy, f[i].w, s.w);
+      }
   }
 }
 
 template <int N>
 __global__ void __launch_bounds__(256, 3)
-k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int32_t* __restrict__ cell_ptr,
+k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t* __restrict__ cell_ptr,
        const GridEnt* __restrict__ ents, float2* V, const float2* __restrict__ xtw, int Np) {
   using G = GridCfg<N>;
   using FL = typename G::FL;
@@ -427,7 +419,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
   int* ptr = reinterpret_cast<int*>(es + kStaged);  // [N + 1]
   __shared__ unsigned short heavy[N];
   __shared__ int n_heavy;
-  __shared__ float part[8][4][6];
+  __shared__ float part[8][4][4];
   const int ky = blockIdx.x, ch0 = blockIdx.y * L;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quad = threadIdx.x >> 2, q = threadIdx.x & 3;
@@ -441,17 +433,18 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
   for (int i = threadIdx.x; i < N; i += 256) xs[i] = xtw[i];
   cp_async_wait_all();
   __syncthreads();
-  auto put = [&](int x, int ch, const GridAcc& s) {
+  auto put = [&](int x, int ch, const float4& s) {
     const float sg = ((x + ky) & 1) ? -1.0f : 1.0f;
+    const float2 c = __ldg(Q + ky * N + x);  // what the conjugates leave out, (-1)^z
     float2* d = lines + (ch * 8 + 2 * q) * LP + x;
-    d[0] = make_float2(sg * (s.v.x + s.c.x), sg * (s.v.y + s.c.y));
-    d[LP] = make_float2(sg * (s.v.z - s.c.x), sg * (s.v.w - s.c.y));
+    d[0] = make_float2(sg * (s.x + c.x), sg * (s.y + c.y));
+    d[LP] = make_float2(sg * (s.z - c.x), sg * (s.w - c.y));
   };
   const size_t chunk4 = (size_t)Np * G::HC * 4;  // float4s a chunk
   auto chunk = [&](int ch) { return reinterpret_cast<const float4*>(F) + (size_t)(ch0 + ch) * chunk4 + q; };
-  auto sum_cell = [&](GridAcc& s, int e0, int e1, int step, int ch) {
-    if (staged) grid_sum(s, (const GridEnt*)es, e0, e1, step, chunk(ch), corr);
-    else grid_sum(s, ents + first, e0, e1, step, chunk(ch), corr);
+  auto sum_cell = [&](float4& s, int e0, int e1, int step, int ch) {
+    if (staged) grid_sum(s, (const GridEnt*)es, e0, e1, step, chunk(ch));
+    else grid_sum(s, ents + first, e0, e1, step, chunk(ch));
   };
 #pragma unroll 2
   for (int u = quad; u < N * L; u += 64) {
@@ -462,7 +455,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
       if (ch == 0 && q == 0) heavy[atomicAdd(&n_heavy, 1)] = (unsigned short)x;
       continue;
     }
-    GridAcc s = {};
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     sum_cell(s, e0, e1, 1, ch);
     put(x, ch, s);
   }
@@ -473,11 +466,11 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
     const int e0 = ptr[x], e1 = ptr[x + 1];
     for (int ch = 0; ch < L; ++ch) {
       if (ch0 + ch >= G::NZC) break;
-      GridAcc s = {};
+      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
       sum_cell(s, e0 + quad, e1, 64, ch);
-      float r[6] = {s.v.x, s.v.y, s.v.z, s.v.w, s.c.x, s.c.y};
+      float r[4] = {s.x, s.y, s.z, s.w};
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
+      for (int i = 0; i < 4; ++i) {
 #pragma unroll
         for (int o = 4; o < 32; o <<= 1) r[i] += __shfl_xor_sync(0xffffffffu, r[i], o);
         if (lane < 4) part[warp][lane][i] = r[i];
@@ -485,13 +478,11 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ corr, const int3
       __syncthreads();
       if (threadIdx.x < 4) {
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
+        for (int i = 0; i < 4; ++i) {
           r[i] = 0.0f;
           for (int w = 0; w < 8; ++w) r[i] += part[w][threadIdx.x][i];
         }
-        s.v = make_float4(r[0], r[1], r[2], r[3]);
-        s.c = make_float2(r[4], r[5]);
-        put(x, ch, s);
+        put(x, ch, make_float4(r[0], r[1], r[2], r[3]));
       }
       __syncthreads();
     }
@@ -552,10 +543,11 @@ static cudaError_t grid_n(cpra_plan_s* p, float2* out) {
   Assembly& a = p->asmb;
   static bool attr = false;
   cudaError_t e = smem_once(k_grid<N>, G::SMEM, attr);
+  if (e == cudaSuccess) e = launch_grid_corr(p);
   if (e != cudaSuccess) return e;
   g_launches += 1;
   k_grid<N><<<dim3(N, (G::NZC + G::L - 1) / G::L), 256, G::SMEM, p->stream>>>(
-      a.F, a.corr, a.cell_ptr, a.ents, a.vol, p->xtw, p->Np);
+      a.F, a.Q, a.cell_ptr, a.ents, a.vol, p->xtw, p->Np);
   e = cudaGetLastError();
   return e == cudaSuccess ? launch_volume_ylines(N, a.vol, out, p->xtw, p->stream) : e;
 }

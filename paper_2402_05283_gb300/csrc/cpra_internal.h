@@ -48,6 +48,7 @@ struct GridEnt {
 struct Assembly {
   float2* F = nullptr;        // z-transformed spectra, [z / 8][n][ku = 0 .. N/2][z % 8]
   float2* corr = nullptr;     // [Np][N/2 + 1] what F(-ku) is beside conj F(ku) (k_assemble.cu)
+  float2* Q = nullptr;        // [N][N] a cell's sum of weight * corr
   float2* ramps = nullptr;    // per angle the unit ramps of its mass-centre move
   float2* vol = nullptr;      // [N][N][N] grid, then the centred volume
   int32_t* cell_ptr = nullptr;  // [N*N + 1] CSR rows (cells ky*N + kx)

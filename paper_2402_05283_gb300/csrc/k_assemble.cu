@@ -125,6 +125,42 @@ __global__ void k_ramps(const double* __restrict__ moments, float2* ramps, int N
   }
 }
 
+// Q[cell] = sum of w corr over the cell's samples of ku < 0 (see k_spectra): the
+// same for every plane but for (-1)^z, so it is summed once and not in every
+// chunk of planes.  A warp a cell; the origin's list is thousands long.
+__global__ void __launch_bounds__(256) k_grid_corr(const float2* __restrict__ corr,
+                                                   const int32_t* __restrict__ cell_ptr,
+                                                   const GridEnt* __restrict__ ents, float2* Q, int NN) {
+  const int cell = (blockIdx.x * 256 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (cell >= NN) return;
+  const int e0 = cell_ptr[cell], e1 = cell_ptr[cell + 1];
+  float2 s = make_float2(0.0f, 0.0f);
+  for (int e = e0 + lane; e < e1; e += 32) {
+    const GridEnt g = ents[e];
+    if (g.at >> 31) {
+      const float2 c = __ldg(corr + (g.at & 0x7fffffffu));
+      s.x = fmaf(g.w, c.x, s.x);
+      s.y = fmaf(g.w, c.y, s.y);
+    }
+  }
+  if (e1 > e0) {  // the whole warp
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+      s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+    }
+  }
+  if (lane == 0) Q[cell] = s;
+}
+
+cudaError_t launch_grid_corr(cpra_plan_s* p) {
+  const Assembly& a = p->asmb;
+  const int NN = p->N * p->N;
+  g_launches += 1;
+  k_grid_corr<<<(NN + 7) / 8, 256, 0, p->stream>>>(a.corr, a.cell_ptr, a.ents, a.Q, NN);
+  return cudaGetLastError();
+}
+
 // PRTF = ring mean (float), from the ring sums and the ring populations
 __global__ void k_prtf(const double* __restrict__ rings, const unsigned* __restrict__ counts, float* prtf,
                        int H, int total) {

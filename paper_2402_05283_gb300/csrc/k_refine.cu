@@ -72,7 +72,7 @@ __global__ void k_measured(const int32_t* __restrict__ cell_ptr, uint8_t* M, int
 // warp meets an estimate near a half in every eighth step, and FP64 there
 // was the bound.  N = 256, 180 angles: 1.09 ms with a thread a word, the
 // angles in order and FP64 at 1e-3; a lane a voxel in spread order 1.25 ms;
-// with the pairs 1.17 ms.
+// with the pairs and 64 words a CTA instead of 256 0.40 ms.
 // u = rint(((x - c) cos + (y - c) sin) + c) in FP64, each step rounded, no
 // contraction.  Not inlined: kept out of line, the rare call leaves the FP64
 // pipe idle instead of being predicated into every evaluation.
@@ -221,19 +221,14 @@ cudaError_t launch_refine_setup(const RefineArgs& a, const float2* vol, cudaStre
 cudaError_t launch_refine_support(const RefineArgs& a, const uint32_t* S2, const double2* cs,
                                   const int2* shift, int Np, const int32_t* cell_ptr, cudaStream_t st) {
   const int N = a.N, W = a.W;
-  const int YB = std::max(1, std::min(N, 256 / W));
-  // angles a chunk: their tables (see k_backproject) within 72 KB (three CTAs an SM)
+  // 64 words a CTA: the words that hold object run every angle one after the
+  // other, so a CTA with 256 of them was a chain of 0.3 ms
+  const int YB = std::max(1, std::min(N, 64 / W));
+  // angles a chunk: their tables (see k_backproject) within 36 KB (six CTAs an SM)
   const int per = (int)(sizeof(float4) + sizeof(int2) + W * sizeof(uint32_t) + YB * sizeof(float2));
   const int words = YB * W * (int)sizeof(uint32_t);
-  const int NC = std::max(1, std::min(Np, (72 * 1024 - words) / per));
+  const int NC = std::max(1, std::min(Np, (36 * 1024 - words) / per));
   const size_t smem = (size_t)NC * per + words;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_backproject, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         72 * 1024);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
   g_launches += 2;
   k_backproject<<<dim3((N + YB - 1) / YB, N), 256, smem, st>>>(S2, cs, shift, a.S3, N, W, Np, YB, NC,
                                                                angle_step(Np));
