@@ -70,19 +70,27 @@ constexpr bool kRowMaskInRegs = kSlimLines<FL> && FL::L == 1 && N == 512;
 __host__ __device__ constexpr int row_warps(int tasks) {
   return tasks % 4 == 0 ? 4 : tasks % 5 == 0 ? 5 : tasks % 3 == 0 ? 3 : tasks % 2 == 0 ? 2 : 1;
 }
-template <int N, class FL_> struct RowCfg {
+// GS: the rows have shared memory of their own; else the old rows are copied
+// into the transpose tile once the inverse transform has left it, which takes
+// half the shared memory and so lets four CTAs of the L-line plans share an SM
+// (row pass, us an angle, own rows / tile: N = 1024 3.28 / 2.58, 700 2.01 /
+// 1.79, 384 0.50 / 0.39; prime, which has no old rows, 1024 3.12 / 2.56)
+template <int N, class FL_, bool GS_ = true> struct RowCfg {
   using FL = FL_;
+  static constexpr bool GS = GS_;
   static_assert((N / 2) % FL::L == 0, "row pairs fill whole warps");
   static constexpr int WARPS = kSlimLines<FL> ? 8 : row_warps((N / 2) / FL::L);
   static constexpr int GROWS = 2 * FL::L;                  // image rows per warp
   static constexpr int GFLOATS = GROWS * N;
-  static constexpr int WARP_F2 = FL::TSIZE + GFLOATS / 2;  // float2 per warp
+  static constexpr int WARP_F2 = FL::TSIZE + (GS ? GFLOATS / 2 : 0);  // float2 per warp
+  static constexpr int MINB = GS || WARPS > 4 ? 3 : 4;
   static constexpr size_t SMEM = sizeof(float2) * (N + WARPS * WARP_F2);
 };
-template <int N, int PREC> using RowW = RowCfg<N, typename WLines<N, PREC>::type>;
+template <int N, int PREC>
+using RowW = RowCfg<N, typename WLines<N, PREC>::type, PREC != kPrecFP32 || kSlimLines<typename WLines<N, PREC>::type>>;
 // the prime keeps the L-line plans: its three taps a pixel are loaded in
 // registers, where the extra warps of the one-line plan do not pay
-template <int N, int PREC> using PrimeW = RowCfg<N, WarpLines<N>>;
+template <int N, int PREC> using PrimeW = RowCfg<N, WarpLines<N>, PREC != kPrecFP32>;
 
 // extra shared memory of the tensor-core path (TcLayout of fftw_tc.cuh): the
 // block DFT matrices, the CTA's A tile, the unscale factors, the mbarrier
@@ -195,7 +203,7 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
   float2* xs = smem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* T = smem + N + warp * RW::WARP_F2;
-  float* Gs = reinterpret_cast<float*>(T + FL::TSIZE);  // this warp's 2L rows of g
+  float* Gs = reinterpret_cast<float*>(T + (RW::GS ? FL::TSIZE : 0));  // this warp's 2L rows of g
   uint32_t tc_phase = 0;
   const TcCtx tc = tc_setup<N, PREC, RW::WARPS>(reinterpret_cast<char*>(smem + N + RW::WARPS * RW::WARP_F2),
                                                 J->tcw, J->status, &tc_phase);
@@ -214,12 +222,15 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
     cp_async_commit();
   }
   constexpr int GC = RW::GFLOATS / 4;  // 16-byte pieces
-  if (algo != kER) {  // ER does not look at the old iterate: 4 of 16 N^2 bytes less
+  auto load_old = [&] {  // ER does not look at the old iterate: 4 of 16 N^2 bytes less
+    if (algo != kER) {
 #pragma unroll
-    for (int k = 0; k < (GC + 31) / 32; ++k)
-      if (GC % 32 == 0 || lane + 32 * k < GC) cp_async16(Gs + 4 * (lane + 32 * k), grow + 4 * lane + 128 * k);
-  }
-  cp_async_commit();
+      for (int k = 0; k < (GC + 31) / 32; ++k)
+        if (GC % 32 == 0 || lane + 32 * k < GC) cp_async16(Gs + 4 * (lane + 32 * k), grow + 4 * lane + 128 * k);
+    }
+    cp_async_commit();
+  };
+  if constexpr (RW::GS) load_old();
   if (bx == 0 && threadIdx.x == 0) {
     if (err_slot >= 0) {
       const double den = sumA2[n];
@@ -232,7 +243,7 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
   if constexpr (kRowMaskInRegs<N, FL>)
     smask = __ldg(S + ((size_t)n * N + 2 * pair0 + (lane >> 4)) * W + (lane & 15));
   load_xtw<N>(xs, xtw, RW::WARPS * 32);
-  cp_async_wait_group<1>();  // this lane's spectrum copies have landed
+  cp_async_wait_group<RW::GS ? 1 : 0>();  // this lane's spectrum copies have landed
   __syncthreads();           // xs, and every lane's copies
   // packed row spectra -> Z = H(row 2p) + i H(row 2p+1), B layout, without
   // branches: k < H reads column k, k > H column N - k (sign s = -1)
@@ -275,7 +286,8 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
   }
   __syncwarp();  // the tile is the transforms' scratch from here on
   float2 a[FL::TA][FL::E1];
-  lines_inv<N, PREC, FL>(b, a, T, xs, lane, &tc);
+  if constexpr (RW::GS) lines_inv<N, PREC, FL>(b, a, T, xs, lane, &tc);
+  else FL::inv(b, a, T, xs, lane, load_old);
   if constexpr (kRowMaskInRegs<N, FL>) smask = warp_bit_transpose(smask, lane);
   cp_async_wait_all();
   __syncwarp();
@@ -320,6 +332,7 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
   else if (algo == kER) update_rows(std::integral_constant<int, kER>{});
   else update_rows(std::integral_constant<int, kRAAR>{});
   if (forward) {
+    if constexpr (!RW::GS) __syncwarp();  // the old rows leave the tile
     lines_fwd<N, PREC, FL>(a, b, T, xs, lane, &tc);
     store_pairs_w<N, FL>(b, T, Hn, pair0, lane);
   }
@@ -327,7 +340,7 @@ __device__ __forceinline__ void rowpass_tile(const JobStatic* __restrict__ js,
 }
 
 template <int N, int PREC>
-__global__ void __launch_bounds__(RowW<N, PREC>::WARPS * 32, 3)
+__global__ void __launch_bounds__(RowW<N, PREC>::WARPS * 32, RowW<N, PREC>::MINB)
 k_rowpass_w(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
             const int2* __restrict__ tiles) {
   rowpass_tile<N, PREC>(js, st, tiles[blockIdx.y], blockIdx.x);
@@ -514,7 +527,7 @@ template <int N, int PREC> struct ColW {
   static_assert((N / 2) % CB == 0 && CB % FL::L == 0, "column blocks");
   static constexpr int WARPS = CB / FL::L;
   static constexpr int NT = WARPS * 32;
-  static constexpr int MINB = kSlimLines<FL> ? 3 : (NT <= 256 || N == 700 ? 2 : 1);
+  static constexpr int MINB = kSlimLines<FL> ? 3 : NT <= 128 ? 4 : (NT <= 256 || N == 700 ? 2 : 1);
   static constexpr int SP = CB + 1;  // staging pitch
   static constexpr int N2 = N / 2;
   static constexpr int STAGE = N * SP;
