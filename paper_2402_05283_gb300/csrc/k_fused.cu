@@ -69,43 +69,54 @@ __device__ __forceinline__ uint32_t slab_at(uint32_t sb, int y, int c) {
   return dsm_map(sb + 8u * (uint32_t)(y * F::SP + (c & (F::CW - 1))), (uint32_t)(c / F::CW));
 }
 
-// Z = H(row 2p) + i H(row 2p+1) of this warp's row pairs, B layout, read
-// from the packed spectra in the cluster's slabs
+// Z = H(row 2p) + i H(row 2p+1) of this warp's row pairs, B layout, from the
+// packed spectra in the cluster's slabs.  Frequencies k and N - k need the same
+// packed value in different lanes, so the rows come into the warp's tile
+// first, each value once over the cluster's network, all loads in flight
+// (ten iterations of 180 angles at N = 256: 704 us with a remote load a use,
+// 651 so).  A cluster of one CTA (N = 64) reads its own slab directly.
 template <int N, class FL>
-__device__ __forceinline__ void gather_pairs(float2 (&b)[FL::TB][FL::E2], uint32_t sb, int pair0,
-                                             int lane) {
+__device__ __forceinline__ void gather_pairs(float2 (&b)[FL::TB][FL::E2], float2* T, const float2* slab,
+                                             uint32_t sb, int pair0, int lane) {
   using F = FusedCfg<N, 2>;
-  constexpr int H = N / 2;
+  constexpr int H = N / 2, RV = 2 * FL::L * H / 32;  // values a lane
+  static_assert(H % 32 == 0, "row spectra");
+  constexpr bool local = F::C == 1;
+  constexpr int R1 = local ? F::SP : H;  // from a pair's first row to its second
+  if constexpr (!local) {
+    float2 v[RV];
+#pragma unroll
+    for (int q = 0; q < RV; ++q)
+      v[q] = dsm_ld(slab_at<N>(sb, 2 * pair0 + q / (H / 32), lane + 32 * (q % (H / 32))));
+#pragma unroll
+    for (int q = 0; q < RV; ++q) T[lane + 32 * q] = v[q];
+    __syncwarp();
+  }
   static_for<0, FL::TB>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
-    const int y0 = 2 * (pair0 + FL::b_line(t));
+    const float2* r0 = local ? slab + 2 * (pair0 + FL::b_line(t)) * F::SP : T + FL::b_line(t) * N;
+    const float2* r1 = r0 + R1;
     static_for<0, FL::E2>([&](auto KK) {
       constexpr int j = decltype(KK)::value;
       const int k = FL::b_k(t, j);
-      const int c = k < H ? k : (k == H ? 0 : N - k);
-      const uint32_t a0 = slab_at<N>(sb, y0, c);
-      const float2 h0 = dsm_ld(a0), h1 = dsm_ld(a0 + 8u * F::SP);
-      float2 z;
-      if (k == 0) {
-        z = make_float2(h0.x, h1.x);
-      } else if (k == H) {
-        z = make_float2(h0.y, h1.y);
-      } else if (k < H) {
-        z = make_float2(h0.x - h1.y, h0.y + h1.x);
-      } else {
-        z = make_float2(h0.x + h1.y, h1.x - h0.y);
-      }
+      const bool up = k > H;
+      const int c = up ? N - k : (k == H ? 0 : k);
+      const float s = up ? -1.0f : 1.0f;
+      const float2 h0 = r0[c], h1 = r1[c];
+      float2 z = make_float2(fmaf(-s, h1.y, h0.x), fmaf(s, h0.y, h1.x));
+      if (c == 0) z = k == 0 ? make_float2(h0.x, h1.x) : make_float2(h0.y, h1.y);
       b[i][j] = z;
     });
   });
+  __syncwarp();  // the tile is the transforms' scratch from here on
 }
 
 // Z (B layout) of this warp's row pairs -> packed half spectra of both rows
 // of each pair, written to the slabs (T pairs index k with N - k)
 template <int N, class FL>
-__device__ __forceinline__ void scatter_pairs(float2 (&b)[FL::TB][FL::E2], float2* T, uint32_t sb,
-                                              int pair0, int lane) {
+__device__ __forceinline__ void scatter_pairs(float2 (&b)[FL::TB][FL::E2], float2* T, float2* slab,
+                                              uint32_t sb, int pair0, int lane) {
   using F = FusedCfg<N, 2>;
   constexpr int H = N / 2;
   static_for<0, FL::TB>([&](auto II) {
@@ -134,9 +145,14 @@ __device__ __forceinline__ void scatter_pairs(float2 (&b)[FL::TB][FL::E2], float
         h0 = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
         h1 = make_float2(0.5f * (z.y + zm.y), 0.5f * (zm.x - z.x));
       }
-      const uint32_t a0 = slab_at<N>(sb, y0, k);
-      dsm_st(a0, h0);
-      dsm_st(a0 + 8u * F::SP, h1);
+      if constexpr (F::C == 1) {
+        slab[y0 * F::SP + k] = h0;
+        slab[(y0 + 1) * F::SP + k] = h1;
+      } else {
+        const uint32_t a0 = slab_at<N>(sb, y0, k);
+        dsm_st(a0, h0);
+        dsm_st(a0 + 8u * F::SP, h1);
+      }
     }
   }
   __syncwarp();
@@ -220,7 +236,7 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
     if (ca.store_g) store_rows<N, FL>(a, Z->g_dst + (size_t)n * N * N, pair0, lane);
     float2 b[FL::TB][FL::E2];
     FL::fwd(a, b, T, xs, lane);
-    scatter_pairs<N, FL>(b, T, sb, pair0, lane);
+    scatter_pairs<N, FL>(b, T, slab, sb, pair0, lane);
   }
   cluster_sync_all();
 
@@ -378,12 +394,12 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
       if (rule != kER && q) load_old(q, old);
       float2 b[FL::TB][FL::E2];
       float2 a[FL::TA][FL::E1];
-      gather_pairs<N, FL>(b, sb, pq, lane);
+      gather_pairs<N, FL>(b, T, slab, sb, pq, lane);
       FL::inv(b, a, T, xs, lane);
       update(q, a, old, rule);
       if (fwd) {
         FL::fwd(a, b, T, xs, lane);
-        scatter_pairs<N, FL>(b, T, sb, pq, lane);
+        scatter_pairs<N, FL>(b, T, slab, sb, pq, lane);
       }
     }
     if (rank == 0 && warp == 0 && err_slot >= 0) {
