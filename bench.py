@@ -150,7 +150,8 @@ NCU_ITERATION_TRAFFIC = {
 # the kernels' sources and the host code that orders their launches and
 # tiles (the order decides what the L2 still holds between passes)
 KERNEL_SOURCES = ("fast_kernels.cuh", "fftw.cuh", "fftw_pair.cuh", "fft.cuh", "cpra_internal.h",
-                  "k_fast.cu", "k_fused.cu", "taps.cuh", "api.cu")
+                  "k_fast.cu", "k_fast_a.cu", "k_fast_b.cu", "k_fast_c.cu", "k_fused.cu", "cluster.cuh",
+                  "taps.cuh", "api.cu")
 
 
 def kernel_fingerprint() -> str:

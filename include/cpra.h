@@ -314,8 +314,8 @@ cpra_status cpra_download_wait(cpra_plan_t plan);
  * twin choice against the best episode, averaging); PRTF as in its results
  * section (its ref. 23).  The call runs on the guesses' and dst's streams and
  * returns when the merge is complete.  Besides the assembly buffers, dst
- * allocates about 8 N^2 Np bytes of scratch on first use (4 N^2 Np more
- * with prtf).  Each guess's
+ * allocates about 8 N^2 Np bytes of scratch on first use and 12 N Np bytes
+ * a kept guess (4 N Np more with prtf).  Each guess's
  * state is only read; its row spectra buffer is reused.  INVALID_ARG for bad
  * counts, sizes or pointers, NOT_READY for a guess that has not iterated or
  * has absent angles. */
@@ -391,7 +391,7 @@ int64_t cpra_launch_count(void);
 /* Shrink-wrap support update without any device allocation.
  *
  * The paper has no counterpart: this is a library service.  It runs the same
- * kernels and the same arithmetic as the shrink-wrap step of cpra_iterate
+ * arithmetic as the shrink-wrap step of cpra_iterate, in the same order
  * (blur P_{S+} g with the periodic Gaussian of sigma pixels, keep pixels at
  * or above tau times each pattern's maximum; a pattern whose maximum is 0
  * keeps S_in), for callers that cannot call cudaMalloc: cudaMalloc and
@@ -443,9 +443,10 @@ typedef struct cpra_batch_s* cpra_batch_t;
  * Jacobi plans must not use shrink-wrap (UNSUPPORTED).  Gauss-Seidel plans
  * (sweep 1) of the same N, engine and n_ei form a group whose sweeps run
  * together: their Step A as rows over every member's angle 0, then one
- * launch per angle of the sweep (fused engine; prime + n_ei column and row
- * launches otherwise) over every member that has that angle, shrink-wrap at
- * episode ends; calls must run whole episodes (INVALID_ARG otherwise) and
+ * launch an episode (block-wide engine, N in {16, 32, 48, 96, 160, 320};
+ * fused engine, N in {64, 128, 256}) or one launch per angle of the sweep
+ * (fused engine; prime + n_ei column and row launches otherwise) over every
+ * member that has that angle, shrink-wrap at episode ends; calls must run whole episodes (INVALID_ARG otherwise) and
  * are not captured in a graph.  Plans must stay alive until
  * cpra_batch_destroy.  The batch holds device tables only. */
 cpra_status cpra_batch_create(const cpra_plan_t* plans, int32_t n, int32_t use_graph,

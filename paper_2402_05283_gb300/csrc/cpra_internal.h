@@ -391,11 +391,14 @@ bool fused_supported(int N);
 cudaError_t prepare_kernels_fused(int N);
 cudaError_t launch_fused(const Launch& L);
 
-// One launch for a whole Gauss-Seidel episode (k_sweep.cu): tile j = (member,
+// One launch for a whole Gauss-Seidel episode (k_sweep.cu at the block-wide
+// engine's sizes, k_fused.cu for N = 64, 128, 256): tile j = (member,
 // 0), the member's angles in order inside the launch; step row: the coupling
 // arguments, g_src, g = g_dst, err_slot, n_iters, hio_left.
 bool sweep_supported(int N, int engine);
 cudaError_t launch_sweep(const Launch& L);
+bool fused_sweep_supported(int N);
+cudaError_t launch_fused_sweep(const Launch& L);
 
 // records a failure of a call without a plan (cpra_last_error(NULL))
 cpra_status record_error(cpra_status st, const std::string& msg);

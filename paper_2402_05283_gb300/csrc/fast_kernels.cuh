@@ -354,7 +354,8 @@ k_rowpass_w(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
 // object) combination runs its own loop: pixel x reads column x, or N - x
 // mirrored (0 for x = 0, which only m = 0 can hold), at a per-lane base plus
 // a constant offset.
-template <int N, class FL, bool MIR, bool OBJ>
+// NC: the images are not written during the launch (read-only loads).
+template <int N, class FL, bool MIR, bool OBJ, bool NC>
 __device__ __forceinline__ void blend_tap(float2 (&a)[FL::TA][FL::E1], const float* src,
                                           const uint32_t* sk, float alpha, int W, int pair0,
                                           int lane) {
@@ -369,8 +370,8 @@ __device__ __forceinline__ void blend_tap(float2 (&a)[FL::TA][FL::E1], const flo
       constexpr int m = decltype(MM)::value;
       const int x = FL::a_x(t, m);
       const int xs_ = MIR ? (m == 0 && x == 0 ? 0 : N - x) : x;
-      float v0 = __ldg(r0 + xs_);
-      float v1 = __ldg(r0 + N + xs_);
+      float v0 = NC ? __ldg(r0 + xs_) : r0[xs_];
+      float v1 = NC ? __ldg(r0 + N + xs_) : r0[N + xs_];
       if constexpr (OBJ) {
         const bool in0 = (__ldg(m0 + (xs_ >> 5)) >> (xs_ & 31)) & 1u;
         const bool in1 = (__ldg(m0 + W + (xs_ >> 5)) >> (xs_ & 31)) & 1u;
@@ -383,7 +384,7 @@ __device__ __forceinline__ void blend_tap(float2 (&a)[FL::TA][FL::E1], const flo
   });
 }
 
-template <int N, class FL = WarpLines<N>>
+template <int N, class FL = WarpLines<N>, bool NC = true>
 __device__ __forceinline__ void blend_rows(float2 (&a)[FL::TA][FL::E1], const TapTab& tt,
                                            const CoupleArgs& ca, int W, int pair0, int lane) {
   const int ntaps = ca.n_taps;
@@ -397,11 +398,11 @@ __device__ __forceinline__ void blend_rows(float2 (&a)[FL::TA][FL::E1], const Ta
     const float* src = tt.src[k];
     const uint32_t* sk = tt.s[k];
     if (tt.mir[k]) {
-      if (obj) blend_tap<N, FL, true, true>(a, src, sk, alpha, W, pair0, lane);
-      else blend_tap<N, FL, true, false>(a, src, sk, alpha, W, pair0, lane);
+      if (obj) blend_tap<N, FL, true, true, NC>(a, src, sk, alpha, W, pair0, lane);
+      else blend_tap<N, FL, true, false, NC>(a, src, sk, alpha, W, pair0, lane);
     } else {
-      if (obj) blend_tap<N, FL, false, true>(a, src, sk, alpha, W, pair0, lane);
-      else blend_tap<N, FL, false, false>(a, src, sk, alpha, W, pair0, lane);
+      if (obj) blend_tap<N, FL, false, true, NC>(a, src, sk, alpha, W, pair0, lane);
+      else blend_tap<N, FL, false, false, NC>(a, src, sk, alpha, W, pair0, lane);
     }
   }
 }

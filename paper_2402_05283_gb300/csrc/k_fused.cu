@@ -184,9 +184,16 @@ __device__ __forceinline__ void support_mask(uint32_t (&mk)[FusedCfg<N, 2>::MASK
 // in the other form): a test of the serving loop submits 2000 iterations of
 // eight angles and needs them to outlast 20 ms.
 constexpr int kFewTiles64 = 8;
-template <int N, int Q> constexpr bool kPublishAtOnce = N == 64 && Q == 2;
+template <int N, int Q>
+__device__ __forceinline__ bool publish_at_once() { return N == 64 && Q == 2 && gridDim.y <= kFewTiles64; }
 
-template <int N, bool MASKED, int Q>
+// SWEEP: a Gauss-Seidel episode, the angles of the member one after the other
+// inside the launch (a launch per angle left its one to four CTAs a guess alone
+// on the device; 90 angles, 16 guesses, 2 iterations: N = 64 25 us an angle,
+// 128 42, 256 54; in one launch 16, 28 and 40).
+// An angle's rows stay with their warp, so the taps on earlier angles read
+// what the warp wrote itself.
+template <int N, bool MASKED, int Q, bool SWEEP = false>
 __global__ void __launch_bounds__(FusedCfg<N, Q>::NT, FusedCfg<N, Q>::MINB)
 k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
         const int2* __restrict__ tiles) {
@@ -203,7 +210,6 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
   const JobStep* Z = st + tl.x;
   if (!Z->active) return;  // the same for every CTA of the cluster
   const int rank = (int)cg::this_cluster().block_rank();
-  const int n = tl.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* T = smem + F::SLAB + warp * FL::TSIZE;
   const uint32_t sb = smem_u32(slab);
@@ -217,218 +223,221 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
   const long long err_slot = Z->err_slot;
 
   load_xtw<N>(xs, J->xtw, F::NT);
-  fill_taps<N>(tt, ca, Z->g_src, Z->g_dst, J->S, n, Np, W, J->present);
-  // the support is fixed during a launch: each lane keeps its pixels' bits
-  uint32_t mask[Q][F::MASKW];
-  static_for<0, Q>([&](auto QQ) {
-    constexpr int q = decltype(QQ)::value;
-    support_mask<N, FL>(mask[q], J->S + (size_t)n * N * W, W,
-                        rank * F::CW + (warp + q * F::NW) * FL::L, lane);
-  });
-  cluster_sync_all();  // every CTA runs before any DSMEM access; xs and taps visible
-
-  // ---- prime: (coupled) rows -> R2C -> slabs
+  const int n_end = SWEEP ? Np : tl.y + 1;
 #pragma unroll 1
-  for (int q = 0; q < Q; ++q) {
-    const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
-    float2 a[FL::TA][FL::E1];
-    blend_rows<N, FL>(a, tt, ca, W, pair0, lane);
-    if (ca.store_g) store_rows<N, FL>(a, Z->g_dst + (size_t)n * N * N, pair0, lane);
-    float2 b[FL::TB][FL::E2];
-    FL::fwd(a, b, T, xs, lane);
-    scatter_pairs<N, FL>(b, T, slab, sb, pair0, lane);
-  }
-  cluster_sync_all();
+  for (int n = SWEEP ? 0 : tl.y; n < n_end; ++n) {
+    fill_taps<N>(tt, ca, Z->g_src, Z->g_dst, J->S, n, Np, W, J->present);
+    // the support is fixed during a launch: each lane keeps its pixels' bits
+    uint32_t mask[Q][F::MASKW];
+    static_for<0, Q>([&](auto QQ) {
+      constexpr int q = decltype(QQ)::value;
+      support_mask<N, FL>(mask[q], J->S + (size_t)n * N * W, W,
+                          rank * F::CW + (warp + q * F::NW) * FL::L, lane);
+    });
+    cluster_sync_all();  // every CTA runs before any DSMEM access; xs and taps visible
 
-  const float inv = 1.0f / N;
-  // A_sym of column task q (B layout), read through L1
-  auto load_av = [&](int q, float (&av)[FL::TB][FL::E2]) {
-    const int cg0 = rank * F::CW + (warp + q * F::NW) * FL::L;
-    static_for<0, FL::TB>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      const float* Ac = A_T + ((size_t)n * H + cg0 + FL::b_line(t)) * N;
-      static_for<0, FL::E2>([&](auto KK) {
-        constexpr int j = decltype(KK)::value;
-        av[i][j] = __ldg(Ac + FL::b_k(t, j));
-      });
-    });
-  };
-  // the old iterate of row task q (A layout), read by the HIO and RAAR rules
-  auto load_old = [&](int q, float2 (&old)[FL::TA][FL::E1]) {
-    const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
-    static_for<0, FL::TA>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      const float* g0 = g + ((size_t)n * N + 2 * (pair0 + FL::a_line(t))) * N;
-      static_for<0, FL::E1>([&](auto MM) {
-        constexpr int m = decltype(MM)::value;
-        const int x = FL::a_x(t, m);
-        old[i][m] = make_float2(g0[x], g0[N + x]);
-      });
-    });
-  };
-  // column task q: FFT_y, projection onto A_sym (error terms of weight 2
-  // into err2, of weight 1 into err1), IFFT_y
-  auto col_task = [&](int q, const float (&av)[FL::TB][FL::E2], float& err2, float& err1) {
-    const int cl0 = (warp + q * F::NW) * FL::L;  // first local column of the task
-    const int cg0 = rank * F::CW + cl0;           // its packed column index
-    float2 a[FL::TA][FL::E1];
-    static_for<0, FL::TA>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      const int line = FL::a_line(t);
-      static_for<0, FL::E1>([&](auto MM) {
-        constexpr int m = decltype(MM)::value;
-        a[i][m] = slab[FL::a_x(t, m) * F::SP + cl0 + line];
-      });
-    });
-    float2 b[FL::TB][FL::E2];
-    FL::fwd(a, b, T, xs, lane);
-    static_for<0, FL::TB>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      if (cg0 + FL::b_line(t) != 0) {
+    // ---- prime: (coupled) rows -> R2C -> slabs
+#pragma unroll 1
+    for (int q = 0; q < Q; ++q) {
+      const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
+      float2 a[FL::TA][FL::E1];
+      blend_rows<N, FL, !SWEEP>(a, tt, ca, W, pair0, lane);
+      if (ca.store_g) store_rows<N, FL>(a, Z->g_dst + (size_t)n * N * N, pair0, lane);
+      float2 b[FL::TB][FL::E2];
+      FL::fwd(a, b, T, xs, lane);
+      scatter_pairs<N, FL>(b, T, slab, sb, pair0, lane);
+    }
+    cluster_sync_all();
+
+    const float inv = 1.0f / N;
+    // A_sym of column task q (B layout), read through L1
+    auto load_av = [&](int q, float (&av)[FL::TB][FL::E2]) {
+      const int cg0 = rank * F::CW + (warp + q * F::NW) * FL::L;
+      static_for<0, FL::TB>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        const int t = lane + 32 * i;
+        const float* Ac = A_T + ((size_t)n * H + cg0 + FL::b_line(t)) * N;
         static_for<0, FL::E2>([&](auto KK) {
           constexpr int j = decltype(KK)::value;
-          b[i][j] = project_w<MASKED>(b[i][j], av[i][j], err2);
+          av[i][j] = __ldg(Ac + FL::b_k(t, j));
         });
-      }
-    });
-    if (cg0 == 0) {
-      // column 0 packs G(., 0) + i G(., N/2); both are Hermitian along ky
-      static_for<0, FL::TB>([&](auto II) {
+      });
+    };
+    // the old iterate of row task q (A layout), read by the HIO and RAAR rules
+    auto load_old = [&](int q, float2 (&old)[FL::TA][FL::E1]) {
+      const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
+      static_for<0, FL::TA>([&](auto II) {
         constexpr int i = decltype(II)::value;
         const int t = lane + 32 * i;
-        if (FL::b_line(t) == 0) {
-          static_for<0, FL::E2>([&](auto KK) {
-            constexpr int j = decltype(KK)::value;
-            T[FL::b_k(t, j)] = b[i][j];
-          });
-        }
+        const float* g0 = g + ((size_t)n * N + 2 * (pair0 + FL::a_line(t))) * N;
+        static_for<0, FL::E1>([&](auto MM) {
+          constexpr int m = decltype(MM)::value;
+          const int x = FL::a_x(t, m);
+          old[i][m] = make_float2(g0[x], g0[N + x]);
+        });
       });
-      __syncwarp();
-      const float* An = J->A_nyq + (size_t)n * N;
-      static_for<0, FL::TB>([&](auto II) {
-        constexpr int i = decltype(II)::value;
-        const int t = lane + 32 * i;
-        if (FL::b_line(t) == 0) {
-          static_for<0, FL::E2>([&](auto KK) {
-            constexpr int j = decltype(KK)::value;
-            const int ky = FL::b_k(t, j);
-            const float2 z = T[ky], zm = T[(N - ky) % N];
-            const float2 g0 = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
-            const float2 gn = make_float2(0.5f * (z.y + zm.y), 0.5f * (zm.x - z.x));
-            const float2 p0 = project_w<MASKED>(g0, av[i][j], err1);
-            const float2 pn = project_w<MASKED>(gn, __ldg(An + ky), err1);
-            b[i][j] = make_float2(p0.x - pn.y, p0.y + pn.x);
-          });
-        }
-      });
-      __syncwarp();
-    }
-    FL::inv(b, a, T, xs, lane);
-    static_for<0, FL::TA>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      const int line = FL::a_line(t);
-      static_for<0, FL::E1>([&](auto MM) {
-        constexpr int m = decltype(MM)::value;
-        slab[FL::a_x(t, m) * F::SP + cl0 + line] = cscale(a[i][m], inv);
-      });
-    });
-  };
-  // HIO / RAAR / ER update of row task q from g' = a / N; a <- the new iterate
-  auto update = [&](int q, float2 (&a)[FL::TA][FL::E1], const float2 (&old)[FL::TA][FL::E1],
-                    int rule) {
-    const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
-    uint32_t mq[F::MASKW];
-    static_for<0, F::MASKW>([&](auto WW) {
-      constexpr int w = decltype(WW)::value;
-      mq[w] = q ? mask[Q - 1][w] : mask[0][w];
-    });
-    static_for<0, FL::TA>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      float* g0 = g + ((size_t)n * N + 2 * (pair0 + FL::a_line(t))) * N;
-      static_for<0, FL::E1>([&](auto MM) {
-        constexpr int m = decltype(MM)::value;
-        constexpr int bit = (i * FL::E1 + m) * 2;
-        const int x = FL::a_x(t, m);
-        const float2 z = a[i][m];
-        const float gp0 = z.x * inv, gp1 = z.y * inv;
-        const bool s0 = (mq[bit >> 5] >> (bit & 31)) & 1u;
-        const bool s1 = (mq[bit >> 5] >> ((bit + 1) & 31)) & 1u;
-        const float n0 = update_pixel(old[i][m].x, gp0, s0, rule, beta, c2);
-        const float n1 = update_pixel(old[i][m].y, gp1, s1, rule, beta, c2);
-        g0[x] = n0;
-        g0[N + x] = n1;
-        a[i][m] = make_float2(n0, n1);
-      });
-    });
-  };
-
-  float av[FL::TB][FL::E2];
-  float2 old[FL::TA][FL::E1];
-  load_av(0, av);
-  for (int it = 0; it < n_iters; ++it) {
-    const int rule = it < hio_left ? Z->algo : kER;  // HIO or RAAR, then ER
-    const bool fwd = it + 1 < n_iters;
-    float es = 0.0f, ee = 0.0f;  // error terms as an FP32 pair
-#pragma unroll 1
-    for (int q = 0; q < Q; ++q) {
-      if (q) load_av(q, av);
-      float err2 = 0.0f, err1 = 0.0f;
-      col_task(q, av, err2, err1);
-      two_add(es, ee, 2.0f * err2);
-      two_add(es, ee, err1);
-    }
-    const double errd = warp_sum(es, ee);
-    if (lane == 0) red[warp] = errd;
-    cluster_arrive();
-    if (rule != kER) load_old(0, old);  // in flight across the barrier
-    cluster_wait();
-#pragma unroll 1
-    for (int q = 0; q < Q; ++q) {
-      const int pq = rank * F::CW + (warp + q * F::NW) * FL::L;
-      if (rule != kER && q) load_old(q, old);
-      float2 b[FL::TB][FL::E2];
+    };
+    // column task q: FFT_y, projection onto A_sym (error terms of weight 2
+    // into err2, of weight 1 into err1), IFFT_y
+    auto col_task = [&](int q, const float (&av)[FL::TB][FL::E2], float& err2, float& err1) {
+      const int cl0 = (warp + q * F::NW) * FL::L;  // first local column of the task
+      const int cg0 = rank * F::CW + cl0;           // its packed column index
       float2 a[FL::TA][FL::E1];
-      gather_pairs<N, FL>(b, T, slab, sb, pq, lane);
-      FL::inv(b, a, T, xs, lane);
-      update(q, a, old, rule);
-      if (fwd) {
-        FL::fwd(a, b, T, xs, lane);
-        scatter_pairs<N, FL>(b, T, slab, sb, pq, lane);
+      static_for<0, FL::TA>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        const int t = lane + 32 * i;
+        const int line = FL::a_line(t);
+        static_for<0, FL::E1>([&](auto MM) {
+          constexpr int m = decltype(MM)::value;
+          a[i][m] = slab[FL::a_x(t, m) * F::SP + cl0 + line];
+        });
+      });
+      float2 b[FL::TB][FL::E2];
+      FL::fwd(a, b, T, xs, lane);
+      static_for<0, FL::TB>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        const int t = lane + 32 * i;
+        if (cg0 + FL::b_line(t) != 0) {
+          static_for<0, FL::E2>([&](auto KK) {
+            constexpr int j = decltype(KK)::value;
+            b[i][j] = project_w<MASKED>(b[i][j], av[i][j], err2);
+          });
+        }
+      });
+      if (cg0 == 0) {
+        // column 0 packs G(., 0) + i G(., N/2); both are Hermitian along ky
+        static_for<0, FL::TB>([&](auto II) {
+          constexpr int i = decltype(II)::value;
+          const int t = lane + 32 * i;
+          if (FL::b_line(t) == 0) {
+            static_for<0, FL::E2>([&](auto KK) {
+              constexpr int j = decltype(KK)::value;
+              T[FL::b_k(t, j)] = b[i][j];
+            });
+          }
+        });
+        __syncwarp();
+        const float* An = J->A_nyq + (size_t)n * N;
+        static_for<0, FL::TB>([&](auto II) {
+          constexpr int i = decltype(II)::value;
+          const int t = lane + 32 * i;
+          if (FL::b_line(t) == 0) {
+            static_for<0, FL::E2>([&](auto KK) {
+              constexpr int j = decltype(KK)::value;
+              const int ky = FL::b_k(t, j);
+              const float2 z = T[ky], zm = T[(N - ky) % N];
+              const float2 g0 = make_float2(0.5f * (z.x + zm.x), 0.5f * (z.y - zm.y));
+              const float2 gn = make_float2(0.5f * (z.y + zm.y), 0.5f * (zm.x - z.x));
+              const float2 p0 = project_w<MASKED>(g0, av[i][j], err1);
+              const float2 pn = project_w<MASKED>(gn, __ldg(An + ky), err1);
+              b[i][j] = make_float2(p0.x - pn.y, p0.y + pn.x);
+            });
+          }
+        });
+        __syncwarp();
       }
+      FL::inv(b, a, T, xs, lane);
+      static_for<0, FL::TA>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        const int t = lane + 32 * i;
+        const int line = FL::a_line(t);
+        static_for<0, FL::E1>([&](auto MM) {
+          constexpr int m = decltype(MM)::value;
+          slab[FL::a_x(t, m) * F::SP + cl0 + line] = cscale(a[i][m], inv);
+        });
+      });
+    };
+    // HIO / RAAR / ER update of row task q from g' = a / N; a <- the new iterate
+    auto update = [&](int q, float2 (&a)[FL::TA][FL::E1], const float2 (&old)[FL::TA][FL::E1],
+                      int rule) {
+      const int pair0 = rank * F::CW + (warp + q * F::NW) * FL::L;
+      uint32_t mq[F::MASKW];
+      static_for<0, F::MASKW>([&](auto WW) {
+        constexpr int w = decltype(WW)::value;
+        mq[w] = q ? mask[Q - 1][w] : mask[0][w];
+      });
+      static_for<0, FL::TA>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        const int t = lane + 32 * i;
+        float* g0 = g + ((size_t)n * N + 2 * (pair0 + FL::a_line(t))) * N;
+        static_for<0, FL::E1>([&](auto MM) {
+          constexpr int m = decltype(MM)::value;
+          constexpr int bit = (i * FL::E1 + m) * 2;
+          const int x = FL::a_x(t, m);
+          const float2 z = a[i][m];
+          const float gp0 = z.x * inv, gp1 = z.y * inv;
+          const bool s0 = (mq[bit >> 5] >> (bit & 31)) & 1u;
+          const bool s1 = (mq[bit >> 5] >> ((bit + 1) & 31)) & 1u;
+          const float n0 = update_pixel(old[i][m].x, gp0, s0, rule, beta, c2);
+          const float n1 = update_pixel(old[i][m].y, gp1, s1, rule, beta, c2);
+          g0[x] = n0;
+          g0[N + x] = n1;
+          a[i][m] = make_float2(n0, n1);
+        });
+      });
+    };
+
+    float av[FL::TB][FL::E2];
+    float2 old[FL::TA][FL::E1];
+    load_av(0, av);
+    for (int it = 0; it < n_iters; ++it) {
+      const int rule = it < hio_left ? Z->algo : kER;  // HIO or RAAR, then ER
+      const bool fwd = it + 1 < n_iters;
+      float es = 0.0f, ee = 0.0f;  // error terms as an FP32 pair
+#pragma unroll 1
+      for (int q = 0; q < Q; ++q) {
+        if (q) load_av(q, av);
+        float err2 = 0.0f, err1 = 0.0f;
+        col_task(q, av, err2, err1);
+        two_add(es, ee, 2.0f * err2);
+        two_add(es, ee, err1);
+      }
+      const double errd = warp_sum(es, ee);
+      if (lane == 0) red[warp] = errd;
+      cluster_arrive();
+      if (rule != kER) load_old(0, old);  // in flight across the barrier
+      cluster_wait();
+#pragma unroll 1
+      for (int q = 0; q < Q; ++q) {
+        const int pq = rank * F::CW + (warp + q * F::NW) * FL::L;
+        if (rule != kER && q) load_old(q, old);
+        float2 b[FL::TB][FL::E2];
+        float2 a[FL::TA][FL::E1];
+        gather_pairs<N, FL>(b, T, slab, sb, pq, lane);
+        FL::inv(b, a, T, xs, lane);
+        update(q, a, old, rule);
+        if (fwd) {
+          FL::fwd(a, b, T, xs, lane);
+          scatter_pairs<N, FL>(b, T, slab, sb, pq, lane);
+        }
+      }
+      if (rank == 0 && warp == 0 && err_slot >= 0) {
+        // Fourier error of the iterate entering this iteration, summed in a
+        // fixed order over the cluster's warps (the partials stay put until
+        // every CTA has passed the barrier below)
+        double s = 0.0;
+        for (int q = lane; q < F::C * F::NW; q += 32)
+          s += dsm_ld_f64(dsm_map(smem_u32(red + q % F::NW), (uint32_t)(q / F::NW)));
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        // the raw sum; the square root and division wait until the last
+        // iteration (see publish_at_once for the exception)
+        if (lane == 0)
+          J->err_hist[(size_t)(err_slot + it) * Np + n] =
+              publish_at_once<N, Q>() ? publish_error(s, J->Cn[n], J->sumA2[n], J->status, n) : s;
+      }
+      cluster_arrive();
+      if (fwd) load_av(0, av);  // in flight across the barrier
+      cluster_wait();
     }
-    if (rank == 0 && warp == 0 && err_slot >= 0) {
-      // Fourier error of the iterate entering this iteration, summed in a
-      // fixed order over the cluster's warps (the partials stay put until
-      // every CTA has passed the barrier below)
-      double s = 0.0;
-      for (int q = lane; q < F::C * F::NW; q += 32)
-        s += dsm_ld_f64(dsm_map(smem_u32(red + q % F::NW), (uint32_t)(q / F::NW)));
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      // the raw sum; the square root and division wait until the last
-      // iteration (not in the short chains of kPublishAtOnce)
-      if (lane == 0)
-        J->err_hist[(size_t)(err_slot + it) * Np + n] =
-            kPublishAtOnce<N, Q> ? publish_error(s, J->Cn[n], J->sumA2[n], J->status, n) : s;
-    }
-    cluster_arrive();
-    if (fwd) load_av(0, av);  // in flight across the barrier
-    cluster_wait();
-  }
-  if (!kPublishAtOnce<N, Q> && rank == 0 && warp == 0 && err_slot >= 0) {
-    __syncwarp();
-    for (int it = lane; it < n_iters; it += 32) {
-      double* e = J->err_hist + (size_t)(err_slot + it) * Np + n;
-      *e = publish_error(__ldcg(e), J->Cn[n], J->sumA2[n], J->status, n);
+    if (!publish_at_once<N, Q>() && rank == 0 && warp == 0 && err_slot >= 0) {
+      __syncwarp();
+      for (int it = lane; it < n_iters; it += 32) {
+        double* e = J->err_hist + (size_t)(err_slot + it) * Np + n;
+        *e = publish_error(__ldcg(e), J->Cn[n], J->sumA2[n], J->status, n);
+      }
     }
   }
 }
-
 
 // ---------------------------------------------------------------- host side
 template <int N, int Q>
@@ -449,11 +458,11 @@ static cudaLaunchConfig_t fused_config(int ntiles, cudaLaunchAttribute* at, cuda
 }
 
 // attributes of both instances; *clusters: resident clusters of this shape
-template <int N, int Q>
+template <int N, int Q, bool SWEEP = false>
 static cudaError_t fused_attrs(int* clusters) {
   using F = FusedCfg<N, Q>;
   cudaError_t e = cudaSuccess;
-  for (auto kernel : {k_fused<N, false, Q>, k_fused<N, true, Q>}) {
+  for (auto kernel : {k_fused<N, false, Q, SWEEP>, k_fused<N, true, Q, SWEEP>}) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F::SMEM);
     if (e == cudaSuccess && F::C > 8)
@@ -462,7 +471,7 @@ static cudaError_t fused_attrs(int* clusters) {
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at;
   cudaLaunchConfig_t cfg = fused_config<N, Q>(1, &at, nullptr);
-  e = cudaOccupancyMaxActiveClusters(clusters, k_fused<N, false, Q>, &cfg);
+  e = cudaOccupancyMaxActiveClusters(clusters, k_fused<N, false, Q, SWEEP>, &cfg);
   return e == cudaSuccess && *clusters < 1 ? cudaErrorNotSupported : e;
 }
 
@@ -513,6 +522,51 @@ static cudaError_t fused_launch(const Launch& L) {
   const cudaLaunchConfig_t cfg = fused_config<N, 2>(L.ntiles, &at, L.stream);
   if (L.masked) return cudaLaunchKernelEx(&cfg, k_fused<N, true, 2>, L.js, L.st, L.tiles);
   return cudaLaunchKernelEx(&cfg, k_fused<N, false, 2>, L.js, L.st, L.tiles);
+}
+
+// The sweep form: one task a warp while the members fit that way (a chain is
+// as long as its angle), else two.
+template <int N>
+static int sweep_wide() {  // members that fit with one task a warp, 0: no sweep form here
+  static const int wide = [] {
+    int one = 0, two = 0;
+    if (fused_attrs<N, 2, true>(&two) != cudaSuccess || fused_attrs<N, 1, true>(&one) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return one;
+  }();
+  return wide;
+}
+
+template <int N, int Q>
+static cudaError_t fused_sweep_go(const Launch& L) {
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = fused_config<N, Q>(L.ntiles, &at, L.stream);
+  g_launches += 1;
+  if (L.masked) return cudaLaunchKernelEx(&cfg, k_fused<N, true, Q, true>, L.js, L.st, L.tiles);
+  return cudaLaunchKernelEx(&cfg, k_fused<N, false, Q, true>, L.js, L.st, L.tiles);
+}
+
+bool fused_sweep_supported(int N) {
+  switch (N) {
+    case 64: return sweep_wide<64>() > 0;
+    case 128: return sweep_wide<128>() > 0;
+    case 256: return sweep_wide<256>() > 0;
+    default: return false;
+  }
+}
+
+cudaError_t launch_fused_sweep(const Launch& L) {
+#define CPRA_CASE(NN) \
+  case NN: return L.ntiles <= sweep_wide<NN>() ? fused_sweep_go<NN, 1>(L) : fused_sweep_go<NN, 2>(L);
+  switch (L.N) {
+    CPRA_CASE(64)
+    CPRA_CASE(128)
+    CPRA_CASE(256)
+    default: return cudaErrorInvalidValue;
+  }
+#undef CPRA_CASE
 }
 
 #define CPRA_FOR_EACH_FUSED_N(X) X(64) X(128) X(256) X(512)

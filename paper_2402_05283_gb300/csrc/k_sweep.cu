@@ -333,6 +333,7 @@ cudaError_t sweep_launch(const Launch& L) {
 #define CPRA_FOR_EACH_SWEEP_N(X) X(16) X(32) X(48) X(96) X(160) X(320)
 
 bool sweep_supported(int N, int engine) {
+  if (engine == CPRA_ENGINE_FUSED) return fused_sweep_supported(N);
   if (engine != CPRA_ENGINE_TWO_PASS) return false;
   switch (N) {
 #define CPRA_CASE(NN) \
@@ -345,6 +346,7 @@ bool sweep_supported(int N, int engine) {
 }
 
 cudaError_t launch_sweep(const Launch& L) {
+  if (L.engine == CPRA_ENGINE_FUSED) return launch_fused_sweep(L);
   switch (L.N) {
 #define CPRA_CASE(NN) \
   case NN: return sweep_launch<NN>(L);

@@ -9,15 +9,16 @@ from test_gpu_parity import TOL, _rel, cp  # noqa: F401
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N", [16, 32, 48, 96, 160, 320])
-def test_one_angle_equals_the_block_wide_passes(cp, N):  # noqa: F811
+@pytest.mark.parametrize("N,engine", [(16, 1), (32, 1), (48, 1), (96, 1), (160, 1), (320, 1),
+                                      (64, 2), (128, 2), (256, 2)])
+def test_one_angle_equals_the_jacobi_episode(cp, N, engine):  # noqa: F811
     """A carousel of one angle has no order, so a sweep of it is the Jacobi
-    episode: the sweep kernel against the block-wide passes, bit for bit,
-    across the RAAR -> ER switch inside an episode."""
+    episode: the sweep kernels against the block-wide passes (1) and the fused
+    engine (2), bit for bit, across the RAAR -> ER switch inside an episode."""
     d = synth.make_case("tiny", N=N, Np=1)
     out = []
     for sweep in (0, 1):
-        p = cp.Plan(cp.make_config(N, 1, n_ei=3, seed=4, hio_iters=4, er_iters=2, engine=cp.ENGINE_TWO_PASS,
+        p = cp.Plan(cp.make_config(N, 1, n_ei=3, seed=4, hio_iters=4, er_iters=2, engine=engine,
                                    update=cp.UPDATE_RAAR, wrap_mode=cp.WRAP_MIRROR, sweep=sweep))
         p.load_intensities(d["I"], 0, d["thetas"])
         p.load_support(d["support"])
@@ -28,9 +29,9 @@ def test_one_angle_equals_the_block_wide_passes(cp, N):  # noqa: F811
     np.testing.assert_allclose(out[0][1], out[1][1], rtol=1e-5)  # FP32 partial sums of other threads
 
 
-@pytest.mark.parametrize("N,engine", [(32, "AUTO"), (96, "AUTO"), (160, "AUTO"), (320, "AUTO")])
+@pytest.mark.parametrize("N", [32, 64, 96, 128, 160, 256, 320])
 @pytest.mark.parametrize("objt", [0, 1])
-def test_sweep_against_the_oracle(cp, N, engine, objt):  # noqa: F811
+def test_sweep_against_the_oracle(cp, N, objt):  # noqa: F811
     """Two ER sweeps of five angles, five taps, MIRROR seam; a batch of an
     uneven pair of guesses (5 and 3 angles) ends where each ends alone."""
     d = synth.make_case("tiny", N=N, Np=5)
