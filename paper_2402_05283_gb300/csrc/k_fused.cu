@@ -10,7 +10,7 @@
 // cluster's distributed shared memory.  CTA r keeps packed columns
 // [CW r, CW (r + 1)) of all N rows (its slab; CW = 32, or 16 at N = 512)
 // and does the row work of image rows [2 CW r, 2 CW (r + 1)):
-//   column phase  local to the CTA: its CW columns, two tasks per warp;
+//   column phase  local to the CTA: its CW columns, one or two tasks a warp;
 //   row phase     each row pair gathered from the C slabs over DSMEM,
 //                 inverted, updated against g in global memory, transformed
 //                 again and scattered back to the same slab places.
