@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <fstream>
+#include <initializer_list>
 #include <new>
 #include <sstream>
 #include <string>
@@ -87,6 +88,26 @@ void dev_free(cpra_plan_s* p, void* ptr) {
     }
   if (p->cfg.free) p->cfg.free(ptr, p->cfg.alloc_ctx);
   else if (!p->cfg.alloc) cudaFree(ptr);
+}
+
+// Buffers that one step needs together: every one is allocated, or (out of
+// memory) none is kept and every pointer is NULL, so that a later call with
+// memory free starts over instead of finding part of them.
+struct Want {
+  void** ptr;
+  size_t bytes;
+};
+template <class T>
+Want want(T*& ptr, size_t bytes) { return {(void**)&ptr, bytes}; }
+bool alloc_all(cpra_plan_s* p, std::initializer_list<Want> list) {
+  bool ok = true;
+  for (const Want& w : list) ok = (*w.ptr = ok ? dev_alloc(p, w.bytes) : nullptr) != nullptr;
+  if (!ok)
+    for (const Want& w : list) {
+      dev_free(p, *w.ptr);
+      *w.ptr = nullptr;
+    }
+  return ok;
 }
 
 struct Sizes {
@@ -465,6 +486,7 @@ cpra_status build_gridding(cpra_plan_s* p) {
   }
   Assembly& a = p->asmb;
   if (a.ents && a.n_ent < n_ent) {
+    CK(cudaStreamSynchronize(p->stream), "grid sync");  // an assembly queued before may still read them
     dev_free(p, a.ents);
     a.ents = nullptr;
   }
@@ -1122,17 +1144,10 @@ static cpra_status iterate_core(cpra_plan_s* p, int32_t n_iters, double* err_out
 static cpra_status ensure_assembly(cpra_plan_s* p) {
   const size_t N = p->N, Np = p->Np, NN = N * N;
   Assembly& a = p->asmb;
-  if (!a.F) {
-    a.F = (float2*)dev_alloc(p, spectra_bytes(p->N, p->Np));
-    a.corr = (float2*)dev_alloc(p, corr_bytes(p->N, p->Np));
-    a.Q = (float2*)dev_alloc(p, NN * 8);
-    a.ramps = (float2*)dev_alloc(p, ramps_bytes(p->N, p->Np));
-    a.vol = (float2*)dev_alloc(p, N * NN * 8);
-    a.cell_ptr = (int32_t*)dev_alloc(p, (NN + 1) * 4);
-    a.moments = (double*)dev_alloc(p, 3 * Np * 8);
-    if (!a.F || !a.corr || !a.Q || !a.ramps || !a.vol || !a.cell_ptr || !a.moments)
-      return fail(p, CPRA_ERR_OUT_OF_MEMORY, "assembly allocation failed");
-  }
+  if (!a.F && !alloc_all(p, {want(a.F, spectra_bytes(p->N, p->Np)), want(a.corr, corr_bytes(p->N, p->Np)),
+                             want(a.Q, NN * 8), want(a.ramps, ramps_bytes(p->N, p->Np)), want(a.vol, N * NN * 8),
+                             want(a.cell_ptr, (NN + 1) * 4), want(a.moments, 3 * Np * 8)}))
+    return fail(p, CPRA_ERR_OUT_OF_MEMORY, "assembly allocation failed");
   if (!a.grid_ok) return build_gridding(p);
   return CPRA_OK;
 }
@@ -1206,11 +1221,8 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
   cpra_status st = ensure_assembly(p);
   if (st != CPRA_OK) return st;
   const size_t NN = (size_t)N * N;
-  if (!p->mg_acc) {
-    p->mg_acc = (float2*)dev_alloc(p, Np * NN * 8);
-    p->mg_ref = (float2*)dev_alloc(p, NN * 8);
-    if (!p->mg_acc || !p->mg_ref) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
-  }
+  if (!p->mg_acc && !alloc_all(p, {want(p->mg_acc, Np * NN * 8), want(p->mg_ref, NN * 8)}))
+    return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
   if (prtf && !p->mg_rings) {
     p->mg_rings = (double*)dev_alloc(p, sizeof(double) * Np * (N / 2) + sizeof(unsigned) * (N / 2));
     if (!p->mg_rings) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
@@ -1220,10 +1232,9 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
     dev_free(p, p->mg_dist);
     dev_free(p, p->mg_ramps);
     p->mg_cap = 0;
-    p->mg_guess = (MergeGuess*)dev_alloc(p, sizeof(MergeGuess) * n_l);
-    p->mg_dist = (double*)dev_alloc(p, sizeof(double) * 2 * n_l);
-    p->mg_ramps = (float2*)dev_alloc(p, ramps_bytes(N, Np) * n_l);
-    if (!p->mg_guess || !p->mg_dist || !p->mg_ramps) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
+    if (!alloc_all(p, {want(p->mg_guess, sizeof(MergeGuess) * n_l), want(p->mg_dist, sizeof(double) * 2 * n_l),
+                       want(p->mg_ramps, ramps_bytes(N, Np) * n_l)}))
+      return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
     p->mg_cap = n_l;
   }
   p->merged = false;
@@ -1304,24 +1315,16 @@ cpra_status cpra_refine_3d(cpra_plan_t p, int32_t n_iters, int32_t shrink_every,
     return fail(p, CPRA_ERR_NOT_READY, "no Step D volume: cpra_assemble_3d or cpra_merge first");
   const int N = p->N, Np = p->Np, W3 = (N + 31) / 32;
   const size_t NN = (size_t)N * N, N3 = NN * N;
-  if (!p->rf_X) {
-    p->rf_X = (float2*)dev_alloc(p, N3 * 8);
-    p->rf_W = (float2*)dev_alloc(p, N3 * 8);
-    p->rf_konst = (double*)dev_alloc(p, 2 * sizeof(double));
-    p->rf_R = (float*)dev_alloc(p, N3 * 4);
-    p->rf_B = (float*)dev_alloc(p, N3 * 4);
-    p->rf_S3 = (uint32_t*)dev_alloc(p, NN * W3 * 4);
-    p->rf_M = (uint8_t*)dev_alloc(p, NN);
-    p->rf_cs = (double2*)dev_alloc(p, sizeof(double2) * Np);
-    p->rf_taps = (float*)dev_alloc(p, sizeof(float) * N);
-    p->rf_max = (unsigned*)dev_alloc(p, sizeof(unsigned));
-    p->rf_shift = (int2*)dev_alloc(p, sizeof(int2) * Np);
-    if (!p->rf_X || !p->rf_W || !p->rf_konst || !p->rf_R || !p->rf_B || !p->rf_S3 || !p->rf_M || !p->rf_cs ||
-        !p->rf_taps || !p->rf_max || !p->rf_shift)
-      return fail(p, CPRA_ERR_OUT_OF_MEMORY, "refinement allocation failed");
-  }
+  if (!p->rf_X &&
+      !alloc_all(p, {want(p->rf_X, N3 * 8), want(p->rf_W, N3 * 8), want(p->rf_konst, 2 * sizeof(double)),
+                     want(p->rf_R, N3 * 4), want(p->rf_B, N3 * 4), want(p->rf_S3, NN * W3 * 4), want(p->rf_M, NN),
+                     want(p->rf_cs, sizeof(double2) * Np), want(p->rf_taps, sizeof(float) * N),
+                     want(p->rf_max, sizeof(unsigned)), want(p->rf_shift, sizeof(int2) * Np)}))
+    return fail(p, CPRA_ERR_OUT_OF_MEMORY, "refinement allocation failed");
   if (n_iters > p->rf_err_cap) {
+    CK(cudaStreamSynchronize(p->stream), "refine sync");  // iterations of an earlier call may still write the sums
     dev_free(p, p->rf_err);
+    p->rf_err_cap = 0;
     p->rf_err = (double*)dev_alloc(p, sizeof(double) * 2 * n_iters);
     if (!p->rf_err) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "refinement allocation failed");
     p->rf_err_cap = n_iters;
