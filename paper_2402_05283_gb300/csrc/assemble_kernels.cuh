@@ -516,19 +516,11 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
 }
 
 // ------------------------------------------------------------------ launchers
-template <class K>
-static cudaError_t smem_once(K kernel, size_t bytes, bool& done) {
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) done = true;
-  return e;
-}
-
 template <int N, int MODE>
 static cudaError_t spectra_n(const float2* Hp, const float2* ramps, float2* F, float2* corr, const float2* xtw,
                              const MergeArgs& ma, int count, cudaStream_t st) {
   using C = ColW<N, kPrecFP32>;
-  static bool attr = false;
+  static PerDevice<bool> attr;
   cudaError_t e = smem_once(k_spectra<N, MODE>, spec_smem<N>(), attr);
   if (e != cudaSuccess) return e;
   g_launches += 1;
@@ -541,7 +533,7 @@ template <int N>
 static cudaError_t grid_n(cpra_plan_s* p, float2* out) {
   using G = GridCfg<N>;
   Assembly& a = p->asmb;
-  static bool attr = false;
+  static PerDevice<bool> attr;
   cudaError_t e = smem_once(k_grid<N>, G::SMEM, attr);
   if (e == cudaSuccess) e = launch_grid_corr(p);
   if (e != cudaSuccess) return e;
@@ -576,7 +568,7 @@ cudaError_t merge_n(cpra_plan_s* d, const MergeArgs& ma, int n_l, float2* acc, d
                            float* prtf) {
   using C = ColW<N, kPrecFP32>;
   cudaStream_t st = d->stream;
-  static bool attr = false;
+  static PerDevice<bool> attr;
   cudaError_t e = smem_once(k_merge<N>, spec_smem<N>(), attr);
   const size_t total = (size_t)d->Np * (N / 2);
   unsigned* counts = reinterpret_cast<unsigned*>(rings + total);

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "cpra.h"
+#include "per_device.h"
 
 namespace cpra {
 
@@ -298,6 +299,30 @@ cudaError_t launch_prime(const Launch& L);
 cudaError_t launch_colpass(const Launch& L);
 cudaError_t launch_rowpass(const Launch& L);
 cudaError_t launch_shrinkwrap(cpra_plan_s* p);
+
+// the value of the current device (the one that the caller's stream and buffers
+// are on)
+template <class T, class F>
+cudaError_t on_device(PerDevice<T>& facts, T& v, F&& make) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e == cudaSuccess ? facts.get(dev, v, make) : e;
+}
+// make() once on each device
+template <class F>
+cudaError_t once_on_device(PerDevice<bool>& done, F&& make) {
+  bool v;
+  return on_device(done, v, [&](bool&) { return make(); });
+}
+// opt-in to more than 48 KB of dynamic shared memory
+template <class K>
+cudaError_t smem_attr(K kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+template <class K>
+cudaError_t smem_once(K kernel, size_t bytes, PerDevice<bool>& done) {
+  return once_on_device(done, [&] { return smem_attr(kernel, bytes); });
+}
 
 // assembly (k_assemble.cu)
 // spectra, grid and volume from Hp and the ramps (launch_rho_rows); out: NULL,

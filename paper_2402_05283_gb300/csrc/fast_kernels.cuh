@@ -869,15 +869,8 @@ k_persist_w(const PersistArgs a) {
 }
 
 // ---------------------------------------------------------------- launchers
-template <class K>
-static cudaError_t smem_attr(K kernel, size_t bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 template <int N, int PREC>
-cudaError_t prepare_w() {
-  static bool done = false;
-  if (done) return cudaSuccess;
+cudaError_t prepare_device_w() {
   cudaError_t e = smem_attr(k_rowpass_w<N, PREC>, row_smem<N, PREC>());
   if (e == cudaSuccess) e = smem_attr(k_prime_w<N, PREC>, prime_smem<N, PREC>());
   if constexpr (PREC == kPrecFP32)
@@ -903,8 +896,13 @@ cudaError_t prepare_w() {
     if (e == cudaSuccess) e = fits(k_colpass_w<N, PREC, false>, ColW<N, PREC>::NT, col_smem<N, PREC>(), col_cols);
     if (e == cudaSuccess) e = fits(k_colpass_w<N, PREC, true>, ColW<N, PREC>::NT, col_smem<N, PREC>(), col_cols);
   }
-  if (e == cudaSuccess) done = true;
   return e;
+}
+
+template <int N, int PREC>
+cudaError_t prepare_w() {
+  static PerDevice<bool> done;
+  return once_on_device(done, prepare_device_w<N, PREC>);
 }
 
 template <int N, int PREC>

@@ -478,27 +478,24 @@ static cudaError_t fused_attrs(int* clusters) {
 // N = 512 has one instance: its two tasks a warp fill the SM with 16 warps
 template <int N> constexpr bool kFusedWide = N <= 256;
 
-// looked up once per process and size: a cluster of C CTAs with this much
-// shared memory must fit on the device; *wide: clusters of the one-task form
-// that are resident at a time
+// a cluster of C CTAs with this much shared memory must fit on the current
+// device; *wide: clusters of the one-task form that are resident at a time
 template <int N>
 static cudaError_t fused_prepare(int* wide) {
-  struct Ready {
-    cudaError_t e;
-    int wide = 0;
-    Ready() {
-      int c = 0;
-      e = fused_attrs<N, 2>(&c);
-      if constexpr (kFusedWide<N>)
-        if (e == cudaSuccess && fused_attrs<N, 1>(&wide) != cudaSuccess) {
-          cudaGetLastError();
-          wide = 0;
-        }
-    }
-  };
-  static const Ready r;
-  if (wide) *wide = r.wide;
-  return r.e;
+  static PerDevice<int> resident;
+  int one = 0;
+  const cudaError_t e = on_device(resident, one, [](int& n) {
+    int c = 0;
+    const cudaError_t r = fused_attrs<N, 2>(&c);
+    if constexpr (kFusedWide<N>)
+      if (r == cudaSuccess && fused_attrs<N, 1>(&n) != cudaSuccess) {
+        cudaGetLastError();
+        n = 0;
+      }
+    return r;
+  });
+  if (wide) *wide = one;
+  return e;
 }
 
 // One task a warp where all of the launch's clusters are resident at a time in
@@ -528,15 +525,16 @@ static cudaError_t fused_launch(const Launch& L) {
 // as long as its angle), else two.
 template <int N>
 static int sweep_wide() {  // members that fit with one task a warp, 0: no sweep form here
-  static const int wide = [] {
-    int one = 0, two = 0;
-    if (fused_attrs<N, 2, true>(&two) != cudaSuccess || fused_attrs<N, 1, true>(&one) != cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
-    return one;
-  }();
-  return wide;
+  static PerDevice<int> resident;
+  int one = 0;
+  const cudaError_t e = on_device(resident, one, [](int& n) {
+    int two = 0;
+    const cudaError_t r = fused_attrs<N, 2, true>(&two);
+    return r == cudaSuccess ? fused_attrs<N, 1, true>(&n) : r;
+  });
+  if (e == cudaSuccess) return one;
+  cudaGetLastError();
+  return 0;
 }
 
 template <int N, int Q>

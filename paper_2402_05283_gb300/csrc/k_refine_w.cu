@@ -458,25 +458,23 @@ k_rv(float2* X, const float2* __restrict__ Wd, const uint8_t* __restrict__ M, co
 }
 
 // ------------------------------------------------------------ launchers
-template <class K>
-cudaError_t attr_w(K kernel, size_t bytes) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+template <int N>
+cudaError_t refine_w_attrs() {
+  cudaError_t e = smem_attr(k_xw<N>, xw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_vw<N, false>, vw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_rx<N, kRFwd>, xw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_rx<N, kRInv>, xw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_rx<N, kRBoth>, xw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_rv<N, kLFwd>, vw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_rv<N, kLInv>, vw_smem<N>());
+  if (e == cudaSuccess) e = smem_attr(k_rv<N, kLConstrain>, vw_smem_c<N>());
+  return e;
 }
 
 template <int N>
 cudaError_t refine_w_prepare() {
-  static bool done = false;
-  if (done) return cudaSuccess;
-  cudaError_t e = attr_w(k_xw<N>, xw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_vw<N, false>, vw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_rx<N, kRFwd>, xw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_rx<N, kRInv>, xw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_rx<N, kRBoth>, xw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_rv<N, kLFwd>, vw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_rv<N, kLInv>, vw_smem<N>());
-  if (e == cudaSuccess) e = attr_w(k_rv<N, kLConstrain>, vw_smem_c<N>());
-  if (e == cudaSuccess) done = true;
-  return e;
+  static PerDevice<bool> done;
+  return once_on_device(done, refine_w_attrs<N>);
 }
 
 // V = FFT3(X) in place (X: the data volume), then W and the constant sums
@@ -532,12 +530,9 @@ cudaError_t iter_w(const RefineArgs& a, double* err2, bool first, bool last, cud
 template <int N>
 cudaError_t volume_ylines_n(float2* vol, float2* out, const float2* xtw, cudaStream_t st) {
   using C = VW<N>;
-  static bool done = false;
-  if (!done) {
-    cudaError_t e = attr_w(k_vw<N, true>, vw_smem<N>());
-    if (e != cudaSuccess) return e;
-    done = true;
-  }
+  static PerDevice<bool> attr;
+  const cudaError_t e = smem_once(k_vw<N, true>, vw_smem<N>(), attr);
+  if (e != cudaSuccess) return e;
   g_launches += 1;
   k_vw<N, true><<<dim3(N / C::CB, N), C::NT, vw_smem<N>(), st>>>(vol, out, xtw, (size_t)N * N, (size_t)N);
   return cudaGetLastError();

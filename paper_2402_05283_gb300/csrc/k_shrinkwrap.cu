@@ -347,11 +347,10 @@ template <int CW>
 static cudaError_t blur_cols_go(dim3 grid, size_t smem, const float* in, float* out, const float* taps,
                                 int ntaps, int lo, int N, size_t outer, size_t estride, unsigned* mx,
                                 int per_plane, cudaStream_t st) {
-  static bool big = false;  // the opt-in to more than 48 KB, once
-  if (smem > 48 * 1024 && !big) {
-    cudaError_t e = cudaFuncSetAttribute(k_blur_cols<CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  static PerDevice<bool> big;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = smem_once(k_blur_cols<CW>, 200 * 1024, big);
     if (e != cudaSuccess) return e;
-    big = true;
   }
   k_blur_cols<CW><<<grid, 256, smem, st>>>(in, out, taps, ntaps, lo, N, outer, estride, mx, per_plane);
   return cudaGetLastError();
@@ -451,7 +450,7 @@ cudaError_t static_scratch(StaticScratch& out) {
 
 // device memory of the current device (the kernels run there, with that
 // device's scratch), or managed memory
-bool on_device(const void* ptr, int dev) {
+bool memory_of(const void* ptr, int dev) {
   cudaPointerAttributes a;
   if (!ptr || cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
     cudaGetLastError();
@@ -490,7 +489,7 @@ extern "C" cpra_status cpra_shrinkwrap_static(const float* g, const uint8_t* S_i
     cudaGetLastError();
     return record_error(CPRA_ERR_CUDA, "no current device");
   }
-  if (!on_device(g, dev) || !on_device(S_in, dev) || !on_device(S_out, dev))
+  if (!memory_of(g, dev) || !memory_of(S_in, dev) || !memory_of(S_out, dev))
     return record_error(CPRA_ERR_INVALID_ARG,
                         "g, S_in and S_out must be device memory of the current device");
   StaticScratch sc;

@@ -298,25 +298,19 @@ cudaLaunchConfig_t sweep_config(int members, cudaLaunchAttribute* at, cudaStream
   return cfg;
 }
 
-// the device holds a cluster of this size (looked up once)
+// the current device holds a cluster of this size
 template <int N>
 bool sweep_ready() {
-  static const bool ok = [] {
-    if (cudaFuncSetAttribute(k_sweep<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SweepCfg<N>::SMEM) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
+  static PerDevice<int> resident;
+  int clusters = 0;
+  const cudaError_t e = on_device(resident, clusters, [](int& n) {
+    cudaError_t r = smem_attr(k_sweep<N>, SweepCfg<N>::SMEM);
     cudaLaunchAttribute at;
-    cudaLaunchConfig_t cfg = sweep_config<N>(1, &at, nullptr);
-    int clusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&clusters, k_sweep<N>, &cfg) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    return clusters >= 1;
-  }();
-  return ok;
+    const cudaLaunchConfig_t cfg = sweep_config<N>(1, &at, nullptr);
+    return r == cudaSuccess ? cudaOccupancyMaxActiveClusters(&n, k_sweep<N>, &cfg) : r;
+  });
+  if (e != cudaSuccess) cudaGetLastError();
+  return e == cudaSuccess && clusters >= 1;
 }
 
 template <int N>

@@ -225,14 +225,6 @@ k_rowpass(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
 }
 
 // ---------------------------------------------------------------- launchers
-template <class K>
-static cudaError_t set_smem_once(K kernel, size_t bytes, bool& done) {
-  if (done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) done = true;
-  return e;
-}
-
 template <int N>
 static cudaError_t prepare_n();
 
@@ -271,11 +263,13 @@ static cudaError_t rowpass_n(const Launch& L) {
 
 template <int N>
 static cudaError_t prepare_n() {
-  static bool a1 = false, a2 = false, a3 = false;
-  cudaError_t e = set_smem_once(k_prime<N>, sizeof(float2) * (N + RowTile<N>::SMEM_LINES), a1);
-  if (e == cudaSuccess) e = set_smem_once(k_colpass<N>, sizeof(float2) * (N + ColTile<N>::SMEM_LINES), a2);
-  if (e == cudaSuccess) e = set_smem_once(k_rowpass<N>, sizeof(float2) * (N + RowTile<N>::SMEM_LINES), a3);
-  return e;
+  static PerDevice<bool> done;
+  return once_on_device(done, [] {
+    cudaError_t e = smem_attr(k_prime<N>, sizeof(float2) * (N + RowTile<N>::SMEM_LINES));
+    if (e == cudaSuccess) e = smem_attr(k_colpass<N>, sizeof(float2) * (N + ColTile<N>::SMEM_LINES));
+    if (e == cudaSuccess) e = smem_attr(k_rowpass<N>, sizeof(float2) * (N + RowTile<N>::SMEM_LINES));
+    return e;
+  });
 }
 
 cudaError_t prepare_kernels(int N, int engine, int prec) {
