@@ -126,7 +126,9 @@ Sizes plan_sizes(const cpra_config& c) {
            + Np * NN * 4        // staging
            + 256 * Np * 8;      // initial error history
   if (c.shrinkwrap_every > 0) s.iter += Np * NN * 4 + Np * 4 + N * 4;
-  s.assemble = Np * NN * 8 + N * NN * 8 + (NN + 1) * 4 + 4 * Np * N * 12 + 3 * Np * 8;
+  // what ensure_assembly allocates; a sample has at most four cells
+  s.assemble = spectra_bytes(c.N, c.Np) + corr_bytes(c.N, c.Np) + ramps_bytes(c.N, c.Np) +
+               NN * 8 + N * NN * 8 + (NN + 1) * 4 + 3 * Np * 8 + 4 * Np * N * sizeof(GridEnt);
   return s;
 }
 
