@@ -122,7 +122,7 @@ Sizes plan_sizes(const cpra_config& c) {
            + Np * N * (N / 2) * 4 + Np * N * 4  // A_main, A_nyq
            + 3 * Np * 8         // Cn, sumA2, err_acc
            + Np * N * W * 4     // S
-           + 2 * N * 8          // twiddles
+           + 3 * N * 8          // twiddles
            + Np * NN * 4        // staging
            + 256 * Np * 8;      // initial error history
   if (c.shrinkwrap_every > 0) s.iter += Np * NN * 4 + Np * 4 + N * 4;
@@ -721,7 +721,7 @@ cpra_status cpra_plan(const cpra_config* cfg, void* stream, cpra_plan_t* out) {
   p->err_acc = (double*)A(Np * 8);
   p->S = (uint32_t*)A(Np * N * p->W * 4);
   p->tw = (float2*)A(N * 8);
-  p->xtw = (float2*)A(N * 8);
+  p->xtw = (float2*)A(2 * N * 8);
   p->stage = (float*)A(Np * NN * 4);
   p->bad = (uint8_t*)A(Np);
   p->d_js = (JobStatic*)A(sizeof(JobStatic));
@@ -758,18 +758,21 @@ cpra_status cpra_plan(const cpra_config* cfg, void* stream, cpra_plan_t* out) {
     const double a = -2.0 * M_PI * (double)k / (double)N;
     tw[k] = make_float2((float)std::cos(a), (float)std::sin(a));
   }
-  // cross twiddles of the warp FFT, [k1][l] = exp(-2 pi i (l k1 mod N) / N), FP64 then FP32
-  std::vector<float2> xtw(N, make_float2(1.0f, 0.0f));
+  // cross twiddles of the warp FFT, [k1][l] = exp(-2 pi i (l k1 mod N) / N), FP64
+  // and rounded once, then the low parts that the rounding left (refinement)
+  std::vector<float2> xtw(2 * N, make_float2(0.0f, 0.0f));
   int E1 = 0, E2 = 0;
   if (fast_dims(p->N, &E1, &E2))
     for (int k1 = 0; k1 < E1; ++k1)
       for (int l = 0; l < E2; ++l) {
         const double a = -2.0 * M_PI * (double)((l * k1) % p->N) / (double)N;
-        xtw[k1 * E2 + l] = make_float2((float)std::cos(a), (float)std::sin(a));
+        const double c = std::cos(a), s = std::sin(a);
+        const float2 w = xtw[k1 * E2 + l] = make_float2((float)c, (float)s);
+        xtw[N + k1 * E2 + l] = make_float2((float)(c - w.x), (float)(s - w.y));
       }
   cudaError_t e = cudaMemcpyAsync(p->tw, tw.data(), N * 8, cudaMemcpyHostToDevice, p->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(p->xtw, xtw.data(), N * 8, cudaMemcpyHostToDevice, p->stream);
+    e = cudaMemcpyAsync(p->xtw, xtw.data(), 2 * N * 8, cudaMemcpyHostToDevice, p->stream);
   std::vector<uint16_t> tcw;
   if (cfg->precision != CPRA_FP32) {
     // block DFT matrices [[Re W, Im W], [-Im W, Re W]] of the E1- and

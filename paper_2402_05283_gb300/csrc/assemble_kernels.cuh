@@ -80,7 +80,7 @@ template <int N, class FL, class Only>
 __device__ __forceinline__ void store_f(const float2 (&a)[FL::TA][FL::E1], float2* F, int n, int Np,
                                         int c, int lane, Only&& only) {
   constexpr int H = N / 2;
-  const float inv = 1.0f / N;
+  constexpr Const<FL::ACC> inv(1.0 / N);
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
@@ -89,13 +89,13 @@ __device__ __forceinline__ void store_f(const float2 (&a)[FL::TA][FL::E1], float
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
       const int z = FL::a_x(t, m);
-      F[f_at(z < H ? z + H : z - H, n, c + line, Np, H + 1)] = cscale(a[i][m], inv);
+      F[f_at(z < H ? z + H : z - H, n, c + line, Np, H + 1)] = inv.mul(a[i][m]);
     });
   });
 }
 
 template <int N>
-constexpr size_t spec_smem() { return sizeof(float2) * (3 * N + ColW<N, kPrecFP32>::BUF); }
+constexpr size_t spec_smem() { return sizeof(float2) * (VolLines<N>::XN + 2 * N + ColW<N, kPrecFP32>::BUF); }
 
 // What the spectra kernel makes of a block of columns: F (one guess, all
 // angles: blockIdx.y = angle), REF or DIST (one angle n0 of guess blockIdx.y)
@@ -104,11 +104,11 @@ __global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, ColW<N, kPrecFP32>::MI
 k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float2* F, float2* corr,
           const float2* __restrict__ xtw, const MergeArgs ma) {
   using C = ColW<N, kPrecFP32>;
-  using FL = typename C::FL;
+  using FL = VolLines<N>;
   constexpr int H = N / 2;
   extern __shared__ float2 smem[];
   float2* xs = smem;
-  float2* rz = xs + N;
+  float2* rz = xs + FL::XN;
   float2* z0 = rz + N;  // the packed column 0 after its forward transform
   float2* buf = z0 + N;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -124,6 +124,7 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
   const float2* ru = rn + N;
   for (int i = threadIdx.x; i < N; i += C::NT) {
     xs[i] = xtw[i];
+    if constexpr (FL::XN > N) xs[N + i] = xtw[N + i];
     rz[i] = rn[i];
   }
   float2 a[FL::TA][FL::E1], b[FL::TB][FL::E2];
@@ -221,11 +222,11 @@ __global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, ColW<N, kPrecFP32>::NT
 k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* counts, float2* F,
         float2* corr, const float2* __restrict__ xtw) {
   using C = ColW<N, kPrecFP32>;
-  using FL = typename C::FL;
+  using FL = VolLines<N>;
   constexpr int H = N / 2;
   extern __shared__ float2 smem[];
   float2* xs = smem;
-  float2* rz = xs + N;
+  float2* rz = xs + FL::XN;
   float2* z0 = rz + N;
   float2* buf = z0 + N;
   __shared__ float2 sh[C::CB];  // mean of the partner row kz = -N/2 of the block's columns
@@ -238,7 +239,7 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
   const SpecCols<N> cols;
   const float scale = 1.0f / (float)n_l;
   const bool packed = c0 == 0 && warp == 0;
-  for (int i = threadIdx.x; i < N; i += C::NT) xs[i] = xtw[i];
+  for (int i = threadIdx.x; i < FL::XN; i += C::NT) xs[i] = xtw[i];
   for (int i = threadIdx.x; i < H; i += C::NT) {
     ring[i] = 0.0f;
     cnt[i] = 0u;
@@ -368,14 +369,14 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
 constexpr int kHeavy = 32;
 constexpr int kStaged = 2560;  // samples of a row held in shared memory (else read from L2)
 template <int N> struct GridCfg {
-  using FL = typename WLines<N, kPrecFP32>::type;
+  using FL = VolLines<N>;
   static constexpr int L = FL::L, H = N / 2, HC = H + 1;
   static constexpr int NZC = (N + 7) / 8;  // chunks of eight planes
   // pitch of a line: at least N, room for the warp's tile, 2 mod 8 (the four
   // plane pairs of a quad then start four banks apart)
   static constexpr int P0 = (FL::TSIZE + L - 1) / L > N ? (FL::TSIZE + L - 1) / L : N;
   static constexpr int LP = (P0 + 5) / 8 * 8 + 2;
-  static constexpr size_t SMEM = sizeof(float2) * (N + 8 * L * LP + kStaged) + sizeof(int) * (N + 4);
+  static constexpr size_t SMEM = sizeof(float2) * (FL::XN + 8 * L * LP + kStaged) + sizeof(int) * (N + 4);
   static_assert(LP >= P0 && LP % 8 == 2, "line pitch");
 };
 
@@ -414,7 +415,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
   constexpr int L = G::L, LP = G::LP;
   extern __shared__ __align__(16) float2 smem[];
   float2* xs = smem;
-  float2* lines = smem + N;  // [8 L][LP]
+  float2* lines = smem + FL::XN;  // [8 L][LP]
   GridEnt* es = reinterpret_cast<GridEnt*>(lines + 8 * L * LP);
   int* ptr = reinterpret_cast<int*>(es + kStaged);  // [N + 1]
   __shared__ unsigned short heavy[N];
@@ -430,7 +431,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
   if (staged)
     for (int i = threadIdx.x; i < count; i += 256) cp_async8(es + i, ents + first + i);
   cp_async_commit();
-  for (int i = threadIdx.x; i < N; i += 256) xs[i] = xtw[i];
+  for (int i = threadIdx.x; i < FL::XN; i += 256) xs[i] = xtw[i];
   cp_async_wait_all();
   __syncthreads();
   auto put = [&](int x, int ch, const float4& s) {
@@ -501,7 +502,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
   });
   __syncwarp();
   FL::inv(b, a, T, xs, lane);
-  const float inv = 1.0f / N;
+  constexpr Const<FL::ACC> inv(1.0 / N);
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
@@ -510,7 +511,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
     float2* row = V + ((size_t)z * N + ky) * N;
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
-      row[FL::a_x(t, m)] = cscale(a[i][m], inv);
+      row[FL::a_x(t, m)] = inv.mul(a[i][m]);
     });
   });
 }

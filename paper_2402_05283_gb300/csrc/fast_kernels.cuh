@@ -26,6 +26,10 @@ namespace cpra {
 // plans.
 template <int N, int PREC> struct WLines { using type = WarpLines<N>; };
 template <> struct WLines<512, kPrecFP32> { using type = PairLines512; };
+// lines of the assembly and the merge
+template <int N>
+using VolLines = std::conditional_t<WP<N>::POW2, typename WLines<N, kPrecFP32>::type,
+                                    typename WLines<N, kPrecFP32>::type::Acc>;
 // the one-line plan holds 16 values a lane: small enough for 24 warps an SM
 template <class FL> constexpr bool kSlimLines = FL::L == 1 && FL::E1 <= 16 && FL::E2 <= 16;
 
@@ -106,8 +110,9 @@ template <int N, int PREC>
 constexpr size_t row_smem() {
   return RowW<N, PREC>::SMEM + TcSmem<N, PREC>::template bytes<RowW<N, PREC>::WARPS>();
 }
-template <int N, int PREC>
+template <int N, int PREC, bool MOM = false>
 constexpr size_t prime_smem() {
+  if (MOM && !WP<N>::POW2) return PrimeW<N, PREC>::SMEM + sizeof(float2) * N;
   return PrimeW<N, PREC>::SMEM + TcSmem<N, PREC>::template bytes<PrimeW<N, PREC>::WARPS>();
 }
 
@@ -437,7 +442,8 @@ __global__ void __launch_bounds__(PrimeW<N, PREC>::WARPS * 32, 3)
 k_prime_w(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
           const int2* __restrict__ tiles, double* moments) {
   using RW = PrimeW<N, PREC>;
-  using FL = typename RW::FL;
+  // (rows of rho: the lines of the assembly, with the tiles of the prime)
+  using FL = std::conditional_t<MOM && !WP<N>::POW2, typename RW::FL::Acc, typename RW::FL>;
   constexpr int H = N / 2;
   extern __shared__ float2 smem[];
   const int2 tl = tiles[blockIdx.y];
@@ -453,14 +459,14 @@ k_prime_w(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
   const CoupleArgs& ca = Z->ca;
   float2* xs = smem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* T = smem + N + warp * RW::WARP_F2;
+  float2* T = smem + FL::XN + warp * RW::WARP_F2;
   uint32_t tc_phase = 0;
-  const TcCtx tc = tc_setup<N, PREC, RW::WARPS>(reinterpret_cast<char*>(smem + N + RW::WARPS * RW::WARP_F2),
+  const TcCtx tc = tc_setup<N, PREC, RW::WARPS>(reinterpret_cast<char*>(smem + FL::XN + RW::WARPS * RW::WARP_F2),
                                                 J->tcw, J->status, &tc_phase);
   const int n = tl.y;
   const int pair0 = (blockIdx.x * RW::WARPS + warp) * FL::L;
   __shared__ TapTab tt;
-  load_xtw<N>(xs, xtw, RW::WARPS * 32);
+  load_xtw<FL::XN>(xs, xtw, RW::WARPS * 32);
   fill_taps<N>(tt, ca, g_src, Z->g_dst, S, n, Np, W, J->present);
   __syncthreads();
   float2 a[FL::TA][FL::E1];
@@ -874,7 +880,7 @@ cudaError_t prepare_device_w() {
   cudaError_t e = smem_attr(k_rowpass_w<N, PREC>, row_smem<N, PREC>());
   if (e == cudaSuccess) e = smem_attr(k_prime_w<N, PREC>, prime_smem<N, PREC>());
   if constexpr (PREC == kPrecFP32)
-    if (e == cudaSuccess) e = smem_attr(k_prime_w<N, PREC, true>, prime_smem<N, PREC>());
+    if (e == cudaSuccess) e = smem_attr(k_prime_w<N, PREC, true>, prime_smem<N, PREC, true>());
   if (e == cudaSuccess) e = smem_attr(k_colpass_w<N, PREC, false>, col_smem<N, PREC>());
   if (e == cudaSuccess) e = smem_attr(k_colpass_w<N, PREC, true>, col_smem<N, PREC>());
   if constexpr (PREC != kPrecFP32) {
@@ -927,7 +933,7 @@ cudaError_t prime_w(const Launch& L, double* moments) {
   g_launches += 1;
   if constexpr (PREC == kPrecFP32)
     if (moments) {
-      k_prime_w<N, PREC, true><<<grid, RW::WARPS * 32, smem, L.stream>>>(L.js, L.st, L.tiles, moments);
+      k_prime_w<N, PREC, true><<<grid, RW::WARPS * 32, prime_smem<N, PREC, true>(), L.stream>>>(L.js, L.st, L.tiles, moments);
       return cudaGetLastError();
     }
   k_prime_w<N, PREC><<<grid, RW::WARPS * 32, smem, L.stream>>>(L.js, L.st, L.tiles, nullptr);

@@ -28,6 +28,11 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
+// a * b for b as a pair of floats, b + bl
+__device__ __forceinline__ float2 cmul(float2 a, float2 b, float2 bl) {
+  return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, fmaf(a.x, bl.x, -a.y * bl.y))),
+                     fmaf(a.x, b.y, fmaf(a.y, b.x, fmaf(a.x, bl.y, a.y * bl.x))));
+}
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, make_float2(s, s)); }
 // multiply by -i (DIR = -1) or +i (DIR = +1)
@@ -85,10 +90,21 @@ __device__ __forceinline__ void static_for(F&& f) {
   }
 }
 
-// R-point DFT in registers, y_k = sum_r x_r exp(DIR * 2 pi i r k / R).
-template <int R, int DIR> struct Dft;
+// x * c + y for a constant c, rounded once or, ACC, with c as a pair of floats
+// (48 bits): c's own rounding is the same in every call, so where a transform
+// and its inverse run over the same values hundreds of times it adds up in
+// step, while the other roundings add up at random.
+template <bool ACC> struct Const {
+  float hi, lo;
+  constexpr Const(double c) : hi((float)c), lo((float)(c - (double)(float)c)) {}
+  __device__ __forceinline__ float mul(float x) const { return ACC ? fmaf(x, hi, x * lo) : x * hi; }
+  __device__ __forceinline__ float2 mul(float2 v) const { return make_float2(mul(v.x), mul(v.y)); }
+};
 
-template <int DIR> struct Dft<2, DIR> {
+// R-point DFT in registers, y_k = sum_r x_r exp(DIR * 2 pi i r k / R).
+template <int R, int DIR, bool ACC = false> struct Dft;
+
+template <int DIR, bool ACC> struct Dft<2, DIR, ACC> {
   static __device__ __forceinline__ void run(float2* v) {
     float2 a = v[0], b = v[1];
     v[0] = cadd(a, b);
@@ -96,7 +112,7 @@ template <int DIR> struct Dft<2, DIR> {
   }
 };
 
-template <int DIR> struct Dft<4, DIR> {
+template <int DIR, bool ACC> struct Dft<4, DIR, ACC> {
   static __device__ __forceinline__ void run(float2* v) {
     float2 s02 = cadd(v[0], v[2]), d02 = csub(v[0], v[2]);
     // DIR i (v1 - v3) straight from scalar differences: a swapped pair
@@ -111,18 +127,18 @@ template <int DIR> struct Dft<4, DIR> {
   }
 };
 
-template <int DIR> struct Dft<8, DIR> {
+template <int DIR, bool ACC> struct Dft<8, DIR, ACC> {
   static __device__ __forceinline__ void run(float2* v) {
-    const float h = 0.70710678118654752440f;  // cos(pi/4)
+    constexpr Const<ACC> h(0.70710678118654752440);  // cos(pi/4)
     // two 4-point DFTs on even and odd samples
     float2 e[4] = {v[0], v[2], v[4], v[6]};
     float2 o[4] = {v[1], v[3], v[5], v[7]};
-    Dft<4, DIR>::run(e);
-    Dft<4, DIR>::run(o);
+    Dft<4, DIR, ACC>::run(e);
+    Dft<4, DIR, ACC>::run(o);
     // twiddles exp(DIR 2 pi i k / 8), k = 1, 2, 3
-    float2 o1 = make_float2(h * (o[1].x - DIR * o[1].y), h * (o[1].y + DIR * o[1].x));
+    float2 o1 = make_float2(h.mul(o[1].x - DIR * o[1].y), h.mul(o[1].y + DIR * o[1].x));
     float2 o2 = mul_i<DIR>(o[2]);
-    float2 o3 = make_float2(-h * (o[3].x + DIR * o[3].y), h * (DIR * o[3].x - o[3].y));
+    float2 o3 = make_float2(-h.mul(o[3].x + DIR * o[3].y), h.mul(DIR * o[3].x - o[3].y));
     v[0] = cadd(e[0], o[0]);
     v[4] = csub(e[0], o[0]);
     v[1] = cadd(e[1], o1);
@@ -134,16 +150,16 @@ template <int DIR> struct Dft<8, DIR> {
   }
 };
 
-template <int DIR> struct Dft<3, DIR> {
+template <int DIR, bool ACC> struct Dft<3, DIR, ACC> {
   static __device__ __forceinline__ void run(float2* v) {
-    const float c = -0.5f;                        // cos(2 pi / 3)
-    const float s = DIR * 0.86602540378443864676f;  // DIR * sin(2 pi / 3)
+    const float c = -0.5f;                                 // cos(2 pi / 3)
+    constexpr Const<ACC> s(DIR * 0.86602540378443864676);  // DIR * sin(2 pi / 3)
     float2 a = v[0], b = v[1], d = v[2];
     float2 t = cadd(b, d);
     float2 u = csub(b, d);
     float2 m = make_float2(a.x + c * t.x, a.y + c * t.y);
     // i * s * u
-    float2 r = make_float2(-s * u.y, s * u.x);
+    float2 r = make_float2(-s.mul(u.y), s.mul(u.x));
     v[0] = cadd(a, t);
     v[1] = cadd(m, r);
     v[2] = csub(m, r);
@@ -154,7 +170,7 @@ template <int DIR> struct Dft<3, DIR> {
 //   y_k = x_0 + sum_{r=1}^{(R-1)/2} [ (x_r + x_{R-r}) cos(2 pi r k / R)
 //                                    + DIR i (x_r - x_{R-r}) sin(2 pi r k / R) ],
 // and y_{R-k} the same with the sine term negated.
-template <int R, int DIR> struct DftOdd {
+template <int R, int DIR, bool ACC> struct DftOdd {
   static __device__ __forceinline__ void run(float2* v) {
     constexpr int Hh = (R - 1) / 2;
     float2 s[Hh + 1], d[Hh + 1];
@@ -170,8 +186,15 @@ template <int R, int DIR> struct DftOdd {
     y[0] = y0;
     static_for<1, Hh + 1>([&](auto KK) {
       constexpr int k = decltype(KK)::value;
-      float2 a = v[0];   // the cosine part
+      float2 a = ACC ? make_float2(0.0f, 0.0f) : v[0];  // the cosine part
       float2 b = make_float2(0.0f, 0.0f);  // sum sin * d, to be multiplied by DIR i
+      if constexpr (ACC)  // the constants' low parts first
+        static_for<1, Hh + 1>([&](auto RR) {
+          constexpr int r = decltype(RR)::value;
+          constexpr Const<true> c(cx_cos2pi(r * k, R)), sn(cx_sin2pi(r * k, R));
+          a = make_float2(fmaf(c.lo, s[r].x, a.x), fmaf(c.lo, s[r].y, a.y));
+          b = make_float2(fmaf(sn.lo, d[r].x, b.x), fmaf(sn.lo, d[r].y, b.y));
+        });
       static_for<1, Hh + 1>([&](auto RR) {
         constexpr int r = decltype(RR)::value;
         constexpr float c = (float)cx_cos2pi(r * k, R);
@@ -179,6 +202,7 @@ template <int R, int DIR> struct DftOdd {
         a = make_float2(fmaf(c, s[r].x, a.x), fmaf(c, s[r].y, a.y));
         b = make_float2(fmaf(sn, d[r].x, b.x), fmaf(sn, d[r].y, b.y));
       });
+      if constexpr (ACC) a = cadd(a, v[0]);
       const float2 ib = mul_i<DIR>(b);  // DIR i b
       y[k] = cadd(a, ib);
       y[R - k] = csub(a, ib);
@@ -187,8 +211,8 @@ template <int R, int DIR> struct DftOdd {
     for (int k = 0; k < R; ++k) v[k] = y[k];
   }
 };
-template <int DIR> struct Dft<5, DIR> : DftOdd<5, DIR> {};
-template <int DIR> struct Dft<7, DIR> : DftOdd<7, DIR> {};
+template <int DIR, bool ACC> struct Dft<5, DIR, ACC> : DftOdd<5, DIR, ACC> {};
+template <int DIR, bool ACC> struct Dft<7, DIR, ACC> : DftOdd<7, DIR, ACC> {};
 
 __host__ __device__ constexpr int pick_radix(int rem) {
   return (rem % 8 == 0) ? 8 : (rem % 4 == 0) ? 4 : (rem % 2 == 0) ? 2 : (rem % 3 == 0) ? 3

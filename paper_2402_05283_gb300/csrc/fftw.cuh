@@ -31,11 +31,14 @@ namespace cpra {
 template <int M, int Q, int DIR> struct TwC {
   static constexpr float re = (float)cx_cos2pi(Q, M);
   static constexpr float im = (float)(DIR * cx_sin2pi(Q, M));
+  static constexpr float re_lo = (float)(cx_cos2pi(Q, M) - (double)re);
+  static constexpr float im_lo = (float)(DIR * cx_sin2pi(Q, M) - (double)im);
 };
 
 // In-register E-point DFT, y_k = sum_j v_j exp(DIR 2 pi i jk / E), as
-// self-sorting Stockham passes over compile-time indices.
-template <int E, int DIR, int NS = 1>
+// self-sorting Stockham passes over compile-time indices.  ACC: the constants
+// as pairs of floats (fft.cuh).
+template <int E, int DIR, bool ACC = false, int NS = 1>
 __device__ __forceinline__ void reg_fft(float2 (&v)[E]) {
   if constexpr (NS < E) {
     constexpr int R = pick_radix(E / NS);
@@ -59,12 +62,15 @@ __device__ __forceinline__ void reg_fft(float2 (&v)[E]) {
           } else {
             constexpr float wr = TwC<M, Q, DIR>::re;
             constexpr float wi = TwC<M, Q, DIR>::im;
-            t = make_float2(fmaf(t.x, wr, -t.y * wi), fmaf(t.x, wi, t.y * wr));
+            if constexpr (ACC)
+              t = cmul(t, make_float2(wr, wi), make_float2(TwC<M, Q, DIR>::re_lo, TwC<M, Q, DIR>::im_lo));
+            else
+              t = make_float2(fmaf(t.x, wr, -t.y * wi), fmaf(t.x, wi, t.y * wr));
           }
         }
         x[r] = t;
       });
-      Dft<R, DIR>::run(x);
+      Dft<R, DIR, ACC>::run(x);
       constexpr int base = (j / NS) * NS * R + k;
       static_for<0, R>([&](auto RR) {
         constexpr int r = decltype(RR)::value;
@@ -72,7 +78,7 @@ __device__ __forceinline__ void reg_fft(float2 (&v)[E]) {
       });
     });
     static_for<0, E>([&](auto I) { v[decltype(I)::value] = out[decltype(I)::value]; });
-    reg_fft<E, DIR, NS * R>(v);
+    reg_fft<E, DIR, ACC, NS * R>(v);
   }
 }
 
@@ -106,6 +112,7 @@ template <> struct WarpPlan<768> { static constexpr int E1 = 24, E2 = 32, L = 1;
 
 template <int N> struct WP {
   static constexpr int E1 = WarpPlan<N>::E1, E2 = WarpPlan<N>::E2, L = WarpPlan<N>::L;
+  static constexpr bool POW2 = (N & (N - 1)) == 0;
   static constexpr int NA = L * E2, NB = L * E1;  // step-A and step-B tasks of the warp
   static constexpr int TA = (NA + 31) / 32;       // step-A slots per lane
   static constexpr int TB = (NB + 31) / 32;       // step-B slots per lane
@@ -140,8 +147,10 @@ __device__ __forceinline__ void tc_step_a(float2 (&a)[WP<N>::TA][WP<N>::E1], flo
   __syncwarp();
 }
 
-// A layout -> B layout (forward, unnormalised)
-template <int N, int PREC = kPrecFP32>
+// A layout -> B layout (forward, unnormalised).  ACC: constants as pairs of
+// floats and, unless N is a power of two, the cross twiddles too (their low
+// parts at xtw + N): see WarpLines.
+template <int N, int PREC = kPrecFP32, bool ACC = false>
 __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
                                              float2 (&b)[WP<N>::TB][WP<N>::E2], float2* T,
                                              const float2* xtw, int lane,
@@ -149,7 +158,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
   using P = WP<N>;
   if constexpr (PREC != kPrecFP32) tc_step_a<N, PREC, -1>(a, T, *tc, lane);
   if constexpr (PREC == kPrecFP32)
-    static_for<0, P::TA>([&](auto II) { reg_fft<P::E1, -1>(a[decltype(II)::value]); });
+    static_for<0, P::TA>([&](auto II) { reg_fft<P::E1, -1, ACC>(a[decltype(II)::value]); });
   // cross twiddles: k1 outermost so tasks of a lane that share l share the load
   static_for<0, P::E1>([&](auto KK) {
     constexpr int k1 = decltype(KK)::value;
@@ -158,7 +167,8 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
       constexpr int i = decltype(II)::value;
       const int l = (lane + 32 * i) % P::E2;
       v[i] = a[i][k1];
-      if constexpr (k1 > 0) v[i] = cmul(v[i], xtw[k1 * P::E2 + l]);
+      if constexpr (k1 > 0 && ACC && !P::POW2) v[i] = cmul(v[i], xtw[k1 * P::E2 + l], xtw[N + k1 * P::E2 + l]);
+      else if constexpr (k1 > 0) v[i] = cmul(v[i], xtw[k1 * P::E2 + l]);
     });
     static_for<0, P::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
@@ -182,7 +192,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
         constexpr int l = decltype(LL)::value;
         b[i][l] = T[(line * P::E1 + k1) * P::TP + l];
       });
-    if constexpr (PREC == kPrecFP32) reg_fft<P::E2, -1>(b[i]);
+    if constexpr (PREC == kPrecFP32) reg_fft<P::E2, -1, ACC>(b[i]);
   });
   __syncwarp();
 }
@@ -193,7 +203,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
 struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
-template <int N, int PREC = kPrecFP32, class Hook = NoHook>
+template <int N, int PREC = kPrecFP32, bool ACC = false, class Hook = NoHook>
 __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
                                              float2 (&a)[WP<N>::TA][WP<N>::E1], float2* T,
                                              const float2* xtw, int lane,
@@ -203,7 +213,7 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
     const int line = t / P::E1, k1 = t % P::E1;
-    if constexpr (PREC == kPrecFP32) reg_fft<P::E2, +1>(b[i]);
+    if constexpr (PREC == kPrecFP32) reg_fft<P::E2, +1, ACC>(b[i]);
     if (P::b_on(t))
       static_for<0, P::E2>([&](auto LL) {
         constexpr int l = decltype(LL)::value;
@@ -226,7 +236,9 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
     static_for<0, P::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int l = (lane + 32 * i) % P::E2;
-      if constexpr (k1 > 0) a[i][k1] = cmul(a[i][k1], cconj(xtw[k1 * P::E2 + l]));
+      if constexpr (k1 > 0 && ACC && !P::POW2)
+        a[i][k1] = cmul(a[i][k1], cconj(xtw[k1 * P::E2 + l]), cconj(xtw[N + k1 * P::E2 + l]));
+      else if constexpr (k1 > 0) a[i][k1] = cmul(a[i][k1], cconj(xtw[k1 * P::E2 + l]));
     });
   });
   if constexpr (!std::is_same_v<std::decay_t<Hook>, NoHook>) {
@@ -234,7 +246,7 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
     tile_free();
   }
   if constexpr (PREC == kPrecFP32)
-    static_for<0, P::TA>([&](auto II) { reg_fft<P::E1, +1>(a[decltype(II)::value]); });
+    static_for<0, P::TA>([&](auto II) { reg_fft<P::E1, +1, ACC>(a[decltype(II)::value]); });
   __syncwarp();
   if constexpr (PREC != kPrecFP32) tc_step_a<N, PREC, +1>(a, T, *tc, lane);
 }
@@ -243,8 +255,23 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
 // a layout covers
 //   A layout: line a_line(t), points a_x(t, m), m < E1;
 //   B layout: line b_line(t), frequencies b_k(t, j), j < E2.
-template <int N> struct WarpLines {
+//
+// Acc is the plan with accurate constants, for the refinement (k_refine_w.cu),
+// which runs a transform and its inverse over the same values hundreds of
+// times, and, unless N is a power of two, for the assembly.  The rounding of a
+// constant (cos(pi/4) as a float is 1.7e-8 short) is the same in every pass
+// and adds up in step; it was more than half of the refinement's error.  xs
+// holds XN cross twiddles: pairs where N has an odd factor, whose transforms
+// have more of them and more terms.
+// Error against 64 bits, plain / constants / with cross twiddles: refinement,
+// N = 256, 180 angles, 50 iterations 8.1e-7 / 4.5e-7 / 3.7e-7 in 8.12 / 8.24 /
+// 8.74 ms; N = 160, 60 angles, 10 iterations 3.2e-7 / 2.4e-7 / 2.2e-7 in 0.94
+// / 0.96 / 1.00 ms; assembly, N = 192, 90 angles 3.8e-7 / 3.75e-7 / 3.6e-7.
+template <int N, bool ACC_ = false> struct WarpLines {
   using P = WP<N>;
+  static constexpr bool ACC = ACC_;
+  using Acc = WarpLines<N, true>;
+  static constexpr int XN = ACC && !P::POW2 ? 2 * N : N;
   static constexpr int L = P::L, TA = P::TA, E1 = P::E1, TB = P::TB, E2 = P::E2, TSIZE = P::TSIZE;
   // whether task t exists (else its registers hold nothing)
   static __device__ __forceinline__ bool a_on(int t) { return P::a_on(t); }
@@ -255,12 +282,12 @@ template <int N> struct WarpLines {
   static __device__ __forceinline__ int b_k(int t, int j) { return t % E1 + E1 * j; }
   static __device__ __forceinline__ void fwd(float2 (&a)[TA][E1], float2 (&b)[TB][E2], float2* T,
                                              const float2* xs, int lane) {
-    warp_fft_fwd<N>(a, b, T, xs, lane);
+    warp_fft_fwd<N, kPrecFP32, ACC>(a, b, T, xs, lane);
   }
   template <class Hook = NoHook>
   static __device__ __forceinline__ void inv(float2 (&b)[TB][E2], float2 (&a)[TA][E1], float2* T,
                                              const float2* xs, int lane, Hook&& tile_free = Hook{}) {
-    warp_fft_inv<N, kPrecFP32>(b, a, T, xs, lane, nullptr, tile_free);
+    warp_fft_inv<N, kPrecFP32, ACC>(b, a, T, xs, lane, nullptr, tile_free);
   }
 };
 }  // namespace cpra

@@ -23,8 +23,10 @@
 
 namespace cpra {
 
-struct PairLines512 {
-  static constexpr int N = 512, L = 1, TA = 1, E1 = 16, TB = 1, E2 = 16;
+template <bool ACC_> struct PairLines {
+  static constexpr bool ACC = ACC_;
+  using Acc = PairLines<true>;  // with accurate constants (see WarpLines)
+  static constexpr int N = 512, XN = N, L = 1, TA = 1, E1 = 16, TB = 1, E2 = 16;
   static constexpr int TP = 34;  // even pitch: both transpose directions conflict-free
   static constexpr int TSIZE = 16 * TP;
   static __device__ __forceinline__ bool a_on(int) { return true; }
@@ -37,7 +39,7 @@ struct PairLines512 {
   // A layout -> B layout (forward, unnormalised)
   static __device__ __forceinline__ void fwd(float2 (&a)[1][16], float2 (&b)[1][16], float2* T,
                                              const float2* xs, int lane) {
-    reg_fft<16, -1>(a[0]);
+    reg_fft<16, -1, ACC>(a[0]);
     {
       const float2 w8 = xs[8 * 32 + lane];
       static_for<1, 8>([&](auto KK) {
@@ -59,7 +61,7 @@ struct PairLines512 {
       b[0][l2] = T[k1 * TP + h + 2 * l2];
     });
     __syncwarp();
-    reg_fft<16, -1>(b[0]);
+    reg_fft<16, -1, ACC>(b[0]);
     pair_butterfly<-1>(b[0], h);
   }
 
@@ -68,7 +70,7 @@ struct PairLines512 {
                                              const float2* xs, int lane) {
     const int k1 = lane >> 1, h = lane & 1;
     pair_butterfly<+1>(b[0], h);
-    reg_fft<16, +1>(b[0]);
+    reg_fft<16, +1, ACC>(b[0]);
     static_for<0, 16>([&](auto LL) {
       constexpr int l2 = decltype(LL)::value;
       T[k1 * TP + h + 2 * l2] = b[0][l2];
@@ -89,7 +91,7 @@ struct PairLines512 {
       });
       a[0][8] = cmul(a[0][8], w8);
     }
-    reg_fft<16, +1>(a[0]);
+    reg_fft<16, +1, ACC>(a[0]);
   }
 
  private:
@@ -114,9 +116,15 @@ struct PairLines512 {
     static_for<1, 16>([&](auto JJ) {
       constexpr int j = decltype(JJ)::value;
       const float2 w = h ? make_float2(TwC<32, j, DIR>::re, TwC<32, j, DIR>::im) : make_float2(1.0f, 0.0f);
-      v[j] = cmul(v[j], w);
+      if constexpr (ACC) {
+        const float2 wl = h ? make_float2(TwC<32, j, DIR>::re_lo, TwC<32, j, DIR>::im_lo) : make_float2(0.0f, 0.0f);
+        v[j] = cmul(v[j], w, wl);
+      } else {
+        v[j] = cmul(v[j], w);
+      }
     });
   }
 };
+using PairLines512 = PairLines<false>;
 
 }  // namespace cpra

@@ -35,13 +35,13 @@ namespace cpra {
 
 namespace {
 
-template <int N> using XW = RowCfg<N, typename WLines<N, kPrecFP32>::type>;
+template <int N> using XW = RowCfg<N, typename WLines<N, kPrecFP32>::type::Acc>;
 
 // columns a block of the line passes: the column pass's, but 8 at N = 1024,
 // so that the constraint's data fits beside them
 template <int N> struct VW {
   using C = ColW<N, kPrecFP32>;
-  using FL = typename C::FL;
+  using FL = typename C::FL::Acc;
   static constexpr int CB = N == 1024 ? 8 : C::CB;
   static constexpr int WARPS = CB / FL::L, NT = WARPS * 32;
   static constexpr int MINB = N == 1024 ? 1 : C::MINB;
@@ -54,9 +54,9 @@ template <int N> struct VW {
 };
 
 template <int N>
-constexpr size_t xw_smem() { return sizeof(float2) * (N + XW<N>::WARPS * XW<N>::FL::TSIZE); }
-template <int N>
-constexpr size_t vw_smem() { return sizeof(float2) * (N + VW<N>::BUF); }
+constexpr size_t xw_smem() { return sizeof(float2) * (XW<N>::FL::XN + XW<N>::WARPS * XW<N>::FL::TSIZE); }
+template <int N, class FL = typename VW<N>::FL>
+constexpr size_t vw_smem() { return sizeof(float2) * (FL::XN + VW<N>::BUF); }
 // the constraint pass also stages the data columns (same rows, same pitch)
 template <int N>
 constexpr size_t vw_smem_c() { return vw_smem<N>() + sizeof(float2) * VW<N>::STAGE; }
@@ -97,9 +97,10 @@ __device__ __forceinline__ void take_a(float2 (&a)[FL::TA][FL::E1], const float2
     });
   });
 }
+// (with 1/N as a constant of FL's accuracy)
 template <int N, class FL>
 __device__ __forceinline__ void put_a(const float2 (&a)[FL::TA][FL::E1], float2* buf, int col0, int lane) {
-  const float inv = 1.0f / N;
+  constexpr Const<FL::ACC && !WP<N>::POW2> inv(1.0 / N);
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
@@ -107,7 +108,7 @@ __device__ __forceinline__ void put_a(const float2 (&a)[FL::TA][FL::E1], float2*
     const int col = col0 + FL::a_line(t);
     static_for<0, FL::E1>([&](auto MM) {
       constexpr int m = decltype(MM)::value;
-      buf[FL::a_x(t, m) * VW<N>::SP + col] = cscale(a[i][m], inv);
+      buf[FL::a_x(t, m) * VW<N>::SP + col] = inv.mul(a[i][m]);
     });
   });
 }
@@ -131,8 +132,8 @@ k_xw(float2* X, const float2* __restrict__ xtw, size_t rows) {
   extern __shared__ float2 smem[];
   float2* xs = smem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* T = smem + N + warp * FL::TSIZE;
-  load_xtw<N>(xs, xtw, WARPS * 32);
+  float2* T = smem + FL::XN + warp * FL::TSIZE;
+  load_xtw<FL::XN>(xs, xtw, WARPS * 32);
   __syncthreads();
   const size_t row0 = ((size_t)blockIdx.x * WARPS + warp) * FL::L;
   if (row0 >= rows) return;  // L divides the rows
@@ -160,16 +161,16 @@ template <int N, bool INV>
 __global__ void __launch_bounds__(VW<N>::NT, VW<N>::MINB)
 k_vw(float2* X, float2* out, const float2* __restrict__ xtw, size_t outer, size_t estride) {
   using C = VW<N>;
-  using FL = typename C::FL;
+  using FL = std::conditional_t<INV, VolLines<N>, typename C::FL>;
   extern __shared__ float2 smem[];
   float2* xs = smem;
-  float2* buf = smem + N;  // staging, then the warps' transpose tiles
+  float2* buf = smem + FL::XN;  // staging, then the warps' transpose tiles
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* base = X + blockIdx.y * outer + blockIdx.x * C::CB;
   const VRows<N> rows;
   rows.each([&](int y) { cp_async8(buf + y * C::SP + rows.cc, base + y * estride + rows.cc); });
   cp_async_commit();
-  load_xtw<N>(xs, xtw, C::NT);
+  load_xtw<FL::XN>(xs, xtw, C::NT);
   cp_async_wait_all();
   __syncthreads();
   float2 a[FL::TA][FL::E1], b[FL::TB][FL::E2];
@@ -252,7 +253,7 @@ k_rx(float2* X, float* R, const uint32_t* __restrict__ S3, const float2* __restr
   extern __shared__ float2 smem[];
   float2* xs = smem;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* T = smem + N + warp * FL::TSIZE;
+  float2* T = smem + FL::XN + warp * FL::TSIZE;
   const size_t row0 = 2 * (((size_t)blockIdx.x * WARPS + warp) * FL::L);  // first image row of the warp
   if constexpr (MODE != kRFwd) {
     // 2L spectrum rows of H values into the tile, 16 bytes a piece
@@ -265,7 +266,7 @@ k_rx(float2* X, float* R, const uint32_t* __restrict__ S3, const float2* __restr
     }
     cp_async_commit();
   }
-  load_xtw<N>(xs, xtw, WARPS * 32);
+  load_xtw<FL::XN>(xs, xtw, WARPS * 32);
   if constexpr (MODE != kRFwd) cp_async_wait_all();
   __syncthreads();
   float2 a[FL::TA][FL::E1], b[FL::TB][FL::E2];
@@ -291,7 +292,7 @@ k_rx(float2* X, float* R, const uint32_t* __restrict__ S3, const float2* __restr
     __syncwarp();  // the tile is the transforms' scratch from here on
     FL::inv(b, a, T, xs, lane);
   }
-  const float inv = 1.0f / N;
+  constexpr Const<!WP<N>::POW2> inv(1.0 / N);
   static_for<0, FL::TA>([&](auto II) {
     constexpr int i = decltype(II)::value;
     const int t = lane + 32 * i;
@@ -306,8 +307,8 @@ k_rx(float2* X, float* R, const uint32_t* __restrict__ S3, const float2* __restr
         v0 = R[row * N + x];
         v1 = R[(row + 1) * N + x];
       } else {
-        v0 = a[i][m].x * inv;
-        v1 = a[i][m].y * inv;
+        v0 = inv.mul(a[i][m].x);
+        v1 = inv.mul(a[i][m].y);
       }
       if constexpr (MODE == kRInv) {
         R[row * N + x] = v0;
@@ -364,7 +365,7 @@ k_rv(float2* X, const float2* __restrict__ Wd, const uint8_t* __restrict__ M, co
   __shared__ double red[32];
   __shared__ uint8_t sc[C::CB];  // M(k) + M(-k) of the block's columns
   float2* xs = smem;
-  float2* buf = smem + N;
+  float2* buf = smem + FL::XN;
   float2* wbuf = buf + C::BUF;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int c0 = blockIdx.x * C::CB;
@@ -386,7 +387,7 @@ k_rv(float2* X, const float2* __restrict__ Wd, const uint8_t* __restrict__ M, co
     });
   }
   cp_async_commit();
-  load_xtw<N>(xs, xtw, C::NT);
+  load_xtw<FL::XN>(xs, xtw, C::NT);
   cp_async_wait_all();
   __syncthreads();
   float2 a[FL::TA][FL::E1], b[FL::TB][FL::E2];
@@ -531,10 +532,10 @@ template <int N>
 cudaError_t volume_ylines_n(float2* vol, float2* out, const float2* xtw, cudaStream_t st) {
   using C = VW<N>;
   static PerDevice<bool> attr;
-  const cudaError_t e = smem_once(k_vw<N, true>, vw_smem<N>(), attr);
+  const cudaError_t e = smem_once(k_vw<N, true>, vw_smem<N, VolLines<N>>(), attr);
   if (e != cudaSuccess) return e;
   g_launches += 1;
-  k_vw<N, true><<<dim3(N / C::CB, N), C::NT, vw_smem<N>(), st>>>(vol, out, xtw, (size_t)N * N, (size_t)N);
+  k_vw<N, true><<<dim3(N / C::CB, N), C::NT, vw_smem<N, VolLines<N>>(), st>>>(vol, out, xtw, (size_t)N * N, (size_t)N);
   return cudaGetLastError();
 }
 
