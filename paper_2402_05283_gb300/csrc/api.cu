@@ -1229,7 +1229,7 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
   if (!p->mg_acc && !alloc_all(p, {want(p->mg_acc, Np * NN * 8), want(p->mg_ref, NN * 8)}))
     return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
   if (prtf && !p->mg_rings) {
-    p->mg_rings = (double*)dev_alloc(p, sizeof(double) * Np * (N / 2) + sizeof(unsigned) * (N / 2));
+    p->mg_rings = (unsigned long long*)dev_alloc(p, sizeof(unsigned long long) * Np * (N / 2) + sizeof(unsigned) * (N / 2));
     if (!p->mg_rings) return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
   }
   if (p->mg_cap < n_l) {  // (the stream is idle)

@@ -13,7 +13,7 @@ __host__ __device__ constexpr int ramp_len(int N) { return N + N / 2 + 1; }
 
 // Q = sum over a cell's samples of ku < 0 of weight * corr
 cudaError_t launch_grid_corr(cpra_plan_s* p);
-cudaError_t launch_prtf(const double* rings, const unsigned* counts, float* prtf, int H, int total,
+cudaError_t launch_prtf(const unsigned long long* rings, const unsigned* counts, float* prtf, int H, int total,
                         cudaStream_t st);
 
 // ---------------------------------------------------------------- columns
@@ -209,6 +209,27 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
   }
 }
 
+// The PRTF's ring sums are whole numbers of 2^-50, so they are exact in any
+// order: a ring holds fewer than 2^12 values of at most 1.  Bit 63 (out of the
+// sums' reach) says that one was not a number.  (FP64 sums in shared memory
+// depend on the order in their last bits, and their atomics are loops: N = 256,
+// 144 angles, four guesses 0.783 ms a merge; with FP32 sums 0.722, so 0.734.)
+constexpr double kRingUnit = 8.8817841970012523e-16;  // 2^-50
+constexpr unsigned long long kRingNaN = 1ull << 63;
+// |v| / m (0 where m is 0): the FP32 quotient and its remainder over m
+__device__ __forceinline__ unsigned long long prtf_ratio(float2 v, float m) {
+  if (!(m > 0.0f)) return 0;
+  const float a = sqrtf(fmaf(v.x, v.x, v.y * v.y)), q = a / m;
+  if (!(q <= 2.0f)) return kRingNaN;
+  const float rest = fmaf(-q, m, a) / m;  // (m infinite: not a number, and q is 0)
+  const long long lo = fabsf(rest) < q ? __float2ll_rn(rest * 0x1p50f) : 0;
+  return (unsigned long long)(__float2ll_rn(q * 0x1p50f) + lo);
+}
+__device__ __forceinline__ void add_ring(unsigned long long* ring, unsigned long long f) {
+  if (f < kRingNaN) atomicAdd(ring, f);
+  else atomicOr(ring, kRingNaN);
+}
+
 // One block of columns of angle blockIdx.y through every kept guess: the mean
 // of the corrected spectra (full plane, into acc), the ring sums of
 // |sum E'| / sum |E'| and F of the mean.  E(-k) = conj E(k) but for the row
@@ -219,7 +240,7 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
 // ms at one CTA an SM and 0.16 at two).
 template <int N>
 __global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, ColW<N, kPrecFP32>::NT <= 256 && N <= 512 ? 2 : 1)
-k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* counts, float2* F,
+k_merge(const MergeArgs ma, int n_l, float2* acc, unsigned long long* rings, unsigned* counts, float2* F,
         float2* corr, const float2* __restrict__ xtw) {
   using C = ColW<N, kPrecFP32>;
   using FL = VolLines<N>;
@@ -230,7 +251,7 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
   float2* z0 = rz + N;
   float2* buf = z0 + N;
   __shared__ float2 sh[C::CB];  // mean of the partner row kz = -N/2 of the block's columns
-  __shared__ float ring[H];
+  __shared__ unsigned long long ring[H];
   __shared__ unsigned cnt[H];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* T = buf + warp * FL::TSIZE;
@@ -241,7 +262,7 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
   const bool packed = c0 == 0 && warp == 0;
   for (int i = threadIdx.x; i < FL::XN; i += C::NT) xs[i] = xtw[i];
   for (int i = threadIdx.x; i < H; i += C::NT) {
-    ring[i] = 0.0f;
+    ring[i] = 0;
     cnt[i] = 0u;
   }
   // pass 0: columns c0 .. (column 0 of the packed pair); pass 1, first block
@@ -306,15 +327,10 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
         const int kz = k < H ? k : k - N, ku = c == 0 && pass ? H : c;
         const int r = (int)rintf(sqrtf((float)(kz * kz + ku * ku)));  // exact: no square is near (m + 1/2)^2
         if (r < H) {
-          const float m = mg[i][j];
-          float f = m > 0.0f ? sqrtf(fmaf(v.x, v.x, v.y * v.y)) / m : 0.0f;
+          const unsigned long long f = prtf_ratio(v, mg[i][j]);
           const bool two = c > 0;  // and its partner (-kz, -ku)
-          if (two) {
-            float fm = f;
-            if (k == H) fm = mh[i] > 0.0f ? sqrtf(fmaf(sm[i].x, sm[i].x, sm[i].y * sm[i].y)) / mh[i] : 0.0f;
-            f += fm;
-          }
-          atomicAdd(ring + r, f);
+          if (two && k == H) add_ring(ring + r, prtf_ratio(sm[i], mh[i]));
+          add_ring(ring + r, two && k != H && f < kRingNaN ? 2 * f : f);
           if (n == 0) atomicAdd(cnt + r, two ? 2u : 1u);
         }
       }
@@ -349,7 +365,10 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, double* rings, unsigned* count
   if (rings) {
     __syncthreads();
     for (int i = threadIdx.x; i < H; i += C::NT) {
-      if (ring[i] != 0.0f) atomicAdd(rings + (size_t)n * H + i, (double)ring[i]);
+      if (ring[i]) {
+        add_ring(rings + (size_t)n * H + i, ring[i] & ~kRingNaN);
+        if (ring[i] >= kRingNaN) add_ring(rings + (size_t)n * H + i, kRingNaN);
+      }
       if (n == 0 && cnt[i]) atomicAdd(counts + i, cnt[i]);
     }
   }
@@ -565,7 +584,7 @@ cudaError_t merge_twins_n(cpra_plan_s* d, const MergeArgs& ma, int n_l) {
 }
 
 template <int N>
-cudaError_t merge_n(cpra_plan_s* d, const MergeArgs& ma, int n_l, float2* acc, double* rings,
+cudaError_t merge_n(cpra_plan_s* d, const MergeArgs& ma, int n_l, float2* acc, unsigned long long* rings,
                            float* prtf) {
   using C = ColW<N, kPrecFP32>;
   cudaStream_t st = d->stream;
@@ -574,7 +593,7 @@ cudaError_t merge_n(cpra_plan_s* d, const MergeArgs& ma, int n_l, float2* acc, d
   const size_t total = (size_t)d->Np * (N / 2);
   unsigned* counts = reinterpret_cast<unsigned*>(rings + total);
   if (e == cudaSuccess && rings)
-    e = cudaMemsetAsync(rings, 0, sizeof(double) * total + sizeof(unsigned) * (N / 2), st);
+    e = cudaMemsetAsync(rings, 0, sizeof(unsigned long long) * total + sizeof(unsigned) * (N / 2), st);
   if (e != cudaSuccess) return e;
   g_launches += 1;
   k_merge<N><<<dim3((N / 2) / C::CB, d->Np), C::NT, spec_smem<N>(), st>>>(
@@ -590,6 +609,6 @@ cudaError_t merge_n(cpra_plan_s* d, const MergeArgs& ma, int n_l, float2* acc, d
 #define CPRA_ASSEMBLE_INSTANCES(NN, EXTERN)                                                   \
   EXTERN template cudaError_t assemble_n<NN>(cpra_plan_s*, float2*);                          \
   EXTERN template cudaError_t merge_twins_n<NN>(cpra_plan_s*, const MergeArgs&, int);         \
-  EXTERN template cudaError_t merge_n<NN>(cpra_plan_s*, const MergeArgs&, int, float2*, double*, float*);
+  EXTERN template cudaError_t merge_n<NN>(cpra_plan_s*, const MergeArgs&, int, float2*, unsigned long long*, float*);
 
 }  // namespace cpra

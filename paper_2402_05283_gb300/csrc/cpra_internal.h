@@ -115,7 +115,7 @@ struct cpra_plan_s {
   // Step C merge scratch (cpra_merge with this plan as destination)
   float2* mg_acc = nullptr;    // [Np][N][N] merged spectra (the mean)
   float2* mg_ref = nullptr;    // [N][N] E of the reference PO of the best guess
-  double* mg_rings = nullptr;  // [Np][N/2] ring sums of the PRTF, then N/2 ring populations
+  unsigned long long* mg_rings = nullptr;  // [Np][N/2] ring sums of the PRTF, then N/2 ring populations
   int32_t mg_cap = 0;          // kept guesses that mg_guess, mg_dist and mg_ramps hold
   cpra::MergeGuess* mg_guess = nullptr;
   double* mg_dist = nullptr;   // [mg_cap][2] twin distances
@@ -355,7 +355,7 @@ cudaError_t launch_rho_rows(cpra_plan_s* p, const Launch& L, double* moments, fl
 cudaError_t launch_merge_twins(cpra_plan_s* dst, const MergeArgs& ma, int n_l);
 // acc = mean of the corrected spectra, PRTF (rings and prtf not NULL), its
 // IDFT_z, gridding and the plane IFFTs into dst's volume, on dst's stream
-cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, double* rings,
+cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, unsigned long long* rings,
                          float* prtf);
 // inverse FFT along y of every plane of a volume, in place, and into out when
 // that is not NULL (k_refine_w.cu)

@@ -162,12 +162,13 @@ cudaError_t launch_grid_corr(cpra_plan_s* p) {
 }
 
 // PRTF = ring mean (float), from the ring sums and the ring populations
-__global__ void k_prtf(const double* __restrict__ rings, const unsigned* __restrict__ counts, float* prtf,
+__global__ void k_prtf(const unsigned long long* __restrict__ rings, const unsigned* __restrict__ counts, float* prtf,
                        int H, int total) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= total) return;
   const unsigned c = counts[i % H];
-  prtf[i] = c ? (float)(rings[i] / (double)c) : 0.0f;
+  const unsigned long long s = rings[i];
+  prtf[i] = s >= kRingNaN ? __int_as_float(0x7fc00000) : c ? (float)((double)s * kRingUnit / (double)c) : 0.0f;
 }
 
 // ------------------------------------------------------------------ launchers
@@ -177,7 +178,7 @@ size_t spectra_bytes(int N, int Np) {
   return sizeof(float2) * 8 * (size_t)((N + 7) / 8) * Np * (N / 2 + 1);
 }
 
-cudaError_t launch_prtf(const double* rings, const unsigned* counts, float* prtf, int H, int total,
+cudaError_t launch_prtf(const unsigned long long* rings, const unsigned* counts, float* prtf, int H, int total,
                         cudaStream_t st) {
   g_launches += 1;
   k_prtf<<<(total + 255) / 256, 256, 0, st>>>(rings, counts, prtf, H, total);
@@ -226,7 +227,7 @@ cudaError_t launch_merge_twins(cpra_plan_s* dst, const MergeArgs& ma, int n_l) {
 #undef CPRA_CASE
 }
 
-cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, double* rings,
+cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, unsigned long long* rings,
                          float* prtf) {
 #define CPRA_CASE(NN) \
   case NN: return merge_n<NN>(dst, ma, n_l, acc, rings, prtf);
