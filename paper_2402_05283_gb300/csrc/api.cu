@@ -1237,7 +1237,7 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
     dev_free(p, p->mg_dist);
     dev_free(p, p->mg_ramps);
     p->mg_cap = 0;
-    if (!alloc_all(p, {want(p->mg_guess, sizeof(MergeGuess) * n_l), want(p->mg_dist, sizeof(double) * 2 * n_l),
+    if (!alloc_all(p, {want(p->mg_guess, sizeof(MergeGuess) * n_l), want(p->mg_dist, sizeof(double) * n_l),
                        want(p->mg_ramps, ramps_bytes(N, Np) * n_l)}))
       return fail(p, CPRA_ERR_OUT_OF_MEMORY, "merge scratch");
     p->mg_cap = n_l;
@@ -1275,11 +1275,11 @@ cpra_status cpra_merge(const cpra_plan_t* guesses, int32_t n_r, int32_t n_l, int
   CK(upload_table(), "merge table");
   if (n_l > 1) {  // R16: the version nearer to the best episode's reference PO
     CK(timed(p, CPRA_KERNEL_ASSEMBLE, [&] { return launch_merge_twins(p, ma, n_l); }), "merge twins");
-    std::vector<double> d(2 * (size_t)n_l);
-    CK(cudaMemcpyAsync(d.data(), p->mg_dist, sizeof(double) * 2 * n_l, cudaMemcpyDeviceToHost, p->stream),
+    std::vector<double> d((size_t)n_l);
+    CK(cudaMemcpyAsync(d.data(), p->mg_dist, sizeof(double) * n_l, cudaMemcpyDeviceToHost, p->stream),
        "merge distances");
     CK(cudaStreamSynchronize(p->stream), "merge sync");
-    for (int k = 1; k < n_l; ++k) table[k].inv = flips[k] = d[2 * k + 1] < d[2 * k] ? 1 : 0;
+    for (int k = 1; k < n_l; ++k) table[k].inv = flips[k] = d[k] < 0.0 ? 1 : 0;
     CK(upload_table(), "merge table");
   }
   float* prtf_dev = nullptr;

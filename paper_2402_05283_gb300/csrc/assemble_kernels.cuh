@@ -175,15 +175,16 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
       store_f<N, FL>(a, F, n, Np, H, lane, [](int line) { return line == 0; });
     }
   } else {
-    float dp = 0.0f, dpe = 0.0f, dt = 0.0f, dte = 0.0f;  // |ref - E|^2, |ref - conj E|^2
+    // |ref - E|^2 - |ref - conj E|^2 = -4 Im ref Im E: one FP64 product a value
+    // decides (a merge of four guesses, N = 256, 144 angles: 0.775 ms with both
+    // distances in FP64, 0.737 so)
+    double dot = 0.0;
     auto take = [&](int kz, int ku, float2 v) {
       if constexpr (MODE == kSpecRef) {
         ma.ref[(size_t)kz * N + ku] = v;
       } else {
         const float2 r = ma.ref[(size_t)kz * N + ku];
-        const float ax = r.x - v.x, ay = r.y - v.y, by = r.y + v.y;
-        two_add(dp, dpe, fmaf(ax, ax, ay * ay));
-        two_add(dt, dte, fmaf(ax, ax, by * by));
+        dot += (double)r.y * (double)v.y;
       }
     };
     each_b<FL>(lane, [&](auto II, auto JJ, int t) {
@@ -200,11 +201,8 @@ k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float
       }
     });
     if constexpr (MODE == kSpecDist) {
-      const double d_plain = warp_sum(dp, dpe), d_twin = warp_sum(dt, dte);
-      if (lane == 0) {
-        atomicAdd(ma.dist + 2 * blockIdx.y + 0, d_plain);
-        atomicAdd(ma.dist + 2 * blockIdx.y + 1, d_twin);
-      }
+      dot = warp_sum(dot);
+      if (lane == 0) atomicAdd(ma.dist + blockIdx.y, dot);
     }
   }
 }
@@ -577,7 +575,7 @@ cudaError_t merge_twins_n(cpra_plan_s* d, const MergeArgs& ma, int n_l) {
   cudaStream_t st = d->stream;
   cudaError_t e = spectra_n<N, kSpecRef>(nullptr, nullptr, nullptr, nullptr, d->xtw, ma, 1, st);
   if (e != cudaSuccess || n_l < 2) return e;
-  e = cudaMemsetAsync(ma.dist, 0, sizeof(double) * 2 * n_l, st);
+  e = cudaMemsetAsync(ma.dist, 0, sizeof(double) * n_l, st);
   return e == cudaSuccess
              ? spectra_n<N, kSpecDist>(nullptr, nullptr, nullptr, nullptr, d->xtw, ma, n_l, st)
              : e;

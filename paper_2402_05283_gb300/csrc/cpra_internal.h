@@ -118,7 +118,7 @@ struct cpra_plan_s {
   unsigned long long* mg_rings = nullptr;  // [Np][N/2] ring sums of the PRTF, then N/2 ring populations
   int32_t mg_cap = 0;          // kept guesses that mg_guess, mg_dist and mg_ramps hold
   cpra::MergeGuess* mg_guess = nullptr;
-  double* mg_dist = nullptr;   // [mg_cap][2] twin distances
+  double* mg_dist = nullptr;   // [mg_cap] twin choice (MergeArgs::dist)
   float2* mg_ramps = nullptr;  // [mg_cap] ramps of the kept guesses
   float* mg_prtf = nullptr;    // [Np][N/2] PRTF staging for host outputs
   bool merged = false;         // mg_acc holds the mean of the last merge
@@ -344,14 +344,14 @@ struct MergeArgs {
   int n0;                   // REF, DIST: the PO
   const MergeGuess* guess;  // device table of the kept guesses, best first
   float2* ref;              // E of PO n0 of the best guess, [kz][ku]
-  double* dist;             // [kept][2] sum |ref - E|^2, sum |ref - conj E|^2
+  double* dist;             // [kept] sum Im ref Im E: negative where conj E is the nearer to ref
 };
 // FP64 moments (sum rho, sum rho z, sum rho u) of rho = P_{S+} g of every angle
 cudaError_t launch_moments(cpra_plan_s* p, double* moments, cudaStream_t st);
 // R2C rows of rho into Hp (L: the plan's launch of a plain object prime over
 // every angle), the moments of rho, and the unit ramps of the mass-centre moves
 cudaError_t launch_rho_rows(cpra_plan_s* p, const Launch& L, double* moments, float2* ramps);
-// twin distances of the kept guesses, on dst's stream
+// twin choice of the kept guesses (MergeArgs::dist), on dst's stream
 cudaError_t launch_merge_twins(cpra_plan_s* dst, const MergeArgs& ma, int n_l);
 // acc = mean of the corrected spectra, PRTF (rings and prtf not NULL), its
 // IDFT_z, gridding and the plane IFFTs into dst's volume, on dst's stream

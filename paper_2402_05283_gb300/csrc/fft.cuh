@@ -330,6 +330,13 @@ __device__ __forceinline__ double warp_sum(float s, float e) {
   return (double)s + (double)e;
 }
 
+// the sum over the warp's lanes, in every lane
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
 // support bit x of the row whose first word is at S[row_off]
 __device__ __forceinline__ bool sbit(const uint32_t* S, size_t row_off, int x) {
   return (S[row_off + (x >> 5)] >> (x & 31)) & 1u;

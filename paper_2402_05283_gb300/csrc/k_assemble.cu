@@ -17,9 +17,9 @@
 //            the inverse transform land centred in x and y.
 //   y lines  inverse FFT along ky in place (k_refine_w.cu).
 // Step C merge of several guesses (cpra_merge): the spectra kernel stores the
-// best guess's E of one PO (REF) and sums the squared distances of the other
-// guesses' E to it as is and conjugated, the spectrum of the centrally
-// inverted PO (DIST); k_merge then takes a block of columns through all kept
+// best guess's E of one PO (REF) and tells for the other guesses whether their
+// E or conj E, the spectrum of the centrally inverted PO, is the nearer to it
+// (DIST); k_merge then takes a block of columns through all kept
 // guesses: mean of E or conj(E), ring sums of |sum E'| / sum |E'| for the
 // PRTF, and the inverse DFT along kz of the mean into F.
 // The inverse 3D DFT is applied as IDFT_z on each slice before gridding
