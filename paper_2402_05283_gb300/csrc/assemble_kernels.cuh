@@ -384,16 +384,18 @@ k_merge(const MergeArgs ma, int n_l, float2* acc, unsigned long long* rings, uns
 // plane.  N = 512, 360 angles, with the transform along kx: 0.91 ms; gather
 // 1.04 and rows 0.63 as separate passes over V.
 constexpr int kHeavy = 32;
-constexpr int kStaged = 2560;  // samples of a row held in shared memory (else read from L2)
 template <int N> struct GridCfg {
   using FL = VolLines<N>;
   static constexpr int L = FL::L, H = N / 2, HC = H + 1;
   static constexpr int NZC = (N + 7) / 8;  // chunks of eight planes
+  // samples of a row held in shared memory (else read from L2): less the low
+  // parts of the cross twiddles, so that three CTAs share an SM at every N
+  static constexpr int STAGED = 2560 - (FL::XN - N);
   // pitch of a line: at least N, room for the warp's tile, 2 mod 8 (the four
   // plane pairs of a quad then start four banks apart)
   static constexpr int P0 = (FL::TSIZE + L - 1) / L > N ? (FL::TSIZE + L - 1) / L : N;
   static constexpr int LP = (P0 + 5) / 8 * 8 + 2;
-  static constexpr size_t SMEM = sizeof(float2) * (FL::XN + 8 * L * LP + kStaged) + sizeof(int) * (N + 4);
+  static constexpr size_t SMEM = sizeof(float2) * (FL::XN + 8 * L * LP + STAGED) + sizeof(int) * (N + 4);
   static_assert(LP >= P0 && LP % 8 == 2, "line pitch");
 };
 
@@ -434,7 +436,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
   float2* xs = smem;
   float2* lines = smem + FL::XN;  // [8 L][LP]
   GridEnt* es = reinterpret_cast<GridEnt*>(lines + 8 * L * LP);
-  int* ptr = reinterpret_cast<int*>(es + kStaged);  // [N + 1]
+  int* ptr = reinterpret_cast<int*>(es + G::STAGED);  // [N + 1]
   __shared__ unsigned short heavy[N];
   __shared__ int n_heavy;
   __shared__ float part[8][4][4];
@@ -443,7 +445,7 @@ k_grid(const float2* __restrict__ F, const float2* __restrict__ Q, const int32_t
   const int quad = threadIdx.x >> 2, q = threadIdx.x & 3;
   if (threadIdx.x == 0) n_heavy = 0;
   const int first = __ldg(cell_ptr + ky * N), count = __ldg(cell_ptr + ky * N + N) - first;
-  const bool staged = count <= kStaged;
+  const bool staged = count <= G::STAGED;
   for (int i = threadIdx.x; i <= N; i += 256) ptr[i] = __ldg(cell_ptr + ky * N + i) - first;
   if (staged)
     for (int i = threadIdx.x; i < count; i += 256) cp_async8(es + i, ents + first + i);

@@ -430,6 +430,35 @@ __device__ __forceinline__ void store_rows(const float2 (&a)[FL::TA][FL::E1], fl
   });
 }
 
+// ---------------------------------------------------------------- moments
+// A lane's sum rho, sum rho z, sum rho u of its rows (p: a row's sum, pu: its
+// sum of rho x) as FP32 pairs, with the exact products by z.
+struct Moments {
+  float s0 = 0.0f, e0 = 0.0f, sz = 0.0f, ez = 0.0f, su = 0.0f, eu = 0.0f;
+  __device__ __forceinline__ void add(float p, float pu, float y) {
+    two_add(s0, e0, p);
+    two_add(su, eu, pu);
+    const float pz = __fmul_rn(p, y);
+    two_add(sz, ez, pz);
+    ez = __fadd_rn(ez, fmaf(p, y, -pz));
+  }
+  // no lane of the warp has left FP32's range (a moment is up to N times the
+  // sum of rho): else the rows are added again in FP64
+  __device__ __forceinline__ bool in_range() const {
+    return __all_sync(0xffffffffu, isfinite(s0) && isfinite(sz) && isfinite(su));
+  }
+  __device__ __forceinline__ void total(double (&m)[3]) const {
+    m[0] = warp_sum(s0, e0);
+    m[1] = warp_sum(sz, ez);
+    m[2] = warp_sum(su, eu);
+  }
+};
+__device__ __forceinline__ void add_moments(double (&d)[3], float p, float pu, float y) {
+  d[0] += (double)p;
+  d[1] += (double)p * (double)y;
+  d[2] += (double)pu;
+}
+
 // ---------------------------------------------------------------- prime
 // MOM (rows of rho for the assembly, a single plain tap): also the FP64
 // moments sum rho, sum rho z, sum rho u of the angle, so that rho is not read
@@ -474,36 +503,39 @@ k_prime_w(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
   if (ca.store_g) store_rows<N, FL>(a, g_dst + (size_t)n * N * N, pair0, lane);
   __shared__ double red[MOM ? 3 : 1][RW::WARPS];
   if constexpr (MOM) {
-    float s0 = 0.0f, e0 = 0.0f, sz = 0.0f, ez = 0.0f, su = 0.0f, eu = 0.0f;
-    static_for<0, FL::TA>([&](auto II) {
-      constexpr int i = decltype(II)::value;
-      const int t = lane + 32 * i;
-      if (!FL::a_on(t)) return;
-      float p[2] = {0.0f, 0.0f}, pu[2] = {0.0f, 0.0f};
-      static_for<0, FL::E1>([&](auto MM) {
-        constexpr int m = decltype(MM)::value;
-        const float x = (float)FL::a_x(t, m);
-        p[0] += a[i][m].x;
-        p[1] += a[i][m].y;
-        pu[0] = fmaf(a[i][m].x, x, pu[0]);
-        pu[1] = fmaf(a[i][m].y, x, pu[1]);
-      });
+    // f(sum, sum of x values, y) of the lane's rows
+    auto rows = [&](auto&& f) {
+      static_for<0, FL::TA>([&](auto II) {
+        constexpr int i = decltype(II)::value;
+        const int t = lane + 32 * i;
+        if (!FL::a_on(t)) return;
+        float p[2] = {0.0f, 0.0f}, pu[2] = {0.0f, 0.0f};
+        static_for<0, FL::E1>([&](auto MM) {
+          constexpr int m = decltype(MM)::value;
+          const float x = (float)FL::a_x(t, m);
+          p[0] += a[i][m].x;
+          p[1] += a[i][m].y;
+          pu[0] = fmaf(a[i][m].x, x, pu[0]);
+          pu[1] = fmaf(a[i][m].y, x, pu[1]);
+        });
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const float y = (float)(2 * (pair0 + FL::a_line(t)) + r);
-        two_add(s0, e0, p[r]);
-        two_add(su, eu, pu[r]);
-        const float pz = __fmul_rn(p[r], y);
-        two_add(sz, ez, pz);
-        ez = __fadd_rn(ez, fmaf(p[r], y, -pz));
-      }
-    });
-    const double m0 = warp_sum(s0, e0), mz = warp_sum(sz, ez), mu = warp_sum(su, eu);
-    if (lane == 0) {
-      red[0][warp] = m0;
-      red[MOM ? 1 : 0][warp] = mz;
-      red[MOM ? 2 : 0][warp] = mu;
+        for (int r = 0; r < 2; ++r) f(p[r], pu[r], (float)(2 * (pair0 + FL::a_line(t)) + r));
+      });
+    };
+    Moments mom;
+    rows([&](float p, float pu, float y) { mom.add(p, pu, y); });
+    double m[3];
+    if (mom.in_range()) {
+      mom.total(m);
+    } else {
+      double d[3] = {0.0, 0.0, 0.0};
+      rows([&](float p, float pu, float y) { add_moments(d, p, pu, y); });
+#pragma unroll
+      for (int q = 0; q < 3; ++q) m[q] = warp_sum(d[q]);
     }
+    if (lane == 0)
+#pragma unroll
+      for (int q = 0; q < 3; ++q) red[MOM ? q : 0][warp] = m[q];
   }
   float2 b[FL::TB][FL::E2];
   lines_fwd<N, PREC, FL>(a, b, T, xs, lane, &tc);
@@ -570,8 +602,8 @@ constexpr size_t col_smem() {
 // keeps one sum per weight).  In plans with a missing-data mask (MASKED),
 // a < 0 marks a pixel left free.  Branch-free: G = 0 takes rsqrt(1) and the
 // direction (1, 0), and |G| - a = 0 * 1 - a.  The per-thread partial sum
-// stays in FP32 (at most a few hundred terms); the reduction across
-// threads, blocks and columns is FP64.
+// stays in FP32 (at most a few hundred terms); across a warp's threads it is an
+// FP32 pair, across warps, blocks and columns FP64.
 template <bool MASKED>
 __device__ __forceinline__ float2 project_w(float2 G, float a, float& e) {
   if constexpr (MASKED)
@@ -610,7 +642,6 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
   const float2* __restrict__ xtw = J->xtw;
   float2* xs = smem;
   float2* buf = smem + N;  // staging, then the warps' transpose tiles
-  __shared__ double red[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* As = reinterpret_cast<float*>(buf + C::BUF);  // A_sym of the block, [c][ky]
   uint32_t tc_phase = 0;
@@ -735,16 +766,16 @@ __device__ __forceinline__ void colpass_tile(const JobStatic* __restrict__ js,
     for (int k = 0; k < SR; ++k)
       if (N % RS == 0 || y0 + k * RS < N) dst[(size_t)k * RS * H] = src[k * RS * C::SP];
   }
+  // the warp's error terms: an FP32 pair, FP64 beyond its range.  Each warp adds
+  // its own: a barrier and one thread's sum over the warps would be the block's
+  // tail (ten iterations, with / without: N = 1024, 300 angles 18.90 / 18.67 ms,
+  // 700, 27 angles 1.31 / 1.27, 512, 360 angles 5.06 / 5.05; without the look at
+  // the range 5.02)
   float es = 2.0f * err2, ee = 0.0f;
   two_add(es, ee, err1);
-  const double errd = warp_sum(es, ee);
-  if (lane == 0) red[warp] = errd;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < C::WARPS; ++w) s += red[w];
-    atomicAdd(err_acc + n, s);
-  }
+  warp_add_pairs(es, ee);
+  const double errd = isfinite(es) ? (double)es + (double)ee : warp_sum(2.0 * (double)err2 + (double)err1);
+  if (lane == 0) atomicAdd(err_acc + n, errd);
   tc_finish<PREC>(tc);
 }
 

@@ -319,23 +319,40 @@ __device__ __forceinline__ void two_add(float& s, float& e, float v) {
   e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
   s = t;
 }
-// the sum over the warp's lanes of s + e, in every lane
-__device__ __forceinline__ double warp_sum(float s, float e) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
-    two_add(s, e, s2);
-    e = __fadd_rn(e, e2);
-  }
-  return (double)s + (double)e;
+// the pair in FP64 (where s has left FP32's range, e is not a number)
+__device__ __forceinline__ double pair_value(float s, float e) {
+  return isfinite(s) ? (double)s + (double)e : (double)s;
 }
-
 // the sum over the warp's lanes, in every lane
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+// s + e <- their sum over the warp's lanes.  Sums of two are the same in both
+// lanes, so s is the same in all; where it is not finite, the sum has left
+// FP32's range (or a lane's was not finite) and is taken in FP64 instead.
+__device__ __forceinline__ void warp_add_pairs(float& s, float& e) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+    two_add(s, e, s2);
+    e = __fadd_rn(e, e2);
+  }
+}
+// the sum over the warp's lanes of s + e, in every lane
+__device__ __forceinline__ double warp_sum(float s, float e) {
+  const float s0 = s, e0 = e;
+  warp_add_pairs(s, e);
+  return isfinite(s) ? (double)s + (double)e : warp_sum(pair_value(s0, e0));
+}
+
+// Error terms of weight 2 and 1 are added as eighths, so that the pair of a
+// lane's two tasks stays in FP32's range where the terms do; what is published
+// is kEighths times the sum.
+constexpr double kEighths = 8.0;
+__device__ __forceinline__ float eighths2(float err2) { return 0.25f * err2; }
+__device__ __forceinline__ float eighths1(float err1) { return 0.125f * err1; }
 
 // support bit x of the row whose first word is at S[row_off]
 __device__ __forceinline__ bool sbit(const uint32_t* S, size_t row_off, int x) {

@@ -38,7 +38,8 @@ CPRA_FOR_EACH_N(CPRA_CASE)
 // take them along and for the refinement.
 // One warp per kMomRows rows: each lane sums its pixels of a row in FP32 (at
 // most N/32 terms) and its rows as pairs of FP32 (48 bits, with the exact
-// products by y); FP64 across lanes, warps and CTAs.  Bound by HBM: the FP64
+// products by y; FP64 where that leaves FP32's range); FP64 across warps and
+// CTAs.  Bound by HBM: the FP64
 // pipe is narrow, and ten FP64 shuffles and adds a row made it the bound
 // (N = 256, 144 angles: 44 us, 33 with one reduction of FP32 pairs per 16 rows).
 constexpr int kMomRows = 16;
@@ -48,32 +49,35 @@ __global__ void k_moments(const float* __restrict__ g, const uint32_t* __restric
   const int n = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int y0 = (blockIdx.x * (blockDim.x >> 5) + warp) * kMomRows;
-  float s0 = 0.0f, e0 = 0.0f, sz = 0.0f, ez = 0.0f, su = 0.0f, eu = 0.0f;
+  auto rows = [&](auto&& f) {
 #pragma unroll 4
-  for (int r = 0; r < kMomRows; ++r) {
-    const int y = y0 + r;
-    if (y >= N) break;
-    const float* gy = g + ((size_t)n * N + y) * N;
-    const uint32_t* sy = S + ((size_t)n * N + y) * W;
-    float p0 = 0.0f, pu = 0.0f;
-    for (int x = lane, w = 0; x < N; x += 32, ++w) {
-      const float v = gy[x];
-      const float q = ((sy[w] >> lane) & 1u) && v >= 0.0f ? v : 0.0f;
-      p0 += q;
-      pu = fmaf(q, (float)x, pu);
+    for (int r = 0; r < kMomRows; ++r) {
+      const int y = y0 + r;
+      if (y >= N) break;
+      const float* gy = g + ((size_t)n * N + y) * N;
+      const uint32_t* sy = S + ((size_t)n * N + y) * W;
+      float p0 = 0.0f, pu = 0.0f;
+      for (int x = lane, w = 0; x < N; x += 32, ++w) {
+        const float v = gy[x];
+        const float q = ((sy[w] >> lane) & 1u) && v >= 0.0f ? v : 0.0f;
+        p0 += q;
+        pu = fmaf(q, (float)x, pu);
+      }
+      f(p0, pu, (float)y);
     }
-    two_add(s0, e0, p0);
-    two_add(su, eu, pu);
-    const float pz = __fmul_rn(p0, (float)y);
-    two_add(sz, ez, pz);
-    ez = __fadd_rn(ez, fmaf(p0, (float)y, -pz));
+  };
+  Moments mom;
+  rows([&](float p, float pu, float y) { mom.add(p, pu, y); });
+  double m[3];
+  if (mom.in_range()) {
+    mom.total(m);
+  } else {
+    double d[3] = {0.0, 0.0, 0.0};
+    rows([&](float p, float pu, float y) { add_moments(d, p, pu, y); });
+    for (int q = 0; q < 3; ++q) m[q] = warp_sum(d[q]);
   }
-  const double m0 = warp_sum(s0, e0), mz = warp_sum(sz, ez), mu = warp_sum(su, eu);
-  if (lane == 0) {
-    red[0][warp] = m0;
-    red[1][warp] = mz;
-    red[2][warp] = mu;
-  }
+  if (lane == 0)
+    for (int q = 0; q < 3; ++q) red[q][warp] = m[q];
   __syncthreads();
   if (threadIdx.x < 3) {
     double a = 0.0;

@@ -389,8 +389,8 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
         if (q) load_av(q, av);
         float err2 = 0.0f, err1 = 0.0f;
         col_task(q, av, err2, err1);
-        two_add(es, ee, 2.0f * err2);
-        two_add(es, ee, err1);
+        two_add(es, ee, eighths2(err2));
+        two_add(es, ee, eighths1(err1));
       }
       const double errd = warp_sum(es, ee);
       if (lane == 0) red[warp] = errd;
@@ -419,11 +419,11 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
         for (int q = lane; q < F::C * F::NW; q += 32)
           s += dsm_ld_f64(dsm_map(smem_u32(red + q % F::NW), (uint32_t)(q / F::NW)));
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        // the raw sum; the square root and division wait until the last
+        // the raw sum in eighths; the square root and division wait until the last
         // iteration (see publish_at_once for the exception)
         if (lane == 0)
           J->err_hist[(size_t)(err_slot + it) * Np + n] =
-              publish_at_once<N, Q>() ? publish_error(s, J->Cn[n], J->sumA2[n], J->status, n) : s;
+              publish_at_once<N, Q>() ? publish_error(kEighths * s, J->Cn[n], J->sumA2[n], J->status, n) : s;
       }
       cluster_arrive();
       if (fwd) load_av(0, av);  // in flight across the barrier
@@ -433,7 +433,7 @@ k_fused(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
       __syncwarp();
       for (int it = lane; it < n_iters; it += 32) {
         double* e = J->err_hist + (size_t)(err_slot + it) * Np + n;
-        *e = publish_error(__ldcg(e), J->Cn[n], J->sumA2[n], J->status, n);
+        *e = publish_error(kEighths * __ldcg(e), J->Cn[n], J->sumA2[n], J->status, n);
       }
     }
   }

@@ -17,8 +17,9 @@ std::atomic<long long> g_launches{0};
 //
 // A CTA takes a 32 x 32 tile of the half plane with its partners -k, so each
 // intensity is read and rooted once, and the tile leaves transposed through
-// shared memory.  Each thread sums its terms in FP32 (at most eight), the
-// warp FP32 pairs (48 bits), FP64 across warps and CTAs.  Bound by HBM and
+// shared memory.  Each thread sums its terms in FP32 (at most ten), the
+// warp FP32 pairs (48 bits), FP64 across warps and CTAs; a warp whose sums
+// leave FP32's range takes FP64.  Bound by HBM and
 // the square roots.  N = 512, 360 angles: a warp a row over the full plane and
 // a transpose pass after it 443 + 143 us, this kernel 296 us.
 //
@@ -38,8 +39,9 @@ __global__ void __launch_bounds__(256) k_prepare(const float* __restrict__ I, in
   const uint8_t* Mn = mask ? mask + (size_t)n * mask_stride : nullptr;
   float cf = 0.0f, af = 0.0f;
   int bad = 0;
-  // the pair {(ky, kx), (-ky, -kx)}, 0 <= kx <= h: returns A_sym
-  auto pair = [&](int ky, int kx) {
+  // the pair {(ky, kx), (-ky, -kx)}, 0 <= kx <= h: its terms to add(half the
+  // difference, A(k), A(-k) or 0, how often); returns A_sym
+  auto pair = [&](int ky, int kx, auto&& add) {
     const int ry = ky < h ? ky + h : ky - h;               // centred row of +ky
     const int my = ky <= h ? h - ky : N + h - ky;           // centred row of -ky
     const int rx = kx < h ? kx + h : 0, mx = h - kx;        // centred columns of +kx and -kx
@@ -49,22 +51,36 @@ __global__ void __launch_bounds__(256) k_prepare(const float* __restrict__ I, in
     if (Mn && !(Mn[p] && Mn[q])) return -1.0f;
     const float ap = sqrtf(fmaxf(ip, 0.0f)), am = sqrtf(fmaxf(im, 0.0f));
     const float d = 0.5f * (ap - am);
-    if (kx == 0 || kx == h) {  // the partner is in the same column and has its own turn
-      cf = fmaf(d, d, cf);
-      af = fmaf(ap, ap, af);
-    } else {
-      cf = fmaf(2.0f * d, d, cf);
-      af = fmaf(ap, ap, fmaf(am, am, af));
-    }
+    // in the columns 0 and N/2 the partner is in the same column and has its own turn
+    if (kx == 0 || kx == h) add(d, ap, 0.0f, 1.0f);
+    else add(d, ap, am, 2.0f);
     return 0.5f * (ap + am);
   };
+  auto all = [&](auto&& add) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int ky = ky0 + ty + 8 * j, kx = kx0 + tx;
-    if (ky < N && kx < h) tile[ty + 8 * j][tx] = pair(ky, kx);
+    for (int j = 0; j < 4; ++j) {
+      const int ky = ky0 + ty + 8 * j, kx = kx0 + tx;
+      if (ky < N && kx < h) tile[ty + 8 * j][tx] = pair(ky, kx, add);
+    }
+    if (kx0 == 0 && ty == 0 && ky0 + tx < N) A_nyq[(size_t)n * N + ky0 + tx] = pair(ky0 + tx, h, add);
+  };
+  all([&](float d, float ap, float am, float w) {
+    cf = fmaf(w * d, d, cf);
+    af = fmaf(ap, ap, fmaf(am, am, af));
+  });
+  double c_part, a_part;
+  if (__all_sync(0xffffffffu, isfinite(cf) && isfinite(af))) {
+    c_part = warp_sum(cf, 0.0f);
+    a_part = warp_sum(af, 0.0f);
+  } else {  // beyond FP32: the terms again in FP64
+    c_part = a_part = 0.0;
+    all([&](float d, float ap, float am, float w) {
+      c_part += (double)w * d * d;
+      a_part += (double)ap * ap + (double)am * am;
+    });
+    c_part = warp_sum(c_part);
+    a_part = warp_sum(a_part);
   }
-  if (kx0 == 0 && ty == 0 && ky0 + tx < N) A_nyq[(size_t)n * N + ky0 + tx] = pair(ky0 + tx, h);
-  const double c_part = warp_sum(cf, 0.0f), a_part = warp_sum(af, 0.0f);
   if (tx == 0) { sc[ty] = c_part; sa[ty] = a_part; }
   const int block_bad = __syncthreads_or(bad);
 #pragma unroll

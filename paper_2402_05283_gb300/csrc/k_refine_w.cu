@@ -14,12 +14,13 @@ CPRA_FOR_EACH_N(CPRA_CASE)
 __global__ void k_rdata(const float2* __restrict__ V, const uint8_t* __restrict__ M, float2* W, double* konst,
                         int N, int HP) {
   const int H = N / 2, ky = blockIdx.x, my = (N - ky) % N;
-  float k = 0.0f, ke = 0.0f, d = 0.0f, de = 0.0f;
+  double sk = 0.0, sd = 0.0;
   for (int c = threadIdx.x; c <= H; c += blockDim.x) {
     const int mc = (N - c) % N;
     const bool m1 = M[ky * N + c], m2 = M[my * N + mc];
     if (!m1 && !m2) continue;
     const float wt = (c == 0 || c == H) ? 0.5f : 1.0f;  // the partner is in the same column
+    float k = 0.0f, ke = 0.0f, d = 0.0f, de = 0.0f;  // N/16 planes
 #pragma unroll 4
     for (int kz = blockIdx.y; kz < N; kz += gridDim.y) {
       const int mz = (N - kz) % N;
@@ -37,8 +38,11 @@ __global__ void k_rdata(const float2* __restrict__ V, const uint8_t* __restrict_
         two_add(k, ke, 0.5f * wt * fmaf(dx, dx, dy * dy));
       }
     }
+    sk += pair_value(k, ke);
+    sd += pair_value(d, de);
   }
-  const double sk = warp_sum(k, ke), sd = warp_sum(d, de);
+  sk = warp_sum(sk);
+  sd = warp_sum(sd);
   if ((threadIdx.x & 31) == 0) {
     atomicAdd(konst + 0, sk);
     atomicAdd(konst + 1, sd);

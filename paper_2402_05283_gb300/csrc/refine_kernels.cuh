@@ -391,6 +391,10 @@ k_rv(float2* X, const float2* __restrict__ Wd, const uint8_t* __restrict__ M, co
         }
       });
     }
+    if constexpr (MODE == kLConstrain) {  // the warp's error terms, while other warps transform
+      const double e = warp_sum(ef, 0.0f);
+      if (lane == 0) red[warp] = e;
+    }
     if constexpr (MODE != kLFwd) {
       if constexpr (MODE == kLConstrain) __syncwarp();
       FL::inv(b, a, T, xs, lane);
@@ -408,12 +412,9 @@ k_rv(float2* X, const float2* __restrict__ Wd, const uint8_t* __restrict__ M, co
   __syncthreads();
   if (rows.cc < nc) rows.each([&](int y) { base[y * estride + rows.cc] = buf[y * C::SP + rows.cc]; });
   if constexpr (MODE == kLConstrain) {
-    const double e = warp_sum(ef, 0.0f);
-    if (lane == 0) red[warp] = e;
-    __syncthreads();
     if (threadIdx.x == 0) {
       double s = 0.0;
-      for (int w = 0; w < C::WARPS; ++w) s += red[w];
+      for (int w = 0; w < C::WARPS && w * FL::L < nc; ++w) s += red[w];
       if (blockIdx.x == 0 && blockIdx.y == 0) {
         s += konst[0];
         err2[1] = konst[1];
