@@ -95,7 +95,7 @@ __device__ __forceinline__ void store_f(const float2 (&a)[FL::TA][FL::E1], float
 }
 
 template <int N>
-constexpr size_t spec_smem() { return sizeof(float2) * (VolLines<N>::XN + 2 * N + ColW<N, kPrecFP32>::BUF); }
+constexpr size_t spec_smem() { return sizeof(float2) * (SpecLines<N>::XN + 2 * N + ColW<N, kPrecFP32>::BUF); }
 
 // What the spectra kernel makes of a block of columns: F (one guess, all
 // angles: blockIdx.y = angle), REF or DIST (one angle n0 of guess blockIdx.y)
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, ColW<N, kPrecFP32>::MI
 k_spectra(const float2* __restrict__ Hp, const float2* __restrict__ ramps, float2* F, float2* corr,
           const float2* __restrict__ xtw, const MergeArgs ma) {
   using C = ColW<N, kPrecFP32>;
-  using FL = VolLines<N>;
+  using FL = SpecLines<N>;
   constexpr int H = N / 2;
   extern __shared__ float2 smem[];
   float2* xs = smem;
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(ColW<N, kPrecFP32>::NT, ColW<N, kPrecFP32>::NT
 k_merge(const MergeArgs ma, int n_l, float2* acc, unsigned long long* rings, unsigned* counts, float2* F,
         float2* corr, const float2* __restrict__ xtw) {
   using C = ColW<N, kPrecFP32>;
-  using FL = VolLines<N>;
+  using FL = SpecLines<N>;
   constexpr int H = N / 2;
   extern __shared__ float2 smem[];
   float2* xs = smem;
@@ -388,9 +388,7 @@ template <int N> struct GridCfg {
   using FL = VolLines<N>;
   static constexpr int L = FL::L, H = N / 2, HC = H + 1;
   static constexpr int NZC = (N + 7) / 8;  // chunks of eight planes
-  // samples of a row held in shared memory (else read from L2): less the low
-  // parts of the cross twiddles, so that three CTAs share an SM at every N
-  static constexpr int STAGED = 2560 - (FL::XN - N);
+  static constexpr int STAGED = 2560;  // samples of a row held in shared memory (else read from L2)
   // pitch of a line: at least N, room for the warp's tile, 2 mod 8 (the four
   // plane pairs of a quad then start four banks apart)
   static constexpr int P0 = (FL::TSIZE + L - 1) / L > N ? (FL::TSIZE + L - 1) / L : N;

@@ -148,9 +148,9 @@ __device__ __forceinline__ void tc_step_a(float2 (&a)[WP<N>::TA][WP<N>::E1], flo
 }
 
 // A layout -> B layout (forward, unnormalised).  ACC: constants as pairs of
-// floats and, unless N is a power of two, the cross twiddles too (their low
-// parts at xtw + N): see WarpLines.
-template <int N, int PREC = kPrecFP32, bool ACC = false>
+// floats, XACC: the cross twiddles too (their low parts at xtw + N): see
+// WarpLines.
+template <int N, int PREC = kPrecFP32, bool ACC = false, bool XACC = false>
 __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
                                              float2 (&b)[WP<N>::TB][WP<N>::E2], float2* T,
                                              const float2* xtw, int lane,
@@ -167,7 +167,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
       constexpr int i = decltype(II)::value;
       const int l = (lane + 32 * i) % P::E2;
       v[i] = a[i][k1];
-      if constexpr (k1 > 0 && ACC && !P::POW2) v[i] = cmul(v[i], xtw[k1 * P::E2 + l], xtw[N + k1 * P::E2 + l]);
+      if constexpr (k1 > 0 && XACC) v[i] = cmul(v[i], xtw[k1 * P::E2 + l], xtw[N + k1 * P::E2 + l]);
       else if constexpr (k1 > 0) v[i] = cmul(v[i], xtw[k1 * P::E2 + l]);
     });
     static_for<0, P::TA>([&](auto II) {
@@ -203,7 +203,7 @@ __device__ __forceinline__ void warp_fft_fwd(float2 (&a)[WP<N>::TA][WP<N>::E1],
 struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
-template <int N, int PREC = kPrecFP32, bool ACC = false, class Hook = NoHook>
+template <int N, int PREC = kPrecFP32, bool ACC = false, bool XACC = false, class Hook = NoHook>
 __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
                                              float2 (&a)[WP<N>::TA][WP<N>::E1], float2* T,
                                              const float2* xtw, int lane,
@@ -236,7 +236,7 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
     static_for<0, P::TA>([&](auto II) {
       constexpr int i = decltype(II)::value;
       const int l = (lane + 32 * i) % P::E2;
-      if constexpr (k1 > 0 && ACC && !P::POW2)
+      if constexpr (k1 > 0 && XACC)
         a[i][k1] = cmul(a[i][k1], cconj(xtw[k1 * P::E2 + l]), cconj(xtw[N + k1 * P::E2 + l]));
       else if constexpr (k1 > 0) a[i][k1] = cmul(a[i][k1], cconj(xtw[k1 * P::E2 + l]));
     });
@@ -256,22 +256,24 @@ __device__ __forceinline__ void warp_fft_inv(float2 (&b)[WP<N>::TB][WP<N>::E2],
 //   A layout: line a_line(t), points a_x(t, m), m < E1;
 //   B layout: line b_line(t), frequencies b_k(t, j), j < E2.
 //
-// Acc is the plan with accurate constants, for the refinement (k_refine_w.cu),
-// which runs a transform and its inverse over the same values hundreds of
-// times, and, unless N is a power of two, for the assembly.  The rounding of a
-// constant (cos(pi/4) as a float is 1.7e-8 short) is the same in every pass
-// and adds up in step; it was more than half of the refinement's error.  xs
-// holds XN cross twiddles: pairs where N has an odd factor, whose transforms
-// have more of them and more terms.
+// Acc is the plan with accurate constants, for the refinement
+// (refine_kernels.cuh), which runs a transform and its inverse over the same
+// values hundreds of times, and, unless N is a power of two, for the assembly.
+// The rounding of a constant (cos(pi/4) as a float is 1.7e-8 short) is the
+// same in every pass and adds up in step; it was more than half of the
+// refinement's error.  Where N has an odd factor, and so more terms and more
+// twiddles, the XN cross twiddles in xs are pairs too; AccConst leaves them
+// single, for the lines of the volume, where they cost more than they give.
 // Error against 64 bits, plain / constants / with cross twiddles: refinement,
 // N = 256, 180 angles, 50 iterations 8.1e-7 / 4.5e-7 / 3.7e-7 in 8.12 / 8.24 /
-// 8.74 ms; N = 160, 60 angles, 10 iterations 3.2e-7 / 2.4e-7 / 2.2e-7 in 0.94
-// / 0.96 / 1.00 ms; assembly, N = 192, 90 angles 3.8e-7 / 3.75e-7 / 3.6e-7.
-template <int N, bool ACC_ = false> struct WarpLines {
+// 8.74 ms; N = 384, 90 angles, 10 iterations 4.7e-7 / 3.9e-7 / 3.5e-7 in 7.8 /
+// 8.0 / 8.3 ms.
+template <int N, bool ACC_ = false, bool XACC_ = ACC_ && !WP<N>::POW2> struct WarpLines {
   using P = WP<N>;
-  static constexpr bool ACC = ACC_;
+  static constexpr bool ACC = ACC_, XACC = XACC_;
   using Acc = WarpLines<N, true>;
-  static constexpr int XN = ACC && !P::POW2 ? 2 * N : N;
+  using AccConst = WarpLines<N, true, false>;
+  static constexpr int XN = XACC ? 2 * N : N;
   static constexpr int L = P::L, TA = P::TA, E1 = P::E1, TB = P::TB, E2 = P::E2, TSIZE = P::TSIZE;
   // whether task t exists (else its registers hold nothing)
   static __device__ __forceinline__ bool a_on(int t) { return P::a_on(t); }
@@ -282,12 +284,12 @@ template <int N, bool ACC_ = false> struct WarpLines {
   static __device__ __forceinline__ int b_k(int t, int j) { return t % E1 + E1 * j; }
   static __device__ __forceinline__ void fwd(float2 (&a)[TA][E1], float2 (&b)[TB][E2], float2* T,
                                              const float2* xs, int lane) {
-    warp_fft_fwd<N, kPrecFP32, ACC>(a, b, T, xs, lane);
+    warp_fft_fwd<N, kPrecFP32, ACC, XACC>(a, b, T, xs, lane);
   }
   template <class Hook = NoHook>
   static __device__ __forceinline__ void inv(float2 (&b)[TB][E2], float2 (&a)[TA][E1], float2* T,
                                              const float2* xs, int lane, Hook&& tile_free = Hook{}) {
-    warp_fft_inv<N, kPrecFP32, ACC>(b, a, T, xs, lane, nullptr, tile_free);
+    warp_fft_inv<N, kPrecFP32, ACC, XACC>(b, a, T, xs, lane, nullptr, tile_free);
   }
 };
 }  // namespace cpra

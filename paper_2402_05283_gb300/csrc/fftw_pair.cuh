@@ -26,6 +26,7 @@ namespace cpra {
 template <bool ACC_> struct PairLines {
   static constexpr bool ACC = ACC_;
   using Acc = PairLines<true>;  // with accurate constants (see WarpLines)
+  using AccConst = Acc;
   static constexpr int N = 512, XN = N, L = 1, TA = 1, E1 = 16, TB = 1, E2 = 16;
   static constexpr int TP = 34;  // even pitch: both transpose directions conflict-free
   static constexpr int TSIZE = 16 * TP;
