@@ -443,11 +443,12 @@ typedef struct cpra_batch_s* cpra_batch_t;
  * Jacobi plans must not use shrink-wrap (UNSUPPORTED).  Gauss-Seidel plans
  * (sweep 1) of the same N, engine and n_ei form a group whose sweeps run
  * together: their Step A as rows over every member's angle 0, then one
- * launch an episode (block-wide engine, N in {16, 32, 48, 96, 160, 320};
- * fused engine, N in {64, 128, 256}) or one launch per angle of the sweep
- * (fused engine; prime + n_ei column and row launches otherwise) over every
- * member that has that angle, shrink-wrap at episode ends; calls must run whole episodes (INVALID_ARG otherwise) and
- * are not captured in a graph.  Plans must stay alive until
+ * launch an episode (fused engine, N in {64, 128, 256}; block-wide engine, N
+ * in {16, 32, 48, 96, 160, 320}, unless the group is so large that the passes
+ * are faster) or one launch per angle of the sweep (fused engine; prime + n_ei
+ * column and row launches otherwise) over every member that has that angle,
+ * shrink-wrap at episode ends; calls must run whole episodes (INVALID_ARG
+ * otherwise) and are not captured in a graph.  Plans must stay alive until
  * cpra_batch_destroy.  The batch holds device tables only. */
 cpra_status cpra_batch_create(const cpra_plan_t* plans, int32_t n, int32_t use_graph,
                               cpra_batch_t* out);

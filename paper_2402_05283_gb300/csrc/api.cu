@@ -978,7 +978,7 @@ static cpra_status iterate_sweep(cpra_plan_s* p, int32_t n_iters, double* err_ou
   cpra_status st = ensure_err_cap(p, p->t + n_iters);
   if (st != CPRA_OK) return st;
   const bool fused = p->engine == CPRA_ENGINE_FUSED;
-  const bool whole = sweep_supported(p->N, p->engine);
+  const bool whole = sweep_supported(p->N, p->engine, 1);
   const int64_t t0 = p->t;
   if (whole) {
     std::vector<JobStep> rows;
@@ -1871,7 +1871,7 @@ namespace {
 // (column, row).
 int64_t sweep_launches(const cpra_batch_s::Group& g, int32_t n_iters) {
   const int64_t episodes = n_iters / g.n_ei;
-  if (sweep_supported(g.N, g.engine)) return episodes;
+  if (sweep_supported(g.N, g.engine, (int)g.members.size())) return episodes;
   return episodes * g.np_max * (g.engine == CPRA_ENGINE_FUSED ? 1 : 1 + 2 * (int64_t)g.n_ei);
 }
 
@@ -1902,9 +1902,10 @@ cudaError_t group_steps(cpra_batch_s* b, cpra_batch_s::Group& g, const std::vect
 }
 
 // Steps A and B of a Gauss-Seidel group: Step A of every member that has not
-// started, as rows over the members' angle 0, then whole sweeps, one launch
-// (or prime + n_ei column and row launches) per angle over every member that
-// has that angle.  Every member computes what cpra_iterate computes.
+// started, as rows over the members' angle 0, then whole sweeps: one launch an
+// episode where a sweep kernel is the faster form for this many members, else
+// one launch (or prime + n_ei column and row launches) per angle over every
+// member that has that angle.  Every member computes what cpra_iterate computes.
 cpra_status batch_sweep_group(cpra_batch_s* b, cpra_batch_s::Group& g, int32_t n_iters) {
   const size_t m = g.members.size();
   const int E = g.n_ei;
@@ -1978,7 +1979,7 @@ cpra_status batch_sweep_group(cpra_batch_s* b, cpra_batch_s::Group& g, int32_t n
     p->state_ready = true;
     p->hp_valid = false;
   }
-  if (sweep_supported(g.N, g.engine)) {
+  if (sweep_supported(g.N, g.engine, (int)m)) {
     // one launch an episode: every member's chain of angles on its own cluster
     const int eps = n_iters / E;
     std::vector<JobStep> rows((size_t)eps * m);

@@ -420,7 +420,7 @@ cudaError_t launch_fused(const Launch& L);
 // engine's sizes, k_fused.cu for N = 64, 128, 256): tile j = (member,
 // 0), the member's angles in order inside the launch; step row: the coupling
 // arguments, g_src, g = g_dst, err_slot, n_iters, hio_left.
-bool sweep_supported(int N, int engine);
+bool sweep_supported(int N, int engine, int members);
 cudaError_t launch_sweep(const Launch& L);
 bool fused_sweep_supported(int N);
 cudaError_t launch_fused_sweep(const Launch& L);

@@ -17,10 +17,9 @@
 // The transforms, the projection and the update are those of k_twopass.cu,
 // term by term, so the iterates are the same bits; the error sums are taken
 // in another order.
-// N = 160, Np = 90, 2 iterations an episode: 1, 16 and 100 guesses took 11.8,
-// 14.5 and 16.7 ms with a launch per angle and pass, 2.7, 2.9 and 11.5 ms in
-// one launch (N = 96: 10.1 and 12.1 ms for 1 and 16, now 1.6 and 3.4;
-// N = 320: 15.1 and 17.7, now 6.4 and 13.6).
+// The chains of a wave of clusters take as long as one; with enough guesses the
+// passes, which fill the device as guesses are added, are the faster form
+// (sweep_choice).
 #include <cooperative_groups.h>
 
 #include "cluster.cuh"
@@ -36,13 +35,10 @@ namespace cpra {
 
 namespace {
 
-// C = 8 CTAs a cluster, the portable limit, for the shortest chain; 5 at
-// N = 160, so that about 25 clusters are resident at one CTA an SM (16 guesses:
-// 2.9 ms against 4.7 ms with 8, where 16 clusters need a second wave).
 // Threads: one a radix-4 butterfly of the CTA's lines, one a radix-8 butterfly
 // where that would be more than 640.
-template <int N> struct SweepCfg {
-  static constexpr int H = N / 2, C = N == 160 ? 5 : 8, CW = H / C;
+template <int N, int C_> struct SweepCfg {
+  static constexpr int H = N / 2, C = C_, CW = H / C;
   static constexpr int P = CW;            // row pairs of a CTA
   static constexpr int PI = P | 1;        // odd pitch of the row buffer
   static constexpr int NT = warps32(clampi(CW * N / 4 <= 640 ? CW * N / 4 : CW * N / 8, 64, 1024));
@@ -67,11 +63,11 @@ __device__ __forceinline__ void add_error(float e, double* hist, long long at) {
   if ((threadIdx.x & 31) == 0 && at >= 0) atomicAdd(hist + at, s);
 }
 
-template <int N>
-__global__ void __launch_bounds__(SweepCfg<N>::NT, 1)
+template <int N, int C>
+__global__ void __launch_bounds__(SweepCfg<N, C>::NT, 1)
 k_sweep(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
         const int2* __restrict__ tiles) {
-  using F = SweepCfg<N>;
+  using F = SweepCfg<N, C>;
   constexpr int H = F::H, CW = F::CW, P = F::P, PI = F::PI, NT = F::NT;
   extern __shared__ float2 smem[];
   float2* slab = smem;           // [row][CW]
@@ -281,9 +277,9 @@ k_sweep(const JobStatic* __restrict__ js, const JobStep* __restrict__ st,
     }
 }
 
-template <int N>
+template <int N, int C>
 cudaLaunchConfig_t sweep_config(int members, cudaLaunchAttribute* at, cudaStream_t st) {
-  using F = SweepCfg<N>;
+  using F = SweepCfg<N, C>;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(F::C, members);
   cfg.blockDim = dim3(F::NT);
@@ -298,27 +294,86 @@ cudaLaunchConfig_t sweep_config(int members, cudaLaunchAttribute* at, cudaStream
   return cfg;
 }
 
-// the current device holds a cluster of this size
-template <int N>
-bool sweep_ready() {
+// clusters of this shape that the current device holds at a time (0: none)
+template <int N, int C>
+int sweep_resident() {
   static PerDevice<int> resident;
   int clusters = 0;
   const cudaError_t e = on_device(resident, clusters, [](int& n) {
-    cudaError_t r = smem_attr(k_sweep<N>, SweepCfg<N>::SMEM);
+    const cudaError_t r = smem_attr(k_sweep<N, C>, SweepCfg<N, C>::SMEM);
     cudaLaunchAttribute at;
-    const cudaLaunchConfig_t cfg = sweep_config<N>(1, &at, nullptr);
-    return r == cudaSuccess ? cudaOccupancyMaxActiveClusters(&n, k_sweep<N>, &cfg) : r;
+    const cudaLaunchConfig_t cfg = sweep_config<N, C>(1, &at, nullptr);
+    return r == cudaSuccess ? cudaOccupancyMaxActiveClusters(&n, k_sweep<N, C>, &cfg) : r;
   });
-  if (e != cudaSuccess) cudaGetLastError();
-  return e == cudaSuccess && clusters >= 1;
+  if (e == cudaSuccess) return clusters;
+  cudaGetLastError();
+  return 0;
+}
+
+// How a group of guesses is swept: a cluster of FEW CTAs a guess has the
+// shortest chain, of MANY CTAs (0: no such form) a longer one with more
+// clusters resident; per_few and per_many are the times of an angle (2
+// iterations) with the device full, a wave of guesses at a time.  The passes of
+// k_twopass.cu take max(pass0 + pass1 G, pass2 G) for G guesses.  Measured, us an
+// angle, few / many / passes:
+//   N = 96:  1 guess 18.1 / 22.0 / 120, 24: 36.4 / 22.7 / 134, 256: 241 / 189 / 172
+//   N = 160: 1 guess 27.2 / 32.1 / 138, 16: 58.4 / 34.0 / 166, 256: 533 / 336 / 356
+//   N = 320: 1 guess 71.4 / 116 / 165, 16: 155 / 137 / 205, 32: 236 / 273 / 233,
+//            48: 319 / 295 / 306, 64: 404 / 427 / 485
+//   N = 32:  1 guess 8.9 / 13.2 / 52.7, 96: 20.2 / 13.6 / 60.4
+// At N = 16 and 48 one form is the fastest throughout (N = 16: 2 CTAs 8.7 for 1
+// guess and 10.7 for 256, 8 CTAs 8.6 and 39.1; N = 48: 4 CTAs 13.3 and 61.1, 8
+// CTAs 14.9 and 71.3; passes 33.8 and 47.3, 48.6 and 78.1).
+template <int N> struct SweepForms;
+#define CPRA_SWEEP_FORMS(N, FEW_, MANY_, T_FEW, T_MANY, P0, P1, P2)                      \
+  template <> struct SweepForms<N> {                                                     \
+    static constexpr int FEW = FEW_, MANY = MANY_;                                       \
+    static constexpr float per_few = T_FEW, per_many = T_MANY, pass0 = P0, pass1 = P1, pass2 = P2; \
+  };
+CPRA_SWEEP_FORMS(16, 2, 0, 9.5f, 0.0f, 34.0f, 0.052f, 0.1f)
+CPRA_SWEEP_FORMS(32, 8, 2, 10.3f, 14.5f, 53.0f, 0.1f, 0.1f)
+CPRA_SWEEP_FORMS(48, 4, 0, 14.9f, 0.0f, 49.0f, 0.12f, 0.1f)
+CPRA_SWEEP_FORMS(96, 6, 4, 19.0f, 23.5f, 120.0f, 0.2f, 0.5f)
+CPRA_SWEEP_FORMS(160, 8, 5, 29.7f, 34.4f, 145.0f, 0.5f, 1.4f)
+CPRA_SWEEP_FORMS(320, 8, 5, 79.0f, 148.0f, 165.0f, 2.0f, 6.3f)
+#undef CPRA_SWEEP_FORMS
+
+enum SweepChoice { kSweepPasses, kSweepFew, kSweepMany };
+
+template <int N>
+SweepChoice sweep_choice(int members) {
+  using S = SweepForms<N>;
+  const float g = (float)members;
+  float best = S::pass0 + S::pass1 * g > S::pass2 * g ? S::pass0 + S::pass1 * g : S::pass2 * g;
+  SweepChoice choice = kSweepPasses;
+  auto offer = [&](SweepChoice c, int resident, float us) {
+    if (resident < 1) return;
+    const float t = (float)((members + resident - 1) / resident) * us;
+    if (t < best) {
+      best = t;
+      choice = c;
+    }
+  };
+  offer(kSweepFew, sweep_resident<N, S::FEW>(), S::per_few);
+  if constexpr (S::MANY > 0) offer(kSweepMany, sweep_resident<N, S::MANY>(), S::per_many);
+  return choice;
+}
+
+template <int N, int C>
+cudaError_t sweep_go(const Launch& L) {
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = sweep_config<N, C>(L.ntiles, &at, L.stream);
+  g_launches += 1;
+  return cudaLaunchKernelEx(&cfg, k_sweep<N, C>, L.js, L.st, L.tiles);
 }
 
 template <int N>
 cudaError_t sweep_launch(const Launch& L) {
-  cudaLaunchAttribute at;
-  cudaLaunchConfig_t cfg = sweep_config<N>(L.ntiles, &at, L.stream);
-  g_launches += 1;
-  return cudaLaunchKernelEx(&cfg, k_sweep<N>, L.js, L.st, L.tiles);
+  using S = SweepForms<N>;
+  const SweepChoice c = sweep_choice<N>(L.ntiles);
+  if constexpr (S::MANY > 0)
+    if (c == kSweepMany) return sweep_go<N, S::MANY>(L);
+  return c == kSweepFew ? sweep_go<N, S::FEW>(L) : cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -326,12 +381,12 @@ cudaError_t sweep_launch(const Launch& L) {
 // sizes whose slab and row buffer fit the shared memory of eight CTAs
 #define CPRA_FOR_EACH_SWEEP_N(X) X(16) X(32) X(48) X(96) X(160) X(320)
 
-bool sweep_supported(int N, int engine) {
+bool sweep_supported(int N, int engine, int members) {
   if (engine == CPRA_ENGINE_FUSED) return fused_sweep_supported(N);
   if (engine != CPRA_ENGINE_TWO_PASS) return false;
   switch (N) {
 #define CPRA_CASE(NN) \
-  case NN: return sweep_ready<NN>();
+  case NN: return sweep_choice<NN>(members) != kSweepPasses;
     CPRA_FOR_EACH_SWEEP_N(CPRA_CASE)
 #undef CPRA_CASE
     default:
