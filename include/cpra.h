@@ -117,7 +117,7 @@ enum {
  *   engine         kernel family.  TWO_PASS: row and column passes with
  *                  block-wide shared-memory FFTs (every supported N).  WARP:
  *                  the same passes with warp-resident two-level FFTs
- *                  (N = 64, 128, 256, 512, 1024).  FUSED: one launch per
+ *                  (N = 64, 128, 192, 256, 384, 512, 1024).  FUSED: one launch per
  *                  run of iterations between coupling steps, each angle's
  *                  spectrum held in the distributed shared memory of a
  *                  thread-block cluster (N = 64, 128, 256, 512; FP32; needs a
@@ -371,7 +371,8 @@ enum {
   CPRA_KERNEL_PRIME = 2,     /* coupling (Eq. 4) + R2C rows                        */
   CPRA_KERNEL_SHRINKWRAP = 3,
   CPRA_KERNEL_ASSEMBLE = 4,
-  CPRA_KERNEL_FUSED = 5,     /* fused engine: prime + a run of whole iterations    */
+  CPRA_KERNEL_FUSED = 5,     /* prime + a run of whole iterations in one launch: the
+                                fused engine, and any engine's whole-episode sweep */
   CPRA_KERNEL_PREPARE = 6,
   CPRA_KERNEL_REFINE = 7,    /* Step D refinement (3D line passes, support)       */
   CPRA_KERNEL_KINDS = 8
@@ -492,11 +493,13 @@ cpra_status cpra_batch_set_persistent(cpra_batch_t batch, int32_t mode, double w
 
 cpra_status cpra_batch_destroy(cpra_batch_t batch);
 
-/* Autotuner: time each engine available for N (TWO_PASS, WARP, FUSED) on a sample
+/* Autotuner: time each engine available for N (TWO_PASS, WARP, FUSED; AUTO,
+ * which runs the warp kernels, at a size that WARP does not name) on a sample
  * of 64 random patterns with CUDA events on a private stream, and keep the
  * fastest per (N, precision, SM count, device name) in a JSON cache file.
  * cache_path NULL = $CPRA_TUNE_CACHE or $HOME/.cache/cpra_tune.json.  A
- * cached entry is returned without timing.  *engine_out receives the engine,
+ * cached entry is returned without timing (one that lacks an engine of its size
+ * is timed anew and replaced).  *engine_out receives the engine,
  * *ms_out (nullable) the measured or cached milliseconds per iteration of the
  * sample. */
 cpra_status cpra_autotune(int32_t N, int32_t precision, const char* cache_path,

@@ -680,8 +680,8 @@ cpra_status cpra_plan(const cpra_config* cfg, void* stream, cpra_plan_t* out) {
       delete p;
       return ts;
     }
-    // where the tuner has only the block-wide engine to choose, AUTO's choice
-    if (!(e == CPRA_ENGINE_TWO_PASS && unlisted)) p->engine = e;
+    // (AUTO: the warp kernels at a size that WARP does not name)
+    if (e != CPRA_ENGINE_AUTO) p->engine = e;
   }
   // AUTO: the fused engine where it is the faster one (N <= 256, FP32) and
   // this device can hold its clusters, else the warp engine
@@ -2532,8 +2532,11 @@ cpra_status cpra_autotune(int32_t N, int32_t precision, const char* cache_path,
   const std::string path = tune_path(cache_path);
   std::vector<std::string> lines = read_lines(path);
   const std::string needle = std::string("{\"key\": \"") + key + "\"";
+  // at the sizes that WARP does not name its kernels are AUTO's choice and are
+  // timed as such; an entry without them is from before they existed there
+  const bool unlisted = !warp_engine_listed(N);
   for (const std::string& l : lines) {
-    if (l.rfind(needle, 0) == 0) {
+    if (l.rfind(needle, 0) == 0 && !(unlisted && l.find("\"ms_engine_0\"") == std::string::npos)) {
       int eng = 0;
       double ms = 0.0;
       const char* q = std::strstr(l.c_str(), "\"engine\": ");
@@ -2549,9 +2552,8 @@ cpra_status cpra_autotune(int32_t N, int32_t precision, const char* cache_path,
   int best = CPRA_ENGINE_TWO_PASS;
   double best_ms = 1e30;
   std::ostringstream detail;
-  const int cands[3] = {CPRA_ENGINE_TWO_PASS, CPRA_ENGINE_WARP, CPRA_ENGINE_FUSED};
+  const int cands[3] = {CPRA_ENGINE_TWO_PASS, unlisted ? CPRA_ENGINE_AUTO : CPRA_ENGINE_WARP, CPRA_ENGINE_FUSED};
   for (int cand : cands) {
-    if (cand == CPRA_ENGINE_WARP && !warp_engine_listed(N)) continue;
     if (cand == CPRA_ENGINE_FUSED && !fused_supported(N)) continue;
     double ms = 0.0;
     cpra_status s = time_engine(N, cand, &ms);
@@ -2566,7 +2568,7 @@ cpra_status cpra_autotune(int32_t N, int32_t precision, const char* cache_path,
   entry << needle << ", \"engine\": " << best << ", \"ms\": " << best_ms << detail.str() << "}";
   std::vector<std::string> entries;
   for (const std::string& l : lines)
-    if (l.rfind("{\"key\": ", 0) == 0) entries.push_back(l.back() == ',' ? l.substr(0, l.size() - 1) : l);
+    if (l.rfind("{\"key\": ", 0) == 0 && l.rfind(needle, 0) != 0) entries.push_back(l.back() == ',' ? l.substr(0, l.size() - 1) : l);
   entries.push_back(entry.str());
   std::ofstream f(path, std::ios::trunc);
   if (f) {
