@@ -358,14 +358,14 @@ cudaError_t launch_merge_twins(cpra_plan_s* dst, const MergeArgs& ma, int n_l);
 cudaError_t launch_merge(cpra_plan_s* dst, const MergeArgs& ma, int n_l, float2* acc, unsigned long long* rings,
                          float* prtf);
 // inverse FFT along y of every plane of a volume, in place, and into out when
-// that is not NULL (k_refine_w.cu)
+// that is not NULL (refine_kernels.cuh)
 cudaError_t launch_volume_ylines(int N, float2* vol, float2* out, const float2* xtw, cudaStream_t st);
 
 // Step D refinement (k_refine.cu): buffers of one plan's refinement
 struct RefineArgs {
   int N, W;            // W = ceil(N/32) words per x row of S3
   float2* X;           // N^3: the data volume, then the half spectrum [z][y][HP]
-  float2* Wd;          // N^3: the data of the half spectrum (k_refine_w.cu), same layout
+  float2* Wd;          // N^3: the data of the half spectrum (refine_kernels.cuh), same layout
   float* R;            // [N^3] real iterate rho
   float* Bv;           // [N^3] shrink-wrap blur scratch
   uint32_t* S3;        // [N][N][W] 3D support bits

@@ -15,7 +15,7 @@
 //            adjoint weights of every sample, normalised by their sum, FP64,
 //            rounded once) are built on the host; the sign (-1)^(kx+ky) makes
 //            the inverse transform land centred in x and y.
-//   y lines  inverse FFT along ky in place (k_refine_w.cu).
+//   y lines  inverse FFT along ky in place (refine_kernels.cuh).
 // Step C merge of several guesses (cpra_merge): the spectra kernel stores the
 // best guess's E of one PO (REF) and tells for the other guesses whether their
 // E or conj E, the spectrum of the centrally inverted PO, is the nearer to it

@@ -6,7 +6,7 @@
 // slices reach (the measured mask M, the same for every kz).  Volumes are
 // [z][y][x], N^3, in the centred frame of the Step D volume (the frame of
 // the 2D supports); V is the spectrum of that volume.  One iteration is four
-// passes over the half spectrum of rho (k_refine_w.cu):
+// passes over the half spectrum of rho (refine_kernels.cuh):
 //   y lines   forward FFT_y
 //   z lines   forward FFT_z -> error, X <- V where M -> IFFT_z
 //   y lines   inverse FFT_y

@@ -210,10 +210,9 @@ struct TileTaps {
 __host__ __device__ constexpr int sw_tiles_x(int N) { return (N + kTileX - 1) / kTileX; }
 __host__ __device__ constexpr int sw_tiles(int N) { return sw_tiles_x(N) * ((N + kTileY - 1) / kTileY); }
 
-// U8: the support is bytes (nonzero = in), else bits, W words a row
-template <bool U8>
-__global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, const void* __restrict__ S, float* b,
-                                                 float* tmax, const TileTaps taps, int ntaps, int lo, int N, int W) {
+// (the support as bytes, nonzero = in)
+__global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, const uint8_t* __restrict__ S, float* b,
+                                                 float* tmax, const TileTaps taps, int ntaps, int lo, int N) {
   static_assert(kTilePA % 2 == 1 && kTilePB % 2 == 1, "pitches");
   __shared__ float A[kTileRows * kTilePA];
   __shared__ float B[kTileRows * kTilePB];
@@ -235,9 +234,7 @@ __global__ void __launch_bounds__(256) k_sw_tile(const float* __restrict__ g, co
       int x = x0 + c + off;
       x = x < 0 ? x + N : (x >= N ? x - N : x);
       const float v = __ldg(g + row * N + x);
-      bool in;
-      if constexpr (U8) in = __ldg(static_cast<const uint8_t*>(S) + row * N + x) != 0;
-      else in = (__ldg(static_cast<const uint32_t*>(S) + row * W + (x >> 5)) >> (x & 31)) & 1u;
+      const bool in = __ldg(S + row * N + x) != 0;
       A[r * kTilePA + c] = (in && v >= 0.0f) ? v : 0.0f;
     }
   }
@@ -531,7 +528,7 @@ extern "C" cpra_status cpra_shrinkwrap_static(const float* g, const uint8_t* S_i
     float* tmax = reinterpret_cast<float*>(sc.mx);  // 64 x 32 pixels a tile: fewer than its 4096 entries
     const bool wide = (((uintptr_t)S_in | (uintptr_t)S_out) & 3) == 0;
     g_launches += 2;
-    k_sw_tile<true><<<dim3(sw_tiles(N), count), 256, 0, st>>>(g, S_in, sc.b, tmax, tt, ntaps, lo, N, W);
+    k_sw_tile<<<dim3(sw_tiles(N), count), 256, 0, st>>>(g, S_in, sc.b, tmax, tt, ntaps, lo, N);
     if (wide)
       k_sw_thresh_u8<true><<<dim3((N * N / 4 + 255) / 256, count), 256, 0, st>>>(sc.b, tmax, S_in, S_out, tau, N);
     else
