@@ -262,8 +262,9 @@ cpra_status cpra_set_present(cpra_plan_t plan, const uint8_t* mask);
 /* Step D: spectra of P_{S+} g with the centre-of-mass phase ramp, Fourier
  * slice gridding (bilinear in kx, ky; exact kz) into an N^3 grid, inverse 3D
  * FFT.  The centred complex64 volume [z][y][x] stays in the plan (read it
- * with CPRA_RESULT_VOLUME) and is also copied to out_volume when that is not
- * NULL (N^3 * 8 bytes, host or device). */
+ * with CPRA_RESULT_VOLUME) and is also written to out_volume when that is not
+ * NULL (N^3 * 8 bytes, host or device; INVALID_ARG for device memory whose
+ * allocation ends before that). */
 cpra_status cpra_assemble_3d(cpra_plan_t plan, void* out_volume);
 
 /* cpra_assemble_3d, then a download of the volume to out that the call does

@@ -15,6 +15,7 @@
 #include <nvtx3/nvToolsExt.h>
 #include <vector>
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -64,6 +65,27 @@ bool local_memory(const cpra_plan_s* p, const void* ptr) {
     return false;
   }
   return a.type == cudaMemoryTypeDevice && own.type == cudaMemoryTypeDevice && a.device == own.device;
+}
+
+// bytes from ptr to the end of its device allocation (SIZE_MAX where the driver
+// does not say), so that a kernel writes only where a copy would have been
+// accepted
+size_t bytes_behind(const void* ptr) {
+  using Range = CUresult(CUDAAPI*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Range range = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuMemGetAddressRange", &fn, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      fn = nullptr;
+    }
+    return (Range)fn;
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range || range(&base, &size, (CUdeviceptr)(uintptr_t)ptr) != CUDA_SUCCESS) return SIZE_MAX;
+  return (size_t)(base + size - (CUdeviceptr)(uintptr_t)ptr);
 }
 
 void* dev_alloc(cpra_plan_s* p, size_t bytes) {
@@ -1175,12 +1197,14 @@ cpra_status cpra_assemble_3d(cpra_plan_t p, void* out) {
   if (!p->state_ready) return fail(p, CPRA_ERR_NOT_READY, "no iterate to assemble");
   if (p->partial) return fail(p, CPRA_ERR_NOT_READY, "assembly needs every angle present");
   const size_t N = p->N, NN = N * N;
-  cpra_status st = ensure_assembly(p);
-  if (st == CPRA_OK) st = upload_rho_rows(p);
-  if (st != CPRA_OK) return st;
   // memory of this device takes the volume from the last kernel itself (the
   // copy afterwards read and wrote it once more: 0.32 of 2.3 ms at N = 512)
   const bool direct = local_memory(p, out);
+  if (direct && bytes_behind(out) < N * NN * 8)
+    return fail(p, CPRA_ERR_INVALID_ARG, "out_volume's allocation ends before N^3 complex values");
+  cpra_status st = ensure_assembly(p);
+  if (st == CPRA_OK) st = upload_rho_rows(p);
+  if (st != CPRA_OK) return st;
   CK(timed(p, CPRA_KERNEL_ASSEMBLE, [&] {
        cudaError_t e = launch_rho_rows(p, plan_launch(p, 0, p->Np), p->asmb.moments, p->asmb.ramps);
        return e == cudaSuccess ? launch_assemble(p, direct ? (float2*)out : nullptr) : e;
