@@ -546,6 +546,9 @@ static cudaError_t fused_sweep_go(const Launch& L) {
   return cudaLaunchKernelEx(&cfg, k_fused<N, false, Q, true>, L.js, L.st, L.tiles);
 }
 
+// However many the members: a launch an angle runs the same clusters in the same
+// waves (256 guesses, us an angle, one launch / a launch an angle: N = 64 22 /
+// 34, 128 56 / 69, 256 217 / 252).
 bool fused_sweep_supported(int N) {
   switch (N) {
     case 64: return sweep_wide<64>() > 0;

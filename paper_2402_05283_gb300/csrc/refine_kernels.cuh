@@ -25,8 +25,9 @@
 //         constraint between its forward and inverse transforms.
 // Bound by HBM and, at N = 256, L2: 36 N^3 bytes an iteration, against
 // (72 + 8 f) N^3 with complex volumes (f: measured fraction).  N = 256, 180
-// angles: 254 us an iteration with complex volumes, 138 now (y lines 26 each,
-// z lines with the data 56, x rows 30).
+// angles: 254 us an iteration with complex volumes, 138 with plain constants (y
+// lines 26 each, z lines with the data 56, x rows 30), 141 with their low parts
+// (WarpLines::Acc), which more than halve the error.
 #pragma once
 #include "cpra_internal.h"
 #include "fast_kernels.cuh"
