@@ -90,10 +90,11 @@ __device__ __forceinline__ void static_for(F&& f) {
   }
 }
 
-// x * c + y for a constant c, rounded once or, ACC, with c as a pair of floats
-// (48 bits): c's own rounding is the same in every call, so where a transform
-// and its inverse run over the same values hundreds of times it adds up in
-// step, while the other roundings add up at random.
+// Products by a constant c, which is rounded to a float or, ACC, kept as a pair
+// of floats (48 bits; the product is rounded once): c's own rounding is the same
+// in every call, so where a transform and its inverse run over the same values
+// hundreds of times it adds up in step, while the other roundings add up at
+// random.
 template <bool ACC> struct Const {
   float hi, lo;
   constexpr Const(double c) : hi((float)c), lo((float)(c - (double)(float)c)) {}
