@@ -35,8 +35,8 @@ def _rel(got, ref):
     return float((got.to(ref.dtype) - ref).norm() / ref.norm())
 
 
-@pytest.mark.parametrize("N,Np,iters", [(16, 9, 3), (32, 12, 3), (48, 12, 3), (96, 12, 3), (160, 9, 2), (192, 9, 2), (320, 7, 2),
-                                        (384, 7, 2), (512, 5, 2), (640, 4, 2), (700, 4, 2), (768, 4, 1), (1024, 3, 1)])
+@pytest.mark.parametrize("N,Np,iters", [(16, 9, 3), (32, 12, 3), (48, 12, 3), (64, 12, 3), (96, 12, 3), (128, 12, 3), (160, 9, 2),
+                                        (192, 9, 2), (256, 9, 2), (320, 7, 2), (384, 7, 2), (512, 5, 2), (640, 4, 2), (700, 4, 2), (768, 4, 1), (1024, 3, 1)])
 def test_refinement(cases, N, Np, iters):
     case = dict(kind="refine", N=N, Np=Np, iters=iters)
     assert _rel(cases.run(cases.prepare(case, 1)), cases.exact(case, 1)) < BOUND
